@@ -31,27 +31,32 @@ namespace bcmc {
 
 template <bool kOne>
 __global__ void __launch_bounds__(kThreads) prep_kernel(Launch L) {
-    const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
-    for (uint32_t v = 0; v < L.n; v++) {
-        const VolEntry &e = vol_of<kOne>(L, v);
+    // Bound by the latency of one dependent read a volume (mc_tiles), so every
+    // volume gets an equal share of the CTAs: with all CTAs walking the
+    // volumes one after another a batch of 64 volumes spent 73 us here, and
+    // its warm pass took 423 instead of 366 us.
+    const uint32_t parts = kOne ? gridDim.x : max(1u, gridDim.x / L.n);
+    for (uint32_t w = blockIdx.x; w < parts * L.n; w += gridDim.x) {
+        const VolEntry &e = vol_of<kOne>(L, kOne ? 0u : w / parts);
+        const uint32_t i0 = (kOne ? w : w % parts) * blockDim.x + threadIdx.x, stride = parts * blockDim.x;
         const DevState &s = e.s;
         const uint32_t n_mc_desc = s.ctl->mc_tiles;   // descriptors the last triangle pass used
-        for (uint32_t i = tid; i < n_mc_desc; i += stride) {
+        for (uint32_t i = i0; i < n_mc_desc; i += stride) {
             s.desc_mc[i] = 0;
             s.desc_occ[i] = 0;
             if (s.desc_vtx) s.desc_vtx[i] = 0;
         }
-        for (uint32_t i = tid; i < e.n_cull_desc; i += stride) {
+        for (uint32_t i = i0; i < e.n_cull_desc; i += stride) {
             s.desc_cull[i] = 0;
             s.desc_cand[i] = 0;
         }
-        for (uint32_t i = tid; i < e.n_lru_desc; i += stride) {
+        for (uint32_t i = i0; i < e.n_lru_desc; i += stride) {
             s.desc_lru_a[i] = 0;
             s.desc_lru_b[i] = 0;
         }
     }
-    for (uint32_t v = tid; v < L.n; v += stride) {
+    for (uint32_t v = tid; v < L.n; v += gridDim.x * blockDim.x) {
         Ctl *c = vol_of<kOne>(L, v).s.ctl;
         c->epoch += 1;
         c->n_active = 0;
