@@ -415,9 +415,11 @@ int iso_set_test_fault(iso_volume *v, uint32_t what);
  * events on the volume's stream between its kernels; iso_stage_times then
  * returns the last extraction's durations in milliseconds, in this order:
  *   0 prep (counters and descriptors), 1 cull (Section 4.1 and the
- *   hit/new split of Algorithm 1), 2 cache update (rest of Algorithm 1),
- *   3 decode (Section 4.2.1), 4 count (Sections 4.3-4.4: per-block
- *   triangle counts), 5 scan (Section 4.4: offsets), 6 emit (Section 4.5).
+ *   hit/new split of Algorithm 1), 2 cache update (rest of Algorithm 1, and
+ *   the classification of the cached active blocks' samples), 3 decode
+ *   (Section 4.2.1, and the same for the new blocks), 4 count (Sections
+ *   4.3-4.4: per-block triangle counts and their offsets, one kernel), 5 scan
+ *   (nothing: part of the count's kernel), 6 emit (Section 4.5).
  * ms must hold n >= 7 floats.  Profiling off (the default) records
  * nothing. */
 #define ISO_NUM_STAGES 7
@@ -510,10 +512,10 @@ typedef struct iso_launch_shape {
     uint32_t cache_update_ctas;  /* Algorithm 1 (both cache-update kernels) */
     uint32_t decode_ctas;        /* Section 4.2.1 */
     uint32_t decode_tile;        /* new blocks per decode CTA: 64, 128 (default) or 256 */
-    uint32_t count_ctas;         /* Section 4.4: per-block triangle counts */
-    uint32_t count_tile;         /* candidate blocks per count CTA: 16, 32 (default) or 64 */
-    uint32_t scan_ctas;          /* Section 4.4: offsets */
-    uint32_t scan_tile;          /* counts per offset-scan tile: 1024, 2048 (default) or 4096 */
+    uint32_t count_ctas;         /* no effect: scan_ctas is the counting kernel's too */
+    uint32_t count_tile;         /* 16, 32 (default) or 64: checked and reported, no effect */
+    uint32_t scan_ctas;          /* Section 4.4: per-block triangle counts and offsets (one kernel) */
+    uint32_t scan_tile;          /* 1024, 2048 (default) or 4096: checked and reported, no effect */
     uint32_t emit_ctas;          /* Section 4.5 */
     uint32_t emit_tile;          /* candidate blocks per emit CTA: 16, 32 (default) or 64 */
 } iso_launch_shape;
@@ -521,9 +523,8 @@ typedef struct iso_launch_shape {
 /* The launch shape of a single volume's extractions (same fields and
  * rules as a batch's; every shape computes the same results).  Takes
  * effect from the next call; the volume's captured graphs are rebuilt.  A
- * volume starts with 4096-count scan tiles at one CTA per SM and 256-block
- * decode CTAs, the rest at the defaults (zeros in a shape passed here mean
- * the general defaults). */
+ * volume starts with scan_tile 4096, the rest at the defaults (zeros in a
+ * shape passed here mean the general defaults). */
 int iso_set_shape(iso_volume *v, const iso_launch_shape *shape);
 int iso_get_shape(const iso_volume *v, iso_launch_shape *shape);
 
@@ -613,17 +614,14 @@ typedef struct iso_server_options {
     uint64_t vertex_budget_bytes;  /* limit on held mesh bytes (48 or 24 per triangle); 0 = none */
     void *stream;                  /* cudaStream_t whose earlier work the server waits for at creation
                                       (NULL = default); the server runs on two streams of its own */
-    uint64_t case_bytes;           /* room for the requests' stored cell cases, 64 bytes a candidate:
-                                      0 = max_batch full candidate lists, at most 4 GiB; below 64 = none
-                                      (every emission classifies again); the meshes are the same */
+    uint64_t case_bytes;           /* no effect (room for stored cell cases, which no emission reads any
+                                      more) */
 } iso_server_options;
 
 /* v must not be loaded with ISO_DEBUG.  The server keeps 2 * max_batch
  * request positions (a running tick's and the next tick's), each with
- * candidate, count, offset and occupied-list arrays of min(cache slots, nb)
- * entries (20 bytes each), a buffer for the requests' stored cell cases
- * (case_bytes; a request whose cases do not fit is classified again by its
- * emission), and creates two streams: the backs run at the
+ * candidate, occupied-list, offset and below-mask arrays of min(cache slots,
+ * nb) entries (24 bytes each), and creates two streams: the backs run at the
  * device's highest stream priority, the fronts at its lowest, so a front
  * overlapping a back takes only the SMs the back leaves idle.  Meshes are
  * complete when a request finishes (the server waits for its emission). */

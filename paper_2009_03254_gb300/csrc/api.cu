@@ -297,11 +297,10 @@ Plan launch_plan(const Plan *want, int device, uint64_t total_blocks, uint64_t t
     auto tiles_of = [&](uint64_t n, int tile) { return (n + tile - 1) / tile + n_vols; };
     clamp(use.cull, tiles_of(total_blocks, use.cull_tile));
     clamp(use.lru_a, 2 * tiles_of(total_slots, kScanTile) + n_vols);
-    clamp(use.lru_b, tiles_of(total_slots, kScanTile));
+    clamp(use.lru_b, tiles_of(total_slots, 32));          // also 4 cached blocks' masks a warp
     clamp(use.decode, tiles_of(total_slots, use.decode_tile));
-    clamp(use.mc_count, tiles_of(total_slots, use.count_tile));
     clamp(use.mc_emit, tiles_of(total_slots, use.emit_tile));
-    clamp(use.mc_scan, tiles_of(total_slots, use.scan_tile));
+    clamp(use.mc_scan, tiles_of(total_slots, kCountTile));
     return use;
 }
 
@@ -364,8 +363,8 @@ int free_volume(iso_volume *v) {
     DevState &s = v->s;
     void *ptrs[] = {v->bits, v->bmin, v->bmax, v->hull, v->hull8, v->seg, v->tables, s.mactive, s.iactive, s.inew, s.icand,
                     s.islot, s.slast, s.sblock, s.lbuf[0], s.lbuf[1], s.newslot, s.slots, s.desc_cull, s.desc_cand,
-                    s.desc_lru_a, s.desc_lru_b, s.desc_mc, s.ctl, s.counts, s.offsets, s.iocc, s.cases, s.dbg_edges,
-                    s.voff, s.cutw};
+                    s.desc_lru_a, s.desc_lru_b, s.desc_mc, s.ctl, s.ihit, s.bmask, s.counts, s.offsets, s.iocc, s.ooff,
+                    s.cases, s.dbg_edges, s.voff};
     for (void *p : ptrs) dfree_on(p, v->stream);
     cudaStreamSynchronize(v->stream);
     (void)cudaGetLastError();
@@ -401,10 +400,9 @@ int enqueue_pipeline(iso_volume *v, cudaStream_t st, Phase phase, bool prof, boo
     if (prof) cudaEventRecord(phase == Phase::kEmit ? v->ev[ISO_NUM_STAGES + 1] : v->ev[0], st);
     if (phase != Phase::kEmit) {
         launch_front(L, v->plan, st, prof ? v->ev : nullptr, v->upload_pending ? v->uploaded : nullptr);
-        launch_mc_count(L, debug, v->plan, st, indexed);
+        launch_mc_scan(L, debug, v->plan, st, indexed);
         if (prof) cudaEventRecord(v->ev[5], st);
-        launch_mc_scan(L, v->plan, st);
-        if (prof) cudaEventRecord(v->ev[6], st);
+        if (prof) cudaEventRecord(v->ev[6], st);         // the scan is part of the count's launch
     }
     if (phase != Phase::kCount) {
         launch_mc_emit(L, debug, v->plan, st, indexed);
@@ -485,16 +483,9 @@ struct Indexed {                   // indexed-mesh outputs of one pass
     unsigned long long vtx_base;   // added to every index
 };
 
-// the first-vertex array of the occupied candidates and the candidates'
-// cut-edge words, made at the first indexed extraction
-int ensure_voff(iso_volume *v) {
-    if (!v->s.voff) {
-        const int rc = dalloc(v, &v->s.voff, v->s.list_cap);
-        if (rc) return rc;
-    }
-    if (!v->s.cutw) return dalloc(v, &v->s.cutw, (size_t)v->s.list_cap * 12);
-    return ISO_OK;
-}
+// the first-vertex array of the occupied candidates, made at the first
+// indexed extraction
+int ensure_voff(iso_volume *v) { return v->s.voff ? ISO_OK : dalloc(v, &v->s.voff, v->s.list_cap); }
 
 int run(iso_volume *v, float iso, void *out, unsigned long long cap_tris, Phase phase = Phase::kAll,
         uint32_t format = kVertexFloat4, uint32_t flags = 0, const Window *w = nullptr,
@@ -797,7 +788,7 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     // descriptors for the smallest tile of each scan (any plan may run)
     v->n_cull_desc = (g.nb + kMinCullTile - 1) / kMinCullTile;
     v->n_lru_desc = (v->cap + kScanTile - 1) / kScanTile;
-    const uint32_t n_mc_desc = (v->cap + kMinMcScanTile - 1) / kMinMcScanTile;   // candidates <= cap
+    const uint32_t n_mc_desc = (v->cap + kCountTile - 1) / kCountTile;   // candidates <= cap
     const bool on_device = (o.flags & ISO_INPUT_ON_DEVICE) != 0;
     TRY(dalloc(v, &v->bits, words));
     if (!on_device) {                 // staging for host ranges (freed once the hulls exist)
@@ -834,12 +825,10 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     TRY(dalloc(v, &s.counts, v->cap));
     TRY(dalloc(v, &s.offsets, v->cap));
     TRY(dalloc(v, &s.iocc, s.list_cap));
-    // the count pass keeps each candidate's cases for the emit pass when they
-    // take at most 8 GB (else emit classifies again); debug volumes always
-    if ((v->flags & ISO_DEBUG) || (uint64_t)s.list_cap * 64 <= (8ull << 30)) {
-        TRY(dalloc(v, &s.cases, (size_t)s.list_cap * 64));
-        s.case_cap = s.list_cap;
-    }
+    TRY(dalloc(v, &s.ooff, s.list_cap));
+    TRY(dalloc(v, &s.ihit, s.list_cap));
+    TRY(dalloc(v, &s.bmask, v->cap));
+    if (v->flags & ISO_DEBUG) TRY(dalloc(v, &s.cases, (size_t)s.list_cap * 64));
     {
         char *block = static_cast<char *>(pinned_take());
         if (!block) {
@@ -891,6 +880,7 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     if (s.iactive) TRYC(cudaMemsetAsync(s.iactive, 0, (size_t)s.list_cap * 4, st));
     TRYC(cudaMemsetAsync(s.inew, 0, (size_t)s.list_cap * 4, st));
     TRYC(cudaMemsetAsync(s.icand, 0, (size_t)s.list_cap * 4, st));
+    TRYC(cudaMemsetAsync(s.ihit, 0, (size_t)s.list_cap * 4, st));
     TRYC(cudaMemsetAsync(s.newslot, 0, (size_t)v->cap * 4, st));
     TRYC(cudaMemsetAsync(s.lbuf[0], 0, (size_t)v->cap * 4, st));
     TRYC(cudaMemsetAsync(s.lbuf[1], 0, (size_t)v->cap * 4, st));
@@ -931,14 +921,10 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
             return ISO_ERR_CORRUPT;
         }
     }
-    // single-volume defaults from a sweep of every tile variant and CTA count
-    // on the 512^3 benchmark: 4096-count scan tiles at one CTA per SM (the
-    // other kernels' defaults were already best; 128-block decode CTAs, with
-    // the list append in its own kernel, beat 256-block CTAs that append
-    // after decoding: 91.0 + 8.5 against 103.8 us per surface)
+    // single-volume defaults (128-block decode CTAs, with the list append in
+    // its own kernel, beat 256-block CTAs that append after decoding)
     v->want = Plan{};
-    v->want.scan_tile = 4096;
-    v->want.mc_scan = 1;
+    v->want.scan_tile = 4096;         // reported; the count and scan has one tile size
     v->plan = launch_plan(&v->want, v->device, g.nb, v->cap, 1, true, g.rate, v->seg != nullptr);
     TRYC(cudaGetLastError());
     *out = v;

@@ -103,9 +103,8 @@ int enqueue_batch(iso_batch *b, cudaStream_t st, bool prof) {
     if (prof) cudaEventRecord(b->ev[0], st);
     launch_batch_params(L, b->d_iso, st);
     launch_front(L, b->plan, st, prof ? b->ev : nullptr);
-    launch_mc_count(L, false, b->plan, st);
-    if (prof) cudaEventRecord(b->ev[5], st);
-    launch_mc_scan(L, b->plan, st);
+    if (prof) cudaEventRecord(b->ev[5], st);             // no kernel of the count's own: the scan counts
+    launch_mc_scan(L, false, b->plan, st);
     if (prof) cudaEventRecord(b->ev[6], st);
     launch_batch_offsets(L, b->d_bo, b->d_tri_base, st);
     launch_mc_emit(L, false, b->plan, st);

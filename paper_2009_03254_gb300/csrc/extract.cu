@@ -6,9 +6,11 @@
 //           cache hits
 //   lru_a   Algorithm 1 (grow, select least recently used free slots,
 //           assign, evict) over the used-slot list
-//   lru_b   append this epoch's slots to the list (most recent last)
-//   decode  Section 4.2.1: decode each new block into its slot
-//   mc      Sections 4.3-4.5 (mc.cu): count, scan, emit
+//   lru_b   append this epoch's slots to the list (most recent last); the
+//           below masks of the cached active blocks
+//   decode  Section 4.2.1: decode each new block into its slot, with its
+//           below mask
+//   mc      Sections 4.3-4.5 (mc.cu): count and scan, emit
 //
 // Sizes that only the device knows (n_active, n_new, ...) never come back
 // to the host between kernels: the kernels are persistent and take their
@@ -199,6 +201,8 @@ __device__ __forceinline__ void cull_tile(const DevState &s, const Geom &g, uint
         if (s.iactive && ((ab >> lane) & 1u) && ai < s.list_cap) s.iactive[ai] = b;
         if (((cb >> lane) & 1u) && ci < s.list_cap) s.icand[ci] = b;
         if (((nbits >> lane) & 1u) && ni < s.list_cap) s.inew[ni] = b;
+        // the active blocks that are not new (their rank among all less that among the new)
+        if ((((ab & ~nbits) >> lane) & 1u) && ai - ni < s.list_cap) s.ihit[ai - ni] = b;
     }
     __syncthreads();
 }
@@ -365,6 +369,64 @@ __global__ void __launch_bounds__(kThreads) lru_a_kernel(Launch L) {
     }
 }
 
+// The below masks of the active blocks already in the cache (the new ones
+// get theirs from the decode): bit i says sample i is below the isovalue.
+// The count reads these 8 bytes of a block instead of its samples.  A warp
+// takes 4 blocks at a time, all eight 128-byte loads before the ballots.
+// Bound by the reads of 256 bytes a block; it runs in lru_b's launch, whose
+// own work is a few latency-bound tiles, rather than in one of its own.
+// Nothing here reads what the cache update or the decode's commit changes (a
+// hit keeps its slot).  Called by all threads of the block.
+constexpr uint32_t kMaskBlocks = 4;
+
+template <bool kOne>
+__device__ __forceinline__ void hit_mask_work(const Launch &L, uint32_t *pre) {
+    const uint32_t total = launch_prefix<kOne>(
+        L, [&](uint32_t v) {
+            const DevState &s = vol_of<kOne>(L, v).s;
+            const Ctl *c = s.ctl;
+            const bool off = s.bmask == nullptr || (c->status & (kStatusBudget | kStatusTimeout)) != 0;
+            return off ? 0u : ceil_div(c->n_active - c->n_new, kMaskBlocks);
+        },
+        pre);
+    const int lane = threadIdx.x & 31;
+    const uint32_t stride = (gridDim.x * blockDim.x) >> 5;
+    auto slot_of = [&](uint32_t t, uint32_t &v) {       // the slot of block lane % 4 of warp tile t
+        v = 0u;
+        if (t >= total) return -1;
+        v = item_vol<kOne>(pre, L.n, t);
+        const DevState &s = vol_of<kOne>(L, v).s;
+        const uint32_t i = (t - item_base<kOne>(pre, v)) * kMaskBlocks + (lane & (kMaskBlocks - 1));
+        if (i >= s.ctl->n_active - s.ctl->n_new) return -1;
+        const uint32_t b = s.ihit[i];
+        const int32_t sl = in_bounds(b < vol_of<kOne>(L, v).g.nb, &s.ctl->status) ? s.islot[b] : -1;
+        return sl >= 0 && in_bounds((uint32_t)sl < s.ctl->cap, &s.ctl->status) ? sl : -1;
+    };
+    uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, v_next;
+    int32_t next = slot_of(t, v_next);
+    for (; t < total; t += stride) {
+        const int32_t mine = next;
+        const uint32_t v = v_next;
+        next = slot_of(t + stride, v_next);              // loaded a tile ahead
+        const DevState &s = vol_of<kOne>(L, v).s;
+        const float iso = s.ctl->params.iso;
+        float x[kMaskBlocks][2];
+#pragma unroll
+        for (int q = 0; q < (int)kMaskBlocks; q++) {
+            const int32_t sl = __shfl_sync(0xffffffffu, mine, q);
+#pragma unroll
+            for (int h = 0; h < 2; h++) x[q][h] = sl >= 0 ? s.slots[(size_t)sl * 64 + 32 * h + lane] : 0.0f;
+        }
+        unsigned long long m = 0;
+#pragma unroll
+        for (int q = 0; q < (int)kMaskBlocks; q++) {
+            const uint32_t lo = __ballot_sync(0xffffffffu, x[q][0] < iso), hi = __ballot_sync(0xffffffffu, x[q][1] < iso);
+            if (lane == q) m = ((unsigned long long)hi << 32) | lo;
+        }
+        if (lane < (int)kMaskBlocks && mine >= 0) s.bmask[mine] = m;
+    }
+}
+
 // lru_b's work: every slot stamped this epoch (hits and new assignments),
 // by index, appended after the list's surviving part.  Run by its own
 // kernel, or by the 256-thread decode kernel once its blocks are decoded
@@ -418,6 +480,8 @@ __device__ __forceinline__ void lru_b_work(const Launch &L, TileScan<kRounds> &t
         }
         __syncthreads();
     }
+    __syncthreads();                                  // `pre` is reused
+    hit_mask_work<kOne>(L, pre);
 }
 
 template <bool kOne>
@@ -484,6 +548,16 @@ __global__ void __launch_bounds__(kDecodeThreads, 768 / kDecodeThreads) decode_n
         float4 *dst = reinterpret_cast<float4 *>(s.slots + (size_t)slot * 64);
 #pragma unroll
         for (int i = 0; i < 16; i++) dst[i] = make_float4(val[4 * i], val[4 * i + 1], val[4 * i + 2], val[4 * i + 3]);
+        if (s.bmask) {                                // the block's below mask, while its samples are here
+            const float iso = c->params.iso;
+            uint32_t lo = 0, hi = 0;
+#pragma unroll
+            for (int i = 0; i < 32; i++) {
+                if (val[i] < iso) lo |= 1u << i;
+                if (val[32 + i] < iso) hi |= 1u << i;
+            }
+            s.bmask[slot] = ((unsigned long long)hi << 32) | lo;
+        }
     }
     if constexpr (decode_runs_lru_b<kDecodeThreads>()) {
         __syncthreads();                              // `pre` is lru_b's from here

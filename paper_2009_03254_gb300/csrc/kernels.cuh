@@ -20,6 +20,8 @@ struct DevState {
     uint32_t *iactive;         // I_active (kept only for debugging: nothing downstream reads it; else null)
     uint32_t *inew;            // I_new
     uint32_t *icand;           // candidates: ids of the blocks the triangle stage visits (ascending)
+    uint32_t *ihit;            // active blocks found in the cache (ascending ids; their below masks are
+                               // taken from the cache, the new blocks' by their decode)
     uint32_t list_cap;         // room of I_active, I_new and the candidates: min(nb, slot cap); longer
                                // lists mean more active blocks than slots, which the cache update refuses
     int32_t *islot;            // I_slot: block -> slot or -1
@@ -31,20 +33,20 @@ struct DevState {
     unsigned long long *desc_cull, *desc_cand, *desc_lru_a, *desc_lru_b, *desc_mc;
     Ctl *ctl;
     const uint8_t *tables;     // num_tri[256] then tri_edges[256][16]
-    uint32_t *counts;          // triangles of each candidate
-    unsigned long long *offsets; // exclusive prefix of counts: first triangle of each candidate
-    uint32_t *iocc;            // I_occ: positions in the candidate list of the occupied candidates (ascending)
+    unsigned long long *bmask; // per slot: bit i says sample i of its block is below this extraction's
+                               // isovalue (active blocks only; null where nothing counts: a serving
+                               // tick of several requests takes each request's masks on its own)
+    uint32_t *counts;          // debug access: triangles of each candidate (null in a request's view)
+    unsigned long long *offsets; // debug access: exclusive prefix of counts (null in a request's view)
+    uint32_t *iocc;            // I_occ: ids of the occupied candidates (ascending)
+    unsigned long long *ooff;  // first triangle of each occupied candidate
     unsigned long long *desc_occ;  // look-back descriptors of the occupied count (next to desc_mc)
     unsigned long long *desc_vtx;  // look-back descriptors of the vertex count (next to desc_occ; null
                                    // where indexed meshes are never made)
     unsigned long long *voff;      // indexed mesh: first vertex of each occupied candidate (null until
                                    // the first indexed extraction)
-    uint32_t *cutw;                // indexed mesh: 12 cut-edge words per candidate, written by count and
-                                   // read by emit (null until the first indexed extraction)
-    uint8_t *cases;            // 64 cell cases per candidate, written by the count pass and read by
-                               // emit instead of classifying again (null: emit classifies)
-    unsigned long long case_cap;   // candidates `cases` holds: with more, both passes act as if it were null
-    // debug copy (null unless the volume was loaded with ISO_DEBUG)
+    // debug copies (null unless the volume was loaded with ISO_DEBUG)
+    uint8_t *cases;            // 64 cell cases per candidate
     unsigned long long *dbg_edges;
 };
 
@@ -80,15 +82,16 @@ struct Plan {
     int prep, cull, lru_a, lru_b, decode, mc_count, mc_scan, mc_emit;   // CTAs per launch
     int cull_tile;       // block ranges per cull tile: 2048 or 4096
     int decode_tile;     // new blocks per decode CTA (one per thread): 64, 128 or 256
-    int count_tile;      // candidates per count CTA round (4 per warp): 16, 32 or 64
-    int scan_tile;       // counts per offset-scan tile: 1024, 2048 or 4096
+    int count_tile;      // 16, 32 or 64, and
+    int scan_tile;       // 1024, 2048 or 4096: checked and reported; one kernel counts and scans, in
+                         // tiles of kCountTile
     int emit_tile;       // candidates per emit CTA round (4 per warp): 16, 32 or 64
 };
 
 constexpr int kThreads = 256;
 constexpr int kScanTile = 4096;          // entries per tile of the cache-update scans
 constexpr int kMinCullTile = 2048;       // smallest cull tile (sizes the cull descriptors)
-constexpr int kMinMcScanTile = 1024;     // smallest offset-scan tile (sizes its descriptors)
+constexpr int kCountTile = 1024;         // candidates per tile of the count and offset scan
 constexpr int kDefaultCullTile = 4096, kDefaultDecodeTile = 128, kDefaultCountTile = 32,
               kDefaultScanTile = 2048, kDefaultEmitTile = 32;
 
@@ -103,10 +106,9 @@ void launch_front(const Launch &L, const Plan &pl, cudaStream_t st, cudaEvent_t 
 void launch_cache_update(const Launch &L, const Plan &pl, cudaStream_t st);
 // the range test alone (Ctl counters and look-back descriptors cleared by the caller)
 void launch_cull(const Launch &L, const Plan &pl, cudaStream_t st);
-// triangle stage: count, scan, emit.  A batch places the volumes' outputs
+// triangle stage: count and scan, emit.  A batch places the volumes' outputs
 // between scan and emit; a rerun into a larger output runs emit alone.
-void launch_mc_count(const Launch &L, bool debug, const Plan &pl, cudaStream_t st, bool indexed = false);
-void launch_mc_scan(const Launch &L, const Plan &pl, cudaStream_t st);
+void launch_mc_scan(const Launch &L, bool debug, const Plan &pl, cudaStream_t st, bool indexed = false);
 void launch_mc_emit(const Launch &L, bool debug, const Plan &pl, cudaStream_t st, bool indexed = false);
 // batches: per-volume isovalues from a packed array; the volumes' outputs
 // placed one after another in `bo->out` (tri_base[v] = first triangle of

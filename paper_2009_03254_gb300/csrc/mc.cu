@@ -9,17 +9,18 @@
 // active and therefore cached.  This is the refinement Section 4.4 notes
 // as possible ("checking which side the neighbor was on").
 //
-//   count   Section 4.4: stage each candidate's 5x5x5 samples, classify its
-//           64 cells, write its triangle count
-//   scan    prefix sum of the counts over the candidates (block offsets
-//           and the total) and compaction of the occupied candidates, one
-//           pass with two decoupled look-backs
+//   count and scan   Section 4.4, one pass, one candidate per thread: from
+//           the 64-bit below masks of its +group (made by the decode for
+//           the new blocks and by lru_b for the cached ones) each
+//           candidate's triangle count, by bit logic on all 64 cells at
+//           once; the counts' prefix sums (block offsets and the total) and
+//           the compaction of the occupied candidates, by decoupled
+//           look-backs side by side
 //   emit    Section 4.5, over the occupied candidates only: stage the
-//           samples (the cases kept by count arrive by asynchronous copies),
-//           per-cell offsets by warp scans, then one triangle (three
-//           vertices) per lane
+//           samples, classify, per-cell offsets by warp scans, then one
+//           triangle (three vertices) per lane
 //
-// Both passes give each warp 4 consecutive candidates at a time (a "warp
+// Emit gives each warp 4 consecutive occupied candidates at a time (a "warp
 // tile") and no warp ever waits for another one:
 //   A  slots of each block's 8 blocks of the +group (8 lanes per block)
 //   B  stage the samples in shared memory: 16 float4 rows of the block,
@@ -53,6 +54,7 @@
 #include "kernels.cuh"
 #include "launch.cuh"
 #include "mc_tables.cuh"
+#include "tile_scan.cuh"
 
 namespace bcmc {
 
@@ -72,14 +74,7 @@ struct WarpTile {                                     // one warp's shared-memor
     uint8_t cases[kBPW][64];
 };
 
-template <int kW>                                     // warps per CTA
-struct CountSmem {
-    WarpTile w[kW];
-    uint32_t win[kWinTable];                          // window rows (indexed meshes)
-    uint8_t num_tri[256];
-};
-
-template <int kW, bool kIdx>
+template <int kW, bool kIdx>                          // kW warps per CTA
 struct EmitSmem {
     WarpTile w[kW];
     float4 stage[kW][kIdx ? 24 : 96];                 // 32 triangles' vertices (indexed: indices) per warp
@@ -126,6 +121,14 @@ __device__ __forceinline__ uint32_t halo_job(int j) {
     return 1u | ((uint32_t)vec << 1) | ((uint32_t)o << 2) | ((uint32_t)src << 5) | ((uint32_t)dst << 11);
 }
 
+// cells of a block per axis inside the volume (0 to 4), 4 bits each
+__device__ __forceinline__ uint32_t cell_limits(const Geom &g, uint32_t bx, uint32_t by, uint32_t bz) {
+    const uint32_t lx = min(4u, g.nx - 1 - min(g.nx - 1, 4 * bx));
+    const uint32_t ly = min(4u, g.ny - 1 - min(g.ny - 1, 4 * by));
+    const uint32_t lz = min(4u, g.nz - 1 - min(g.nz - 1, 4 * bz));
+    return lx | (ly << 4) | (lz << 8);
+}
+
 // Per-lane constants of phases B and C.
 struct LaneConst {
     uint32_t job0, job1;                // halo jobs lane and lane + 32
@@ -148,14 +151,6 @@ struct LaneConst {
         }
     }
 };
-
-// 16-byte global -> shared copy that completes asynchronously (L2 only)
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // the 8-bit case of a cell from the 32 mask bits starting at its lower corner
 // (corner c at bit (c&1) + 5((c>>1)&1) + 25(c>>2))
@@ -221,57 +216,19 @@ __device__ __forceinline__ uint32_t lane_cut_word(const uint32_t m[4], uint32_t 
     return (lo ^ far) & w;
 }
 
-// Phases A-C for the warp tile starting at candidate `base` (count pass)
-// or at occupied candidate `base` (emit pass), nb_w of kBPW slots used.
-// Returns the per-cell triangle counts of the lane's two cells, packed one
-// byte per block: n0p for cell lane, n1p for cell lane + 32.  The count
-// pass (kEmit false) classifies and, when there is room for them
-// (keeps_cases), stores the cases; the emit pass leaves the cases in
-// wt.cases, reading the stored ones instead of classifying again under the
-// same test.  `b` is
-// this lane's block (block lane/8 of the tile) and `ci` its position in
-// the candidate list, loaded by the caller one warp tile ahead.
-//
-// With `indexed` (count pass only), nv_lane receives, in lane q, the number
-// of cut edges (vertices of the indexed mesh) of block q; `win` is the
-// window-row table in shared memory.
-//
-// With `cut_dst` (emit pass of an indexed extraction), the 12 cut-edge
-// words count kept for each of the tile's blocks are copied to
-// cut_dst + 24q (asynchronously, like the cases; the caller waits).
-// whether the count pass keeps the cases (and the emit pass reads them):
-// there is room for all of them (n_cand is final before the count starts)
-__device__ __forceinline__ bool keeps_cases(const DevState &s) {
-    return s.cases != nullptr && s.ctl->n_cand <= s.case_cap;
-}
-
-template <bool kEmit>
-__device__ __forceinline__ void stage_and_classify(const DevState &s, const Geom &g, float iso, uint32_t base,
-                                                   int nb_w, uint32_t b, uint32_t ci, WarpTile &wt,
-                                                   const LaneConst &lc, const uint8_t *num_tri, uint32_t &n0p,
-                                                   uint32_t &n1p, bool indexed, const uint32_t *win,
-                                                   uint32_t &nv_lane, uint32_t *cut_dst = nullptr) {
+// Phases A-C for the warp tile starting at an occupied candidate, nb_w of
+// kBPW blocks used; `b` is this lane's block (block lane/8 of the tile),
+// loaded by the caller one warp tile ahead.  Leaves the cases in wt.cases and
+// returns the per-cell triangle counts of the lane's two cells, packed one
+// byte per block: n0p for cell lane, n1p for cell lane + 32.  With `cut`
+// (indexed meshes), each block's 12 cut-edge words go to cut[q][0..11];
+// `win` is the window-row table in shared memory.
+__device__ __forceinline__ void stage_and_classify(const DevState &s, const Geom &g, float iso, int nb_w, uint32_t b,
+                                                   WarpTile &wt, const LaneConst &lc, const uint8_t *num_tri,
+                                                   uint32_t &n0p, uint32_t &n1p, uint32_t (*cut)[24],
+                                                   const uint32_t *win) {
     const int lane = threadIdx.x & 31, bq = lane >> 3, bo = lane & 7;
     const uint32_t slab = g.nbx * g.nby;
-    const bool keep = keeps_cases(s);                     // uniform
-    const bool stored = kEmit && keep;
-    // The stored cases of the tile's blocks, copied to shared memory while
-    // the samples are staged (16 lanes x 16 bytes; both ends 16-byte
-    // aligned).  The emit pass's blocks are occupied candidates, not
-    // consecutive ones: block q's position in the candidate list is `ci` of
-    // lane 8q.
-    if (stored || (kEmit && cut_dst)) {   // uniform
-        // lanes 0-15: the cases of block lane / 4; lanes 16-27: the cut-edge
-        // words of block (lane - 16) / 3, 16 bytes each
-        const int qk = (cut_dst && lane >= 16) ? min((lane - 16) / 3, 3) : (lane >> 2);
-        const uint32_t cq = __shfl_sync(0xffffffffu, ci, qk * 8);
-        if (stored && lane < 4 * nb_w)
-            cp_async16(&wt.cases[lane >> 2][16 * (lane & 3)], s.cases + (size_t)cq * 64 + 16 * (lane & 3));
-        if (cut_dst && lane >= 16 && lane < 16 + 3 * nb_w) {
-            const int k = (lane - 16) % 3;
-            cp_async16(cut_dst + 24 * qk + 4 * k, s.cutw + (size_t)cq * 12 + 4 * k);
-        }
-    }
     // ---- A: +group slots
     if (bq < nb_w) {
         uint32_t bx, by, bz;
@@ -282,10 +239,7 @@ __device__ __forceinline__ void stage_and_classify(const DevState &s, const Geom
         wt.nslot[bq][bo] = exists && in_bounds(nbid < g.nb, &s.ctl->status) ? s.islot[nbid] : -1;
         if (bo == 0) {
             wt.bid[bq] = b;
-            const uint32_t lx = min(4u, g.nx - 1 - min(g.nx - 1, 4 * bx));
-            const uint32_t ly = min(4u, g.ny - 1 - min(g.ny - 1, 4 * by));
-            const uint32_t lz = min(4u, g.nz - 1 - min(g.nz - 1, 4 * bz));
-            wt.lim[bq] = lx | (ly << 4) | (lz << 8);
+            wt.lim[bq] = cell_limits(g, bx, by, bz);
         }
     }
     __syncwarp();
@@ -328,70 +282,42 @@ __device__ __forceinline__ void stage_and_classify(const DevState &s, const Geom
             }
     }
     __syncwarp();
-    // ---- C: classify (or take the stored cases) and count
+    // ---- C: classify and count
     n0p = 0;
     n1p = 0;
 #pragma unroll
     for (int q = 0; q < kBPW; q++) {
         if (q >= nb_w) continue;          // warp-uniform
-        uint32_t cs[2];
-        if (stored) {
-            if (q == 0) {                 // the copies issued before staging
-                cp_async_wait_all();
-                __syncwarp();
-            }
-            cs[0] = wt.cases[q][lane];
-            cs[1] = wt.cases[q][lane + 32];
-        } else {
-            uint32_t m[4];
-            below_mask(&wt.halo[q][0], lc, iso, m);
-            const uint32_t lim = wt.lim[q];
+        uint32_t cs[2], m[4];
+        below_mask(&wt.halo[q][0], lc, iso, m);
+        const uint32_t lim = wt.lim[q];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const uint32_t lo = lc.up[h] ? m[h + 1] : m[h];
+            const uint32_t hi = lc.up[h] ? m[h + 2] : m[h + 1];
+            cs[h] = case_bits(__funnelshift_r(lo, hi, lc.cshift[h]));
+        }
+        if (lim != 0x444u) {              // warp-uniform: cells past the volume's last sample are empty
 #pragma unroll
             for (int h = 0; h < 2; h++) {
-                const uint32_t lo = lc.up[h] ? m[h + 1] : m[h];
-                const uint32_t hi = lc.up[h] ? m[h + 2] : m[h + 1];
-                cs[h] = case_bits(__funnelshift_r(lo, hi, lc.cshift[h]));
+                const uint32_t cell = (uint32_t)lane + 32u * h;
+                const bool valid = (cell & 3u) < (lim & 15u) && ((cell >> 2) & 3u) < ((lim >> 4) & 15u) &&
+                                   (cell >> 4) < (lim >> 8);
+                cs[h] = valid ? cs[h] : 0u;
             }
-            if (lim != 0x444u) {          // warp-uniform: cells past the volume's last sample are empty
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    const uint32_t cell = (uint32_t)lane + 32u * h;
-                    const bool valid = (cell & 3u) < (lim & 15u) && ((cell >> 2) & 3u) < ((lim >> 4) & 15u) &&
-                                       (cell >> 4) < (lim >> 8);
-                    cs[h] = valid ? cs[h] : 0u;
-                }
-            }
-            if (!kEmit && keep) {         // uniform: keep them for the emit pass
-#pragma unroll
-                for (int h = 0; h < 2; h++)
-                    if (in_bounds(base + q < s.list_cap, &s.ctl->status))
-                        s.cases[(size_t)(base + q) * 64 + lane + 32 * h] = (uint8_t)cs[h];
-            }
-            // uniform: count the cut edges, keep the words for emit; a block
-            // without triangles has none (a cut edge makes its cell cross),
-            // and nothing reads its words
-            if (!kEmit && indexed && __any_sync(0xffffffffu, (num_tri[cs[0]] | num_tri[cs[1]]) != 0u)) {
-                const uint32_t w = lane_cut_word(m, lim, win);
-                const uint32_t nv = __reduce_add_sync(0xffffffffu, __popc(w));
-                if (lane == q) nv_lane = nv;
-                if (lane < 12 && in_bounds(base + q < s.list_cap, &s.ctl->status))
-                    s.cutw[(size_t)(base + q) * 12 + lane] = w;
-            }
+        }
+        if (cut) {                        // compile-time: the block's cut edges
+            const uint32_t w = lane_cut_word(m, lim, win);
+            if (lane < 12) cut[q][lane] = w;
         }
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            if (kEmit && !stored) wt.cases[q][lane + 32 * h] = (uint8_t)cs[h];
+            wt.cases[q][lane + 32 * h] = (uint8_t)cs[h];
             const uint32_t n = num_tri[cs[h]];
             if (h == 0) n0p |= n << (8 * q);
             else n1p |= n << (8 * q);
         }
     }
-}
-
-__device__ __forceinline__ uint32_t warp_sum(uint32_t x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
 }
 
 // candidates the triangle stage visits: none once the cache update failed
@@ -400,163 +326,238 @@ __device__ __forceinline__ uint32_t mc_candidates(const Ctl *c) {
     return (c->status & (kStatusBudget | kStatusTimeout | kStatusTimeoutLru)) ? 0u : c->n_cand;
 }
 
-// A warp tile located in the launch: volume, first entry, entries used,
-// and for this lane's block (entry first + lane/8) its position in the
-// candidate list and its block id, read ahead.  The count pass walks the
-// candidates; the emit pass walks the occupied ones (kOcc).
+// A warp tile located in the launch: volume, first occupied candidate,
+// blocks used, and this lane's block (entry first + lane/8), read ahead.
 struct TileRef {
-    uint32_t v, base, nb_w, b, ci;
+    uint32_t v, base, nb_w, b;
 };
 
-template <bool kOne, bool kOcc = false>
+template <bool kOne>
 __device__ __forceinline__ TileRef locate_tile(const Launch &L, const uint32_t *pre, uint32_t t, uint32_t total) {
-    TileRef r{0u, 0u, 0u, 0u, 0u};
+    TileRef r{0u, 0u, 0u, 0u};
     if (t >= total) return r;
     r.v = item_vol<kOne>(pre, L.n, t);
     const DevState &s = vol_of<kOne>(L, r.v).s;
-    const uint32_t n = kOcc ? s.ctl->n_occ : s.ctl->n_cand;
+    const uint32_t n = s.ctl->n_occ;
     r.base = (t - item_base<kOne>(pre, r.v)) * kBPW;
     r.nb_w = min((uint32_t)kBPW, n - r.base);
     const uint32_t i = r.base + ((uint32_t)(threadIdx.x & 31) >> 3);
-    if (i < n) {
-        r.ci = kOcc ? s.iocc[i] : i;
-        r.b = s.icand[r.ci];
-    }
+    if (i < n) r.b = s.iocc[i];
     return r;
 }
 
 }  // namespace
 
-// ================================================================ count (Section 4.4)
+// ================================================================ count and scan (Section 4.4)
+//
+// One candidate per thread.  Its 64 cells are handled together as 64-bit
+// masks: corner c's mask says, per cell, whether that corner is below the
+// isovalue; the eight masks are the block's own below mask and its
+// neighbours' shifted in.  A cell's triangles follow from the case rule
+// without the table: its segments link into C cycles through its E cut
+// edges, a cycle of length l is fanned into l - 2 triangles, so it has
+// E - 2C.  The cycles separate the regions of the cube's surface, one fewer
+// than there are regions: C = B + A - 1 with B the groups of below corners
+// joined by cube edges and A those of above corners joined by edges and
+// face diagonals (a face with two diagonal below corners cuts each off on
+// its own).  A is 2 exactly when two opposite corners are above alone, else
+// 1; B counts the below corners with no below neighbour, plus one if any
+// other exist, plus one more for two opposite parallel edges.  Every term
+// is a mask, and a block's count the sum of their popcounts.
+//
+// The counting reads 8 bytes a block of each +group (L2 holds most of them)
+// instead of staging 5x5x5 samples.
 
-template <int kW, bool kOne, bool kIdx>
-__global__ void __launch_bounds__(32 * kW, 40 / kW) mc_count_kernel(Launch L) {   // 1280 threads per SM
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    CountSmem<kW> &sm = *reinterpret_cast<CountSmem<kW> *>(smem_raw);
-    __shared__ uint32_t pre[kMaxBatch + 1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint8_t *tables = vol_of<kOne>(L, 0).s.tables;
-    for (int i = threadIdx.x; i < 256; i += 32 * kW) sm.num_tri[i] = tables[i];
-    if (kIdx) load_window_rows(sm.win);
-    const uint32_t total = launch_prefix<kOne>(
-        L, [&](uint32_t v) { return ceil_div(mc_candidates(vol_of<kOne>(L, v).s.ctl), kBPW); }, pre);
-    __syncthreads();                                      // the table
-    LaneConst lc;
-    lc.init(lane);
-    WarpTile &wt = sm.w[warp];
-    const uint32_t stride = gridDim.x * kW;
-    uint32_t t = blockIdx.x * kW + warp;
-    TileRef nxt = locate_tile<kOne>(L, pre, t, total);
-    for (; t < total; t += stride) {
-        const TileRef cur = nxt;
-        nxt = locate_tile<kOne>(L, pre, t + stride, total);   // next warp tile's block, loaded early
-        const DevState &s = vol_of<kOne>(L, cur.v).s;
-        const float iso = s.ctl->params.iso;
-        uint32_t n0p, n1p, nv = 0;
-        stage_and_classify<false>(s, vol_of<kOne>(L, cur.v).g, iso, cur.base, (int)cur.nb_w, cur.b, 0u, wt, lc,
-                                  sm.num_tri, n0p, n1p, kIdx, sm.win, nv);
-        const uint32_t r0 = warp_sum(n0p), r1 = warp_sum(n1p);   // per-byte sums <= 160: no carries
-        if (lane < (int)cur.nb_w)       // triangles (<= 320) in the low 16 bits, vertices (<= 300) above
-            s.counts[cur.base + lane] = ((r0 >> (8 * lane)) & 0xFFu) + ((r1 >> (8 * lane)) & 0xFFu) + (nv << 16);
-    }
+__device__ __forceinline__ unsigned long long in_x(unsigned long long a, unsigned long long n) {   // sample (x+1, y, z)
+    return ((a >> 1) & 0x7777777777777777ull) | ((n << 3) & 0x8888888888888888ull);
+}
+__device__ __forceinline__ unsigned long long in_y(unsigned long long a, unsigned long long n) {   // (x, y+1, z)
+    return ((a >> 4) & 0x0FFF0FFF0FFF0FFFull) | ((n << 12) & 0xF000F000F000F000ull);
+}
+__device__ __forceinline__ unsigned long long in_z(unsigned long long a, unsigned long long n) {   // (x, y, z+1)
+    return (a >> 16) | (n << 48);
 }
 
-// ================================================================ scan (Section 4.4)
-//
-// Exclusive prefix of the candidates' counts -> 64-bit offsets, and the
-// compacted positions of the occupied candidates (I_occ: the blocks the
-// emit pass visits, Section 4.4); the last tile of a volume writes both
-// totals.  kScanItems = 256 * kPT counts per tile, kPT per thread.  Every volume has at least one item; its item 0
-// records how many look-back descriptors the volume used (the next prep
-// clears them).
+// the corner masks m[c] of block b's cells; cells outside the volume (not in
+// the returned mask `valid`) hold anything
+__device__ __forceinline__ void corner_masks(const DevState &s, const Geom &g, uint32_t b, unsigned long long (&m)[8],
+                                             uint32_t &lim) {
+    uint32_t bx, by, bz;
+    block_coords(g, b, bx, by, bz);
+    const bool e[3] = {bx + 1 < g.nbx, by + 1 < g.nby, bz + 1 < g.nbz};
+    lim = cell_limits(g, bx, by, bz);
+    const uint32_t slab = g.nbx * g.nby;
+    int32_t sl[8];
+#pragma unroll
+    for (int o = 0; o < 8; o++) {                        // slots of the +group, all loads first
+        const bool in = (!(o & 1) || e[0]) && (!(o & 2) || e[1]) && (!(o & 4) || e[2]);
+        const uint32_t id = b + ((o & 1) ? 1u : 0u) + ((o & 2) ? g.nbx : 0u) + ((o & 4) ? slab : 0u);
+        sl[o] = in && in_bounds(id < g.nb, &s.ctl->status) ? s.islot[id] : -1;
+    }
+    unsigned long long n[8];
+#pragma unroll
+    for (int o = 0; o < 8; o++)
+        n[o] = sl[o] >= 0 && in_bounds((uint32_t)sl[o] < s.ctl->cap, &s.ctl->status) ? s.bmask[sl[o]] : 0ull;
+    const unsigned long long x23 = in_x(n[2], n[3]), x45 = in_x(n[4], n[5]), x67 = in_x(n[6], n[7]);
+    m[0] = n[0];
+    m[1] = in_x(n[0], n[1]);
+    m[2] = in_y(n[0], n[2]);
+    m[3] = in_y(m[1], x23);
+    m[4] = in_z(n[0], n[4]);
+    m[5] = in_z(m[1], x45);
+    m[6] = in_z(m[2], in_y(n[4], n[6]));
+    m[7] = in_z(m[3], in_y(x45, x67));
+}
 
-template <int kPT, bool kOne>
-__global__ void __launch_bounds__(kThreads) mc_scan_kernel(Launch L) {
-    constexpr int kWarps = kThreads / 32;
-    constexpr uint32_t kScanItems = kThreads * kPT;
-    __shared__ uint32_t wsum[kWarps], wocc[kWarps], wvtx[kWarps];
-    __shared__ unsigned long long s_excl[3];
+// cells with x < lim.x, y < lim.y, z < lim.z
+__device__ __forceinline__ unsigned long long valid_cells(uint32_t lim) {
+    if (lim == 0x444u) return ~0ull;
+    const uint32_t lx = lim & 15u, ly = (lim >> 4) & 15u, lz = lim >> 8;
+    return ((1ull << lx) - 1ull) * 0x1111111111111111ull & (((1ull << (4 * ly)) - 1ull) * 0x0001000100010001ull) &
+           (lz >= 4u ? ~0ull : (1ull << (16 * lz)) - 1ull);
+}
+
+__device__ __forceinline__ uint32_t count_triangles(const unsigned long long (&m)[8], unsigned long long valid) {
+    uint32_t edges = 0, cycles = 0;
+    unsigned long long joined = 0, all = ~0ull;
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+        all &= m[c];
+        cycles += __popcll(m[c] & ~(m[c ^ 1] | m[c ^ 2] | m[c ^ 4]) & valid);        // lone below corners
+#pragma unroll
+        for (int d = 1; d < 8; d <<= 1)
+            if (!(c & d)) {
+                edges += __popcll((m[c] ^ m[c | d]) & valid);
+                joined |= m[c] & m[c | d];
+            }
+    }
+    cycles += __popcll(joined & ~all & valid);
+    // two opposite parallel edges below, the rest above (6 ways), or two
+    // opposite corners above, the rest below (4 ways): one cycle more
+    unsigned long long more = 0;
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) {                    // edges along d at offsets 0, p, q, p | q
+        const int p = d == 1 ? 2 : 1, q = d == 4 ? 2 : 4;
+        more |= m[0] & m[d] & m[p | q] & m[7] & ~(m[p] | m[p | d] | m[q] | m[q | d]);
+        more |= m[p] & m[p | d] & m[q] & m[q | d] & ~(m[0] | m[d] | m[p | q] | m[7]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        unsigned long long six = ~(m[c] | m[7 - c]);
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            if (k != c && k != 7 - c) six &= m[k];
+        more |= six;
+    }
+    cycles += __popcll(more & valid);
+    return edges - 2u * cycles;
+}
+
+// the cut edges of the block's 5x5x5 window: a cell counts its three edges at
+// its lower corner and, as the last one along an axis, those on its far side
+__device__ __forceinline__ uint32_t count_vertices(const unsigned long long (&m)[8], unsigned long long valid,
+                                                   uint32_t lim) {
+    unsigned long long last[3];
+    if (lim == 0x444u) {
+        last[0] = 0x8888888888888888ull;
+        last[1] = 0xF000F000F000F000ull;
+        last[2] = 0xFFFF000000000000ull;
+    } else {
+        const uint32_t lx = lim & 15u, ly = (lim >> 4) & 15u, lz = lim >> 8;
+        if (!lx || !ly || !lz) return 0u;
+        last[0] = valid & ~valid_cells(lim - 1u);
+        last[1] = valid & ~valid_cells(lim - 16u);
+        last[2] = valid & ~valid_cells(lim - 256u);
+    }
+    uint32_t n = 0;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const int p = (a + 1) % 3, q = (a + 2) % 3;      // the other two axes
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int c = ((k & 1) << p) | ((k >> 1) << q);
+            unsigned long long w = (m[c] ^ m[c | (1 << a)]) & valid;
+            if (k & 1) w &= last[p];
+            if (k & 2) w &= last[q];
+            n += __popcll(w);
+        }
+    }
+    return n;
+}
+
+// Tiles of kCountTile candidates: counts, the tile's prefixes from up to three
+// look-backs side by side, then the occupied candidates' ids and offsets;
+// the last tile of a volume writes the totals.  Every volume has at least
+// one item; its item 0 records how many look-back descriptors the volume
+// used (the next prep clears them).
+struct ScanSmem {
+    static constexpr int kR = kCountTile / kThreads;
+    TileScan<kR> tri, occ, vtx;
+    uint32_t val[kR][kThreads];       // triangles (9 bits), vertices (9), triangles before in the warp (14)
+};
+
+template <bool kOne, bool kIdx>
+__global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
+    constexpr int kR = ScanSmem::kR;
+    constexpr uint32_t kScanItems = kCountTile;
+    __shared__ ScanSmem sm;
     __shared__ uint32_t pre[kMaxBatch + 1];
     __shared__ uint32_t s_item;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
     const uint32_t total = launch_prefix<kOne>(
         L, [&](uint32_t v) { return max(1u, ceil_div(mc_candidates(vol_of<kOne>(L, v).s.ctl), kScanItems)); },
         pre);
     while (true) {
-        if (threadIdx.x == 0) s_item = atomicAdd(&L.ctr[kLcScan], 1u);
-        __syncthreads();
-        const uint32_t x = s_item;
-        __syncthreads();
+        const uint32_t x = next_item(&L.ctr[kLcScan], &s_item);
         if (x >= total) break;
         const uint32_t v = item_vol<kOne>(pre, L.n, x);
         const DevState &s = vol_of<kOne>(L, v).s;
+        const Geom &g = vol_of<kOne>(L, v).g;
         Ctl *c = s.ctl;
         const uint32_t tile = x - item_base<kOne>(pre, v);
         const uint32_t n = mc_candidates(c);
         const uint32_t ntiles = ceil_div(n, kScanItems);
         if (tile == 0 && threadIdx.x == 0) c->mc_tiles = ntiles;
         if (ntiles == 0) continue;                        // block-uniform
-        const bool indexed = (c->params.flags & kParamIndexed) != 0;   // block-uniform
-        const uint32_t i0 = tile * kScanItems + threadIdx.x * kPT;
-        uint32_t v8[kPT], sum = 0, occ = 0, vsum = 0;
-        const bool full = i0 + kPT <= n;                  // the thread's counts in 16-byte loads
-        if (full) {
-#pragma unroll
-            for (int k = 0; k < kPT / 4; k++) {
-                const uint4 q = __ldg(reinterpret_cast<const uint4 *>(s.counts + i0) + k);
-                v8[4 * k] = q.x;
-                v8[4 * k + 1] = q.y;
-                v8[4 * k + 2] = q.z;
-                v8[4 * k + 3] = q.w;
+        const uint32_t i0 = tile * kScanItems + threadIdx.x;
+#pragma unroll 1
+        for (int r = 0; r < kR; r++) {
+            const uint32_t i = i0 + r * kThreads;
+            uint32_t nt = 0, nv = 0;
+            if (i < n) {
+                unsigned long long m[8];
+                uint32_t lim;
+                corner_masks(s, g, s.icand[i], m, lim);
+                const unsigned long long valid = valid_cells(lim);
+                nt = count_triangles(m, valid);
+                if (kIdx) nv = count_vertices(m, valid, lim);
+                if (s.counts) s.counts[i] = nt | (nv << 16);
             }
-        } else {
-#pragma unroll
-            for (int k = 0; k < kPT; k++) v8[k] = i0 + k < n ? s.counts[i0 + k] : 0u;
-        }
-#pragma unroll
-        for (int k = 0; k < kPT; k++) {
-            sum += v8[k] & 0xFFFFu;                       // triangles | vertices << 16
-            vsum += v8[k] >> 16;
-            occ += (v8[k] & 0xFFFFu) != 0u;
-        }
-        // triangles in the low 20 bits, occupied candidates above (a warp
-        // holds at most 32 * 16 * 320 triangles and 512 candidates: no carry)
-        const uint32_t own = sum | (occ << 20);
-        uint32_t incl = own, vincl = vsum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (indexed) {
+            uint32_t incl = nt;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, vincl, o);
-                if (lane >= o) vincl += t;
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
             }
-        }
-        if (lane == 31) {
-            wsum[warp] = incl & 0xFFFFFu;
-            wocc[warp] = incl >> 20;
-            wvtx[warp] = vincl;
+            const uint32_t ob = __ballot_sync(0xffffffffu, nt != 0u);
+            const uint32_t vsum = kIdx ? __reduce_add_sync(0xffffffffu, nv) : 0u;
+            if (lane == 31) {
+                sm.tri.cnt[r][warp] = incl;
+                sm.occ.cnt[r][warp] = __popc(ob);
+                if (kIdx) sm.vtx.cnt[r][warp] = vsum;
+            }
+            sm.val[r][threadIdx.x] = nt | (nv << 9) | ((incl - nt) << 18);
         }
         __syncthreads();
         // warp 0: triangle offsets; warp 1: occupied positions; warp 2: vertex offsets
-        if (warp < 2 || (warp == 2 && indexed)) {
-            uint32_t *ws = warp == 0 ? wsum : (warp == 1 ? wocc : wvtx);
-            const uint32_t w = lane < kWarps ? ws[lane] : 0u;
-            uint32_t wi = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, wi, o);
-                if (lane >= o) wi += t;
-            }
-            const uint32_t tot = __shfl_sync(0xffffffffu, wi, kWarps - 1);
-            if (lane < kWarps) ws[lane] = wi - w;                        // exclusive warp offsets
+        if (warp < (kIdx ? 3 : 2)) {
+            TileScan<kR> &ts = warp == 0 ? sm.tri : (warp == 1 ? sm.occ : sm.vtx);
+            const uint32_t tot = scan_tile_counts(ts);
             unsigned long long *desc = warp == 0 ? s.desc_mc : (warp == 1 ? s.desc_occ : s.desc_vtx);
             const unsigned long long excl = lookback_exclusive(desc, tile, tot, &c->status, kStatusTimeoutScan);
             if (lane == 0) {
-                s_excl[warp] = excl;
+                ts.excl = excl;
                 if (tile == ntiles - 1) {
                     if (warp == 0) c->n_tri = excl + tot;
                     else if (warp == 1) c->n_occ = (uint32_t)(excl + tot);
@@ -565,38 +566,48 @@ __global__ void __launch_bounds__(kThreads) mc_scan_kernel(Launch L) {
             }
         }
         __syncthreads();
-        const uint32_t before = incl - own;                              // this thread's exclusive prefix in the warp
-        unsigned long long run = s_excl[0] + wsum[warp] + (before & 0xFFFFFu);
-        uint32_t orun = (uint32_t)s_excl[1] + wocc[warp] + (before >> 20);
-        if (indexed) {
-            unsigned long long vrun = s_excl[2] + wvtx[warp] + (vincl - vsum);
+#pragma unroll 1
+        for (int r = 0; r < kR; r++) {
+            const uint32_t i = i0 + r * kThreads;
+            const uint32_t val = sm.val[r][threadIdx.x], nt = val & 511u, nv = (val >> 9) & 511u;
+            const unsigned long long run = sm.tri.excl + sm.tri.cnt[r][warp] + (val >> 18);
+            const uint32_t ob = __ballot_sync(0xffffffffu, nt != 0u);
+            unsigned long long vrun = 0;
+            if (kIdx) {
+                uint32_t vincl = nv;
 #pragma unroll
-            for (int k = 0; k < kPT; k++) {
-                if (i0 + k < n) s.offsets[i0 + k] = run;
-                if ((v8[k] & 0xFFFFu) && in_bounds(orun < s.list_cap, &c->status)) {
-                    s.voff[orun] = vrun;
-                    s.iocc[orun++] = i0 + k;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(0xffffffffu, vincl, o);
+                    if (lane >= o) vincl += t;
                 }
-                run += v8[k] & 0xFFFFu;
-                vrun += v8[k] >> 16;
+                vrun = sm.vtx.excl + sm.vtx.cnt[r][warp] + (vincl - nv);
             }
-        } else {
-            unsigned long long ofs[kPT];
-#pragma unroll
-            for (int k = 0; k < kPT; k++) {
-                ofs[k] = run;
-                if (v8[k] && in_bounds(orun < s.list_cap, &c->status)) s.iocc[orun++] = i0 + k;
-                run += v8[k];
+            if (i < n && s.offsets) s.offsets[i] = run;
+            const uint32_t at = (uint32_t)sm.occ.excl + sm.occ.cnt[r][warp] + __popc(ob & lt);
+            if (nt && in_bounds(at < s.list_cap, &c->status)) {
+                s.iocc[at] = s.icand[i];
+                s.ooff[at] = run;
+                if (kIdx) s.voff[at] = vrun;
             }
-            if (full) {
+        }
+        __syncthreads();
+    }
+}
+
+// debug volumes: the 64 cell cases of every candidate
+__global__ void __launch_bounds__(kThreads) debug_cases_kernel(Launch L) {
+    const DevState &s = L.one.s;
+    const uint32_t n = mc_candidates(s.ctl);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        unsigned long long m[8];
+        uint32_t lim;
+        corner_masks(s, L.one.g, s.icand[i], m, lim);
+        const unsigned long long valid = valid_cells(lim);
+        for (int cell = 0; cell < 64; cell++) {
+            uint32_t cs = 0;
 #pragma unroll
-                for (int k = 0; k < kPT / 2; k++)
-                    reinterpret_cast<ulonglong2 *>(s.offsets + i0)[k] = make_ulonglong2(ofs[2 * k], ofs[2 * k + 1]);
-            } else {
-#pragma unroll
-                for (int k = 0; k < kPT; k++)
-                    if (i0 + k < n) s.offsets[i0 + k] = ofs[k];
-            }
+            for (int c = 0; c < 8; c++) cs |= (uint32_t)(((m[c] & valid) >> cell) & 1ull) << c;
+            s.cases[(size_t)i * 64 + cell] = (uint8_t)cs;
         }
     }
 }
@@ -640,10 +651,10 @@ __device__ __forceinline__ void emit_body(const Launch &L) {
     float4 *stage = sm.stage[warp];
     const uint32_t stride = gridDim.x * kW;
     uint32_t t = blockIdx.x * kW + warp;
-    TileRef nxt = locate_tile<kOne, true>(L, pre, t, total);
+    TileRef nxt = locate_tile<kOne>(L, pre, t, total);
     for (; t < total; t += stride) {
         const TileRef cur = nxt;
-        nxt = locate_tile<kOne, true>(L, pre, t + stride, total);   // next warp tile's blocks, loaded early
+        nxt = locate_tile<kOne>(L, pre, t + stride, total);   // next warp tile's blocks, loaded early
         const DevState &s = vol_of<kOne>(L, cur.v).s;
         const Geom &g = vol_of<kOne>(L, cur.v).g;
         const Ctl *c = s.ctl;
@@ -653,12 +664,9 @@ __device__ __forceinline__ void emit_body(const Launch &L) {
         float4 *__restrict__ out = reinterpret_cast<float4 *>(c->params.out);
         const uint32_t base = cur.base;
         const int nb_w = (int)cur.nb_w;
-        uint32_t n0p, n1p, unused = 0;
-        stage_and_classify<true>(s, g, iso, base, nb_w, cur.b, cur.ci, wt, lc, sm.num_tri, n0p, n1p, false, nullptr,
-                                 unused, kIdx ? &sm.cut[warp][0][0] : nullptr);
-        // consecutive occupied candidates have adjacent outputs (the empty
-        // ones between them add nothing): the tile starts at its first block's
-        const uint32_t first_ci = __shfl_sync(0xffffffffu, cur.ci, 0);
+        uint32_t n0p, n1p;
+        stage_and_classify(s, g, iso, nb_w, cur.b, wt, lc, sm.num_tri, n0p, n1p, kIdx ? sm.cut[warp] : nullptr,
+                           sm.win);
         // per-cell offsets inside the warp tile: two packed scans (byte q = block q)
         uint32_t i0 = n0p, i1 = n1p;
 #pragma unroll
@@ -672,7 +680,9 @@ __device__ __forceinline__ void emit_body(const Launch &L) {
         for (int q = 0; q < kBPW; q++)
             if (q < nb_w) wtot += ((s0 >> (8 * q)) & 0xFFu) + ((s1 >> (8 * q)) & 0xFFu);
         if (wtot == 0) continue;                       // warp-uniform
-        const unsigned long long gbase = s.offsets[first_ci];
+        // consecutive occupied candidates have adjacent outputs: the tile starts
+        // at its first block's
+        const unsigned long long gbase = s.ooff[base];
         unsigned long long vt = 0;                     // indexed: the tile's first vertex
         if constexpr (kIdx) {
             // Per block, lanes 0-11 take one word each of its cut edges and the
@@ -680,8 +690,7 @@ __device__ __forceinline__ void emit_body(const Launch &L) {
             // in vertex order: axis, then sample), and list the word's edges
             // in the vertex map `tm` at their ranks.
             vt = s.voff[base];
-            cp_async_wait_all();                       // the words (and cases) copied during staging
-            __syncwarp();
+            __syncwarp();                              // the words
             uint32_t nvt = 0;
             const int lk = lane % 12, la = lk >> 2, lr = lk & 3;
             for (int qq = 0; qq < nb_w; qq += 2) {     // lanes 0-11: block qq, lanes 12-23: block qq + 1
@@ -877,11 +886,6 @@ __global__ void __launch_bounds__(32 * kW, 32 / kW) mc_emit_indexed_kernel(Launc
 namespace {
 
 template <int kW, bool kOne, bool kIdx>
-void count_w(const Launch &L, int grid, cudaStream_t st) {
-    mc_count_kernel<kW, kOne, kIdx><<<grid, 32 * kW, sizeof(CountSmem<kW>), st>>>(L);
-}
-
-template <int kW, bool kOne, bool kIdx>
 void emit_w(const Launch &L, bool debug, int grid, cudaStream_t st) {
     constexpr size_t bytes = sizeof(EmitSmem<kW, kIdx>);
     if constexpr (kIdx) {
@@ -929,31 +933,6 @@ int emit_occupancy(bool single) {
                     occupancy(mc_emit_kernel<kW, true, false>, 32 * kW, sizeof(EmitSmem<kW, false>)));
 }
 
-template <int kW>
-int count_occupancy(bool single) {
-    raise_smem(mc_count_kernel<kW, false, false>, sizeof(CountSmem<kW>));
-    raise_smem(mc_count_kernel<kW, true, false>, sizeof(CountSmem<kW>));
-    raise_smem(mc_count_kernel<kW, true, true>, sizeof(CountSmem<kW>));
-    if (single)   // the soup's and the indexed mesh's counts share the CTA count
-        return std::min(occupancy(mc_count_kernel<kW, true, false>, 32 * kW, sizeof(CountSmem<kW>)),
-                        occupancy(mc_count_kernel<kW, true, true>, 32 * kW, sizeof(CountSmem<kW>)));
-    return occupancy(mc_count_kernel<kW, false, false>, 32 * kW, sizeof(CountSmem<kW>));
-}
-
-template <bool kOne, bool kIdx>
-void count_any(const Launch &L, const Plan &pl, cudaStream_t st) {
-    if (pl.count_tile == 16) count_w<4, kOne, kIdx>(L, pl.mc_count, st);
-    else if (pl.count_tile == 64) count_w<16, kOne, kIdx>(L, pl.mc_count, st);
-    else count_w<8, kOne, kIdx>(L, pl.mc_count, st);
-}
-
-template <bool kOne>
-void scan_any(const Launch &L, const Plan &pl, cudaStream_t st) {
-    if (pl.scan_tile == 1024) mc_scan_kernel<4, kOne><<<pl.mc_scan, kThreads, 0, st>>>(L);
-    else if (pl.scan_tile == 4096) mc_scan_kernel<16, kOne><<<pl.mc_scan, kThreads, 0, st>>>(L);
-    else mc_scan_kernel<8, kOne><<<pl.mc_scan, kThreads, 0, st>>>(L);
-}
-
 template <bool kOne, bool kIdx>
 void emit_any(const Launch &L, bool debug, const Plan &pl, cudaStream_t st) {
     if (pl.emit_tile == 16) emit_w<4, kOne, kIdx>(L, debug, pl.mc_emit, st);
@@ -963,16 +942,11 @@ void emit_any(const Launch &L, bool debug, const Plan &pl, cudaStream_t st) {
 
 }  // namespace
 
-// tile = candidates per CTA round = 4 per warp
-void launch_mc_count(const Launch &L, bool /*debug*/, const Plan &pl, cudaStream_t st, bool indexed) {
-    if (L.vols) count_any<false, false>(L, pl, st);
-    else if (indexed) count_any<true, true>(L, pl, st);
-    else count_any<true, false>(L, pl, st);
-}
-
-void launch_mc_scan(const Launch &L, const Plan &pl, cudaStream_t st) {
-    if (L.vols) scan_any<false>(L, pl, st);
-    else scan_any<true>(L, pl, st);
+void launch_mc_scan(const Launch &L, bool debug, const Plan &pl, cudaStream_t st, bool indexed) {
+    if (L.vols) mc_scan_kernel<false, false><<<pl.mc_scan, kThreads, 0, st>>>(L);
+    else if (indexed) mc_scan_kernel<true, true><<<pl.mc_scan, kThreads, 0, st>>>(L);
+    else mc_scan_kernel<true, false><<<pl.mc_scan, kThreads, 0, st>>>(L);
+    if (debug && !L.vols) debug_cases_kernel<<<pl.mc_scan, kThreads, 0, st>>>(L);
 }
 
 // the indexed mesh is made for single volumes only
@@ -982,25 +956,15 @@ void launch_mc_emit(const Launch &L, bool debug, const Plan &pl, cudaStream_t st
     else emit_any<true, false>(L, debug, pl, st);
 }
 
-template <int kPT>
-int scan_occupancy(bool single) {
-    int occ = 0;
-    if (single) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mc_scan_kernel<kPT, true>, kThreads, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mc_scan_kernel<kPT, false>, kThreads, 0);
-    return occ;
-}
-
 void mc_occupancy(Plan *pl, bool single) {
     // every variant's shared-memory limit is raised, whichever is asked for
     const int e4 = emit_occupancy<4>(single), e8 = emit_occupancy<8>(single), e16 = emit_occupancy<16>(single);
     pl->mc_emit = std::max(1, pl->emit_tile == 16 ? e4 : (pl->emit_tile == 64 ? e16 : e8));
-    const int c4 = count_occupancy<4>(single), c8 = count_occupancy<8>(single),
-              c16 = count_occupancy<16>(single);
-    pl->mc_count = std::max(1, pl->count_tile == 16 ? c4 : (pl->count_tile == 64 ? c16 : c8));
-    const int occ = pl->scan_tile == 1024 ? scan_occupancy<4>(single)
-                                          : (pl->scan_tile == 4096 ? scan_occupancy<16>(single)
-                                                                   : scan_occupancy<8>(single));
-    pl->mc_scan = std::max(1, occ);
+    pl->mc_count = 1;
+    // the soup's and the indexed mesh's counts share the CTA count
+    pl->mc_scan = single ? std::min(occupancy(mc_scan_kernel<true, false>, kThreads, 0),
+                                    occupancy(mc_scan_kernel<true, true>, kThreads, 0))
+                         : occupancy(mc_scan_kernel<false, false>, kThreads, 0);
 }
 
 }  // namespace bcmc

@@ -315,7 +315,8 @@ extern "C" int iso_raycast(iso_volume *v, float isovalue, const iso_pinhole *cam
     // the extraction's front for this isovalue: range test, cache update, decode
     *v->host_params = Params{isovalue, kVertexFloat4, 0u, 0u, 0u, 0u, 0ull, 0ull, 0ull, 0ull, 0ull};
     ISO_CK(cudaMemcpyAsync(&v->s.ctl->params, v->host_params, sizeof(Params), cudaMemcpyHostToDevice, st));
-    const Launch L{nullptr, 1u, single_counters(v), VolEntry{v->s, v->g, v->n_cull_desc, v->n_lru_desc}};
+    Launch L{nullptr, 1u, single_counters(v), VolEntry{v->s, v->g, v->n_cull_desc, v->n_lru_desc}};
+    L.one.s.bmask = nullptr;                             // nothing counts here
     launch_front(L, v->plan, st, nullptr);
     void *scratch = nullptr;
     int rc = dalloc_bytes(&scratch, 16, v->device, st);

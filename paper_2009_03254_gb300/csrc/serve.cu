@@ -7,13 +7,15 @@
 //                    and each request's own candidate list (a tick of one
 //                    request without pins runs the single-volume range test)
 //     cache update   Algorithm 1 and the decode (Section 4.2) on the union
-//     front tail     the union's failures become every request's; each
-//                    request gets its region of the stored-cases buffer
+//     masks          each request's below masks of the union's blocks, from
+//                    one read of their samples (a lone request's come from
+//                    the cache update and the decode)
+//     front tail     the union's failures become every request's
 //   back of a tick (the server's stream, queued behind the front's event
 //   without a host round trip)
 //     count, scan    Sections 4.3-4.4 over all the tick's requests in one
-//                    launch each: a request is a "view" of the volume (own
-//                    control block, candidates, counts and offsets; shared
+//                    launch: a request is a "view" of the volume (own
+//                    control block, candidates, masks and offsets; shared
 //                    cache), the views are the entries of a batch launch
 //                    (they find no work if the union failed); on a volume
 //                    with segment ranges one launch per request (per_view)
@@ -74,9 +76,8 @@ struct ServeArgs {
     unsigned long long *desc_occ[kMaxServe];
     uint32_t cand_cap;                // room of each candidate list
     VolEntry *views;                  // the tick's views in device memory (the back's launch table)
+    unsigned long long *bmask[kMaxServe];   // per-request below masks, per slot
     uint32_t single_cull;             // one request, no pins: the single-volume range test runs instead
-    uint8_t *cases;                   // the server's stored-cases buffer (or null)
-    unsigned long long case_cap;      // its room, in candidates (64 bytes each)
 };
 
 __global__ void __launch_bounds__(kThreads) serve_prep_kernel(ServeArgs a) {
@@ -285,25 +286,61 @@ __global__ void __launch_bounds__(kThreads) serve_cull_kernel(ServeArgs a) {
     }
 }
 
+// The below masks of the union's blocks for every request of the tick (one
+// without pins takes its own from the cache update and the decode): the
+// newest n_active entries of the cache's list are their slots, in ascending
+// order, and each block's samples are read once for all the isovalues.  A warp
+// takes 4 blocks at a time.  Bound by those reads.
+template <int kT>
+__global__ void __launch_bounds__(kThreads) serve_mask_kernel(ServeArgs a) {
+    constexpr uint32_t kBlocks = 4;
+    const DevState &s = a.base.s;
+    const Ctl *c = s.ctl;
+    if (c->status & (kStatusBudget | kStatusAnyTimeout)) return;
+    const uint32_t n = c->n_active;
+    const uint32_t *list = s.lbuf[c->lpar] + c->keep_base;
+    const int lane = threadIdx.x & 31;
+    const uint32_t stride = (gridDim.x * blockDim.x) >> 5;
+    uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    auto slot_at = [&](uint32_t tile) {
+        const uint64_t i = (uint64_t)tile * kBlocks + (lane & (kBlocks - 1));
+        if (i >= n) return -1;
+        const uint32_t sl = list[i];
+        return in_bounds(sl < c->cap, &s.ctl->status) ? (int32_t)sl : -1;
+    };
+    int32_t next = slot_at(t);
+    for (; (uint64_t)t * kBlocks < n; t += stride) {
+        const int32_t mine = next;
+        next = slot_at(t + stride);
+        float x[kBlocks][2];
+#pragma unroll
+        for (int q = 0; q < (int)kBlocks; q++) {
+            const int32_t sl = __shfl_sync(0xffffffffu, mine, q);
+#pragma unroll
+            for (int h = 0; h < 2; h++) x[q][h] = sl >= 0 ? s.slots[(size_t)sl * 64 + 32 * h + lane] : 0.0f;
+        }
+#pragma unroll
+        for (int j = 0; j < kT; j++) {
+            if (j >= (int)a.k) break;                      // uniform
+            unsigned long long m = 0;
+#pragma unroll
+            for (int q = 0; q < (int)kBlocks; q++) {
+                const uint32_t lo = __ballot_sync(0xffffffffu, x[q][0] < a.iso[j]),
+                               hi = __ballot_sync(0xffffffffu, x[q][1] < a.iso[j]);
+                if (lane == q) m = ((unsigned long long)hi << 32) | lo;
+            }
+            if (lane < (int)kBlocks && mine >= 0) a.bmask[j][mine] = m;
+        }
+    }
+}
+
 // The end of a tick's front (one thread: k <= 8).  The union's failures
-// (budget, a timeout) become every request's, so the back finds no work;
-// each request, in order, gets the next region of the stored-cases buffer
-// while its candidates fit (a request without one has its cases
-// classified again by the emission, which reads the same pointer).
+// (budget, a timeout) become every request's, so the back finds no work.
 __global__ void serve_front_tail_kernel(ServeArgs a) {
     if (threadIdx.x != 0) return;
     if (a.single_cull) a.ctl[0]->n_cand = a.base.s.ctl->n_cand;   // counted by the single-volume range test
     const uint32_t fail = a.base.s.ctl->status & (kStatusBudget | kStatusAnyTimeout);
-    unsigned long long used = 0;
-    for (uint32_t j = 0; j < a.k; j++) {
-        Ctl *c = a.ctl[j];
-        c->status |= fail;
-        const unsigned long long n = c->n_cand;
-        const bool fits = a.cases != nullptr && used + n <= a.case_cap;
-        a.views[j].s.cases = fits ? a.cases + 64ull * used : nullptr;
-        a.views[j].s.case_cap = fits ? n : 0ull;
-        if (fits) used += n;
-    }
+    for (uint32_t j = 0; j < a.k; j++) a.ctl[j]->status |= fail;
 }
 
 // the tick's request control blocks, then the union's, for one readback
@@ -345,9 +382,8 @@ struct Done {
 
 struct Slot {                           // device state of one request position
     Ctl *ctl = nullptr;
-    uint32_t *icand = nullptr, *counts = nullptr;
-    unsigned long long *offsets = nullptr, *desc_cand = nullptr, *desc_mc = nullptr, *desc_occ = nullptr;
-    uint32_t *iocc = nullptr;
+    uint32_t *icand = nullptr, *iocc = nullptr;
+    unsigned long long *ooff = nullptr, *bmask = nullptr, *desc_cand = nullptr, *desc_mc = nullptr, *desc_occ = nullptr;
 };
 
 enum Stage { kFront = 0, kCount = 1, kEmit = 2 };
@@ -364,8 +400,6 @@ struct Tick {                           // requests in flight on the GPU
     uint32_t run_to = 0;                // the running round takes requests [emitted, run_to)
     ServeArgs args{};                   // its front's arguments (the back's gather reads them too)
 };
-
-constexpr uint64_t kMaxTickCaseBytes = 4ull << 30;   // stored cases of a tick, else emit classifies again
 
 }  // namespace
 
@@ -389,12 +423,11 @@ struct iso_server {
     Params *d_params = nullptr;         // the requests' outputs, copied into their control blocks
     Ctl *h_ctls[2] = {};                // pinned mirrors of d_ctls
     Params *h_params = nullptr;
-    uint8_t *cases = nullptr;           // stored cell cases of a tick's requests (count writes, emit reads)
-    uint64_t case_cap = 0;              // its room in candidates
     bool blocked = false;               // the back waits for meshes to be taken (vertex budget)
     cudaEvent_t front_done[2] = {}, count_done = nullptr;
     cudaEvent_t emit_done[kMaxServe] = {};   // each request's emission in the running round
     Plan one_plan{}, back_plan{};       // launches over one view (kOne) or up to max_batch views
+    int mask_ctas = 1;                  // CTAs of the masks' launch
     uint64_t next_ticket = 1;
     std::deque<Request> queue;
     bool has_front = false, has_back = false;
@@ -420,15 +453,17 @@ ServeArgs serve_args(const iso_server *sv, const Tick &t, const std::vector<Requ
         a.desc_cand[j] = sv->slots[p][j].desc_cand;
         a.desc_mc[j] = sv->slots[p][j].desc_mc;
         a.desc_occ[j] = sv->slots[p][j].desc_occ;
+        a.bmask[j] = sv->slots[p][j].bmask;
     }
     a.k_pin = pins ? (uint32_t)pins->size() : 0u;
     for (uint32_t j = 0; j < a.k_pin; j++) a.iso[a.k + j] = (*pins)[j].iso;
     a.back_ctr = sv->d_ctr[p];
     a.cand_cap = sv->cand_cap;
     a.views = sv->d_views[p];
-    a.cases = sv->cases;
     a.single_cull = (a.k == 1 && a.k_pin == 0) ? 1u : 0u;
-    a.case_cap = sv->case_cap;
+    // the cache update and the decode make a lone request's masks; several
+    // requests' come from serve_mask_kernel
+    a.base.s.bmask = a.single_cull ? a.bmask[0] : nullptr;
     return a;
 }
 
@@ -443,11 +478,11 @@ void free_server(iso_server *sv) {
         for (float *b : sv->back_tick.bufs) dfree_on(b, sv->stream);
     for (auto &half : sv->slots)
         for (Slot &s : half) {
-            void *p[] = {s.ctl, s.icand, s.counts, s.offsets, s.desc_cand, s.desc_mc, s.iocc};
+            void *p[] = {s.ctl, s.icand, s.bmask, s.ooff, s.desc_cand, s.desc_mc, s.iocc};
             for (void *x : p) dfree_on(x, sv->stream);
         }
     void *q[] = {sv->d_views[0], sv->d_views[1], sv->d_ctr[0], sv->d_ctr[1], sv->d_ctls[0], sv->d_ctls[1],
-                 sv->d_params, sv->cases};
+                 sv->d_params};
     for (void *x : q) dfree_on(x, sv->stream);
     cudaStreamSynchronize(sv->stream);
     (void)cudaGetLastError();
@@ -502,6 +537,12 @@ void launch_serve_cull(uint32_t kt, int ctas, const ServeArgs &a, cudaStream_t s
     else serve_cull_kernel<16, kSeg><<<ctas, kThreads, 0, st>>>(a);
 }
 
+void launch_serve_mask(const ServeArgs &a, int ctas, cudaStream_t st) {
+    if (a.k <= 2) serve_mask_kernel<2><<<ctas, kThreads, 0, st>>>(a);
+    else if (a.k <= 4) serve_mask_kernel<4><<<ctas, kThreads, 0, st>>>(a);
+    else serve_mask_kernel<8><<<ctas, kThreads, 0, st>>>(a);
+}
+
 // Admit the queue's first requests as a tick and queue its front on the
 // front stream (pins: the tick in its back, or null).
 int launch_front(iso_server *sv, const std::vector<Request> *pins) {
@@ -534,6 +575,7 @@ int launch_front(iso_server *sv, const std::vector<Request> *pins) {
         launch_serve_cull<false>(kt, v->plan.cull, a, st);
     }
     launch_cache_update(single, v->plan, st);
+    if (!a.single_cull) launch_serve_mask(a, sv->mask_ctas, st);
     serve_front_tail_kernel<<<1, 32, 0, st>>>(a);
     cudaError_t e = cudaEventRecord(sv->front_done[t.parity], st);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -559,18 +601,14 @@ const Plan &back_plan(const iso_server *sv, const Tick &t) {
     return t.reqs.size() == 1 ? sv->one_plan : sv->back_plan;
 }
 
-// On a volume with segment ranges (the largest), a tick's count, scan and
+// On a volume with segment ranges (the largest), a tick's count and
 // emission run one launch per request, each view by value with its own
-// work counters and no stored cases: there a launch over one view is
-// faster per view than one over the table (measured 3.8 against 5.0 ms of
-// count per request of a 10240 x 7680 x 1536 volume), a launch's tail is
-// negligible against its work, and stored cases gain nothing.
+// work counters: there a launch over one view is faster per view than one
+// over the table, and a launch's tail is negligible against its work.
 bool per_view(const iso_server *sv) { return sv->v->seg != nullptr; }
 
 Launch view_launch(const iso_server *sv, const Tick &t, uint32_t j) {
-    VolEntry view = sv->views[t.parity][j];
-    view.s.cases = nullptr;
-    view.s.case_cap = 0;
+    const VolEntry view = sv->views[t.parity][j];
     uint32_t *ctr = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(view.s.ctl) + offsetof(Ctl, ctr));
     return Launch{nullptr, 1u, ctr, view};
 }
@@ -594,14 +632,10 @@ int queue_back(iso_server *sv) {
     if (per_view(sv)) {
         for (uint32_t j = 0; j < k; j++) {
             const Launch L = view_launch(sv, t, j);
-            launch_mc_count(L, false, sv->one_plan, st);
-            launch_mc_scan(L, sv->one_plan, st);
+            launch_mc_scan(L, false, sv->one_plan, st);
         }
     } else {
-        const Launch L = back_launch(sv, t);
-        const Plan &pl = back_plan(sv, t);
-        launch_mc_count(L, false, pl, st);
-        launch_mc_scan(L, pl, st);
+        launch_mc_scan(back_launch(sv, t), false, back_plan(sv, t), st);
     }
     serve_gather_kernel<<<1, 256, 0, st>>>(t.args, sv->d_ctls[t.parity]);
     e = cudaMemcpyAsync(sv->h_ctls[t.parity], sv->d_ctls[t.parity], (k + 1) * sizeof(Ctl), cudaMemcpyDeviceToHost, st);
@@ -694,8 +728,7 @@ int start_emit(iso_server *sv, uint32_t *completed) {
     // one emission per request, its view by value, in order, so a request
     // finishes as soon as its own vertices are written.  Otherwise (a
     // backlog) one emission for all, whose single tail costs less than one
-    // per request.  A view's stored cases are where the front's tail put
-    // them (the same rule, on the host, from the same candidate counts).
+    // per request.
     if (!per_view(sv) && (t.run_to - t.emitted > kEachEmitMax || !sv->queue.empty())) {
         launch_mc_emit(back_launch(sv, t), false, back_plan(sv, t), st);
         for (uint32_t i = t.emitted; i < t.run_to; i++) ISO_CK(cudaEventRecord(sv->emit_done[i], st));
@@ -703,17 +736,8 @@ int start_emit(iso_server *sv, uint32_t *completed) {
         t.stage = kEmit;
         return ISO_OK;
     }
-    uint64_t used = 0;
-    for (uint32_t i = 0; i < k; i++) {
-        VolEntry view = sv->views[t.parity][i];
-        if (k > 1) {
-            const uint64_t n = c[i].n_cand;
-            const bool fits = sv->cases != nullptr && used + n <= sv->case_cap;
-            view.s.cases = fits ? sv->cases + 64ull * used : nullptr;
-            view.s.case_cap = fits ? n : 0ull;
-            if (fits) used += n;
-        }
-        if (i < t.emitted || i >= t.run_to) continue;
+    for (uint32_t i = t.emitted; i < t.run_to; i++) {
+        const VolEntry view = sv->views[t.parity][i];
         if (t.bufs[i]) {
             const Launch L = per_view(sv) ? view_launch(sv, t, i) : Launch{nullptr, 1u, sv->d_ctr[t.parity], view};
             launch_mc_emit(L, false, sv->one_plan, st);
@@ -837,7 +861,7 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
     sv->tri_bytes = o.vertex_format == ISO_VERTEX_PACKED ? 24 : 48;
     const size_t cand = std::min<size_t>(v->cap, v->g.nb);       // candidates of an admitted tick <= cap
     sv->cand_cap = (uint32_t)cand;
-    const size_t n_mc_desc = (cand + kMinMcScanTile - 1) / kMinMcScanTile;
+    const size_t n_mc_desc = (cand + kCountTile - 1) / kCountTile;
     int rc = ISO_OK;
 #define TRY(x)                                   \
     do {                                         \
@@ -863,8 +887,8 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
             Slot &s = sv->slots[p][j];
             TRY(dalloc_on(&s.ctl, 1, sv->device, sv->stream));
             TRY(dalloc_on(&s.icand, cand, sv->device, sv->stream));
-            TRY(dalloc_on(&s.counts, cand, sv->device, sv->stream));
-            TRY(dalloc_on(&s.offsets, cand, sv->device, sv->stream));
+            TRY(dalloc_on(&s.bmask, v->cap, sv->device, sv->stream));
+            TRY(dalloc_on(&s.ooff, cand, sv->device, sv->stream));
             TRY(dalloc_on(&s.desc_cand, v->n_cull_desc, sv->device, sv->stream));
             TRY(dalloc_on(&s.desc_mc, 2 * n_mc_desc, sv->device, sv->stream));
             s.desc_occ = s.desc_mc + n_mc_desc;
@@ -872,15 +896,14 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
             DevState d = v->s;            // the volume's cache and geometry, the request's own lists
             d.ctl = s.ctl;
             d.icand = s.icand;
-            d.counts = s.counts;
-            d.offsets = s.offsets;
+            d.bmask = s.bmask;
+            d.ooff = s.ooff;
+            d.counts = nullptr;           // the debug accessors' arrays are the volume's
+            d.offsets = nullptr;
             d.desc_cand = s.desc_cand;
             d.desc_mc = s.desc_mc;
             d.desc_occ = s.desc_occ;
             d.iocc = s.iocc;
-            d.cases = nullptr;            // set below; a batch launch's per tick by the front
-            d.case_cap = 0;
-            d.cutw = nullptr;
             d.voff = nullptr;
             d.desc_vtx = nullptr;
             d.dbg_edges = nullptr;
@@ -888,22 +911,6 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
         }
     }
     TRY(dalloc_on(&sv->d_params, kMaxServe, sv->device, sv->stream));
-    // Stored cases (the count pass keeps each candidate's 64 cell cases for
-    // the emission, as a volume does): by default for up to max_batch full
-    // candidate lists, at most kMaxTickCaseBytes; without room the emission
-    // classifies again.  A one-request tick's view (by value) holds the whole
-    // buffer, a batch's views their regions (set by the front).
-    {
-        const uint64_t want = o.case_bytes ? o.case_bytes / 64 * 64
-                                           : std::min<uint64_t>(kMaxTickCaseBytes, 64ull * cand * sv->max_batch);
-        if (want && dalloc_on(&sv->cases, want, sv->device, sv->stream) == ISO_OK) sv->case_cap = want / 64;
-        else sv->cases = nullptr;
-        (void)cudaGetLastError();
-        for (int p = 0; p < 2; p++) {
-            sv->views[p][0].s.cases = sv->cases;
-            sv->views[p][0].s.case_cap = sv->case_cap;
-        }
-    }
     if (cudaMallocHost((void **)&sv->h_ctls[0], (kMaxServe + 1) * sizeof(Ctl)) != cudaSuccess ||
         cudaMallocHost((void **)&sv->h_ctls[1], (kMaxServe + 1) * sizeof(Ctl)) != cudaSuccess ||
         cudaMallocHost((void **)&sv->h_params, kMaxServe * sizeof(Params)) != cudaSuccess) {
@@ -929,6 +936,14 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
         return ISO_ERR_CUDA;
     }
 #undef TRY
+    {
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, sv->device) != cudaSuccess) {
+            (void)cudaGetLastError();
+            sms = 1;
+        }
+        sv->mask_ctas = 6 * std::max(1, sms);
+    }
     sv->one_plan = launch_plan(nullptr, sv->device, v->g.nb, cand, 1, true, v->g.rate);
     sv->back_plan = launch_plan(nullptr, sv->device, (uint64_t)v->g.nb * sv->max_batch,
                                 (uint64_t)cand * sv->max_batch, sv->max_batch, false, v->g.rate);
