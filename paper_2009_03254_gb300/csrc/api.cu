@@ -363,7 +363,7 @@ int free_volume(iso_volume *v) {
     DevState &s = v->s;
     void *ptrs[] = {v->bits, v->bmin, v->bmax, v->hull, v->hull8, v->seg, v->tables, s.mactive, s.iactive, s.inew, s.icand,
                     s.islot, s.slast, s.sblock, s.lbuf[0], s.lbuf[1], s.newslot, s.slots, s.desc_cull, s.desc_cand,
-                    s.desc_lru_a, s.desc_lru_b, s.desc_mc, s.ctl, s.ihit, s.bmask, s.counts, s.offsets, s.iocc, s.ooff,
+                    s.desc_lru_a, s.desc_lru_b, s.desc_mc, s.ctl, s.ihit, s.bmask, s.counts, s.offsets, s.iocc, s.ooff, s.ocross,
                     s.cases, s.dbg_edges, s.voff};
     for (void *p : ptrs) dfree_on(p, v->stream);
     cudaStreamSynchronize(v->stream);
@@ -654,6 +654,18 @@ bool build_tables_once(McTables *t) {
     return true;
 }
 
+// the emission's tables, built once per process (null: never expected)
+const EmitTables *emit_tables_once() {
+    static const EmitTables *built = []() -> const EmitTables * {
+        McTables t;
+        static EmitTables e;
+        if (!build_tables_once(&t)) return nullptr;
+        build_emit_tables(t, &e);
+        return &e;
+    }();
+    return built;
+}
+
 }  // namespace
 
 extern "C" {
@@ -800,7 +812,7 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     const bool segments = (o.flags & ISO_SEGMENT_CULL) ||
                           (!(o.flags & ISO_NO_SEGMENT_CULL) && (uint64_t)g.nb >= kSegmentCullMinBlocks);
     if (segments) TRY(dalloc(v, &v->seg, (g.nb + kSegBlocks - 1) / kSegBlocks));
-    TRY(dalloc(v, &v->tables, 256 + 256 * 16));
+    TRY(dalloc(v, &v->tables, 1));
     TRY(dalloc(v, &s.mactive, nwords));
     s.list_cap = std::min<uint32_t>(g.nb, v->cap);
     if (v->flags & ISO_DEBUG) TRY(dalloc(v, &s.iactive, s.list_cap));
@@ -826,6 +838,7 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     TRY(dalloc(v, &s.offsets, v->cap));
     TRY(dalloc(v, &s.iocc, s.list_cap));
     TRY(dalloc(v, &s.ooff, s.list_cap));
+    TRY(dalloc(v, &s.ocross, (size_t)s.list_cap + 3));   // read four at a time
     TRY(dalloc(v, &s.ihit, s.list_cap));
     TRY(dalloc(v, &s.bmask, v->cap));
     if (v->flags & ISO_DEBUG) TRY(dalloc(v, &s.cases, (size_t)s.list_cap * 64));
@@ -845,11 +858,8 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     s.seg = v->seg;
     s.tables = v->tables;
 
-    McTables t;
-    if (!build_tables_once(&t)) { free_volume(v); return ISO_ERR_CUDA; }
-    uint8_t table_bytes[256 + 256 * 16];
-    std::memcpy(table_bytes, t.num_tri, 256);
-    std::memcpy(table_bytes + 256, t.tri_edges, 256 * 16);
+    const EmitTables *emit = emit_tables_once();
+    if (!emit) { free_volume(v); return ISO_ERR_CUDA; }
 
     const cudaMemcpyKind kind = (o.flags & ISO_INPUT_ON_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     cudaStream_t st = v->stream;
@@ -869,7 +879,7 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     const bool async_bits = (o.flags & ISO_ASYNC_UPLOAD) && !on_device;
     if (!async_bits) TRYC(cudaMemcpyAsync(v->bits, compressed, words * 8, kind, st));
 
-    TRYC(cudaMemcpyAsync(v->tables, table_bytes, sizeof(table_bytes), cudaMemcpyHostToDevice, st));
+    TRYC(cudaMemcpyAsync(v->tables, emit, sizeof(*emit), cudaMemcpyHostToDevice, st));
     TRYC(cudaMemsetAsync(s.islot, 0xFF, (size_t)g.nb * 4, st));
     TRYC(cudaMemsetAsync(s.sblock, 0xFF, (size_t)v->cap * 4, st));
     TRYC(cudaMemsetAsync(s.slast, 0, (size_t)v->cap * 4, st));

@@ -237,17 +237,21 @@ __device__ __forceinline__ unsigned long long lookback_exclusive(unsigned long l
 // formed from the samples scaled by 2^-4 or 2^64: the scaling is exact up to
 // underflow of samples far below the difference, the quotient stays the same
 // real number, and the divisor lands inside the reciprocal's range.
-template <bool kExact>
+// kInRange: the caller knows the difference to be inside that range.
+template <bool kExact, bool kInRange = false>
 __device__ __forceinline__ float edge_fraction(float iso, float vlo, float vhi) {
     float a = __fsub_rn(iso, vlo), b = __fsub_rn(vhi, vlo);
     const float mb = fabsf(b);
-    if (!(mb >= 0x1p-100f && mb < 0x1p125f)) {
+    if (!kInRange && !(mb >= 0x1p-100f && mb < 0x1p125f)) {
         const float sc = mb >= 0x1p125f ? 0x1p-4f : 0x1p64f;
         const float slo = __fmul_rn(vlo, sc);
         a = __fsub_rn(__fmul_rn(iso, sc), slo);
         b = __fsub_rn(__fmul_rn(vhi, sc), slo);
     }
-    return kExact ? __fdiv_rn(a, b) : __fdividef(a, b);
+    if (kExact) return __fdiv_rn(a, b);
+    float r;                             // b is normal and its reciprocal too, so this is __fdividef's quotient
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+    return __fmul_rn(a, r);
 }
 
 // ---------------------------------------------------------------- bit tools

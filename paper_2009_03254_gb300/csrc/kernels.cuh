@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "mc_tables.cuh"
 
 namespace bcmc {
 
@@ -32,7 +33,7 @@ struct DevState {
     float *slots;              // decoded blocks, 64 floats per slot
     unsigned long long *desc_cull, *desc_cand, *desc_lru_a, *desc_lru_b, *desc_mc;
     Ctl *ctl;
-    const uint8_t *tables;     // num_tri[256] then tri_edges[256][16]
+    const EmitTables *tables;  // the case table as the emission reads it
     unsigned long long *bmask; // per slot: bit i says sample i of its block is below this extraction's
                                // isovalue (active blocks only; null where nothing counts: a serving
                                // tick of several requests takes each request's masks on its own)
@@ -40,6 +41,7 @@ struct DevState {
     unsigned long long *offsets; // debug access: exclusive prefix of counts (null in a request's view)
     uint32_t *iocc;            // I_occ: ids of the occupied candidates (ascending)
     unsigned long long *ooff;  // first triangle of each occupied candidate
+    unsigned long long *ocross;  // its crossing cells, bit x + 4y + 16z
     unsigned long long *desc_occ;  // look-back descriptors of the occupied count (next to desc_mc)
     unsigned long long *desc_vtx;  // look-back descriptors of the vertex count (next to desc_occ; null
                                    // where indexed meshes are never made)

@@ -17,18 +17,21 @@
 //           the compaction of the occupied candidates, by decoupled
 //           look-backs side by side
 //   emit    Section 4.5, over the occupied candidates only: stage the
-//           samples, classify, per-cell offsets by warp scans, then one
-//           triangle (three vertices) per lane
+//           samples, classify, list the triangles, then one vertex per lane
 //
 // Emit gives each warp 4 consecutive occupied candidates at a time (a "warp
 // tile") and no warp ever waits for another one:
-//   A  slots of each block's 8 blocks of the +group (8 lanes per block)
-//   B  stage the samples in shared memory: 16 float4 rows of the block,
-//      its +x face, +y/+z rows, edges and corner (50 loads per block, 2
-//      per lane, issued two blocks at a time), unpadded: sample
-//      x + 5y + 25z
-//   C  classify: four ballots give the 125 below-iso bits; each cell's
-//      case is 8 bits picked from them; counts from the case table
+//   A  slots of each block's 8 blocks of the +group (8 lanes per block),
+//      loaded two tiles ahead
+//   B  stage the samples in shared memory by asynchronous copies, one tile
+//      ahead, a sample per lane: the 5x5x5 window of each block unpadded
+//      (sample (x, y, z) at x + 5y + 25z)
+//   C  list the crossing cells (the count kept a mask of them), then, one of
+//      them per lane, take their cases from their eight samples and list
+//      their triangles in order
+//   D  write: lane by output vertex, so that every store of the warp is 512
+//      contiguous bytes without passing through shared memory: the vertex's
+//      triangle from the list, its edge from the case table, two samples
 //
 // Over a batch, warp tiles are numbered volume after volume; a warp tile
 // never spans two volumes.
@@ -50,6 +53,8 @@
 #include <algorithm>
 #include <cstdint>
 
+#include <cuda_fp16.h>
+
 #include "common.cuh"
 #include "kernels.cuh"
 #include "launch.cuh"
@@ -60,65 +65,52 @@ namespace bcmc {
 
 namespace {
 
-constexpr int kBPW = 4;                               // candidates per warp tile
-constexpr int kHalo = 128;                            // x + 5y + 25z, x,y,z in [0,5)
-constexpr int kTmap = kBPW * 64 * 5;                  // triangles a warp tile can hold
+constexpr int kBPW = kTileBlocks;                     // blocks per warp tile
+constexpr int kTmap = 256;                            // triangles the list holds (32 cells have at most 160)
+constexpr int kCells = kBPW * 64;                     // crossing cells a tile can have
+constexpr int kVmap = 2 * kTmap + kCells;             // indexed meshes: vertices the same memory holds
 constexpr int kWinWords = 3 * 6 * 4;                  // window rows (indexed meshes), then
 constexpr int kWinTable = kWinWords + 32;             // a per-lane word for blocks inside the volume
+constexpr uint32_t kNoBlock = 0xFFFFFFFFu;
 
-struct WarpTile {                                     // one warp's shared-memory area
-    float halo[kBPW][kHalo];
-    int32_t nslot[kBPW][8];
-    uint32_t bid[kBPW];
-    uint32_t lim[kBPW];                               // cells per axis inside the volume, 4 bits each
-    uint8_t cases[kBPW][64];
+// One warp's shared-memory area: two tiles' samples and lists (one being
+// copied in while the other is used), the crossing cells and the triangle
+// list.
+template <bool kIdx>
+struct EmitWarp {
+    float halo[2][kBPW][kWindow];
+    alignas(16) unsigned long long cross[2][kBPW];    // the blocks' crossing cells
+    unsigned long long first[2][2];                   // the tile's first triangle and first vertex
+    uint32_t bid[2][kBPW];
+    // table row (byte offset) | q << 13 | byte offset of the cell's lower corner in the tile's windows << 16
+    alignas(16) uint32_t tmap[kTmap];
+    uint16_t cells[kCells];                           // crossing cells in order: place of the lower corner | q << 11
+    // indexed: per block, the 12 cut-edge words, then (from word 12) the
+    // vertices of the tile before each word; cells per axis inside the volume
+    uint32_t cut[kIdx ? kBPW : 1][kIdx ? 24 : 2];
+    uint32_t lim[kIdx ? 2 : 1][kIdx ? kBPW : 2];
+};
+
+template <bool kIdx>
+struct EmitTab {                                      // a CTA's copy of what it reads of EmitTables
+    uint16_t info[256];
+    uint16_t corner[kCaseTriangles][4];
+    uint16_t coord[kIdx ? 4 : kBPW * kWindow][4];
 };
 
 template <int kW, bool kIdx>                          // kW warps per CTA
 struct EmitSmem {
-    WarpTile w[kW];
-    float4 stage[kW][kIdx ? 24 : 96];                 // 32 triangles' vertices (indexed: indices) per warp
-    uint16_t tmap[kW][kTmap];                         // block-in-tile (2) | cell (6) | k (3)
-    uint16_t tri_row[256 * kMaxTriPerCell];           // 3 edge numbers of each table triangle, 4 bits each
-    uint8_t num_tri[256];
-    float4 edge_f[12];                                // (dx, dy, dz) and, as bits, the packed edge info
-    // indexed: per block, the 12 cut-edge words, then (from word 12) the
-    // vertices of the tile before each word
-    alignas(16) uint32_t cut[kIdx ? kW : 1][kBPW][24];
-    uint32_t win[kIdx ? kWinTable : 1];               // window rows
+    EmitWarp<kIdx> w[kW];
+    EmitTab<kIdx> tab;
+    uint32_t win[kIdx ? kWinTable : 4];               // window rows
+    // a batch's kMaxBatch + 1 prefix words follow, as many as it has volumes
 };
 
-// Halo load job j of a block (0..63; 50 used): neighbour o, source sample
-// index inside that block, destination sample x + 5y + 25z of the window,
-// a row of 4 samples (one float4 load, four stores) or one sample.
-// Packed: valid(1) | vec(1) | o(3) | src(6) | dst(8).
+// Copy job of window sample j (0..124): the +group member it lies in (3) |
+// its float offset inside that block (6) << 3.
 __device__ __forceinline__ uint32_t halo_job(int j) {
-    int o = 0, src = 0, dst = 0, vec = 0;
-    if (j < 16) {                       // own rows (y, z) = (j & 3, j >> 2)
-        o = 0; src = 4 * j; dst = 5 * (j & 3) + 25 * (j >> 2); vec = 1;
-    } else if (j < 32) {                // +x face: sample (0, y, z) -> halo (4, y, z)
-        const int r = j - 16;
-        o = 1; src = 4 * r; dst = 4 + 5 * (r & 3) + 25 * (r >> 2);
-    } else if (j < 36) {                // +y rows: (x, 0, z) -> (x, 4, z)
-        const int z = j - 32;
-        o = 2; src = 16 * z; dst = 20 + 25 * z; vec = 1;
-    } else if (j < 40) {                // +z rows: (x, y, 0) -> (x, y, 4)
-        const int y = j - 36;
-        o = 4; src = 4 * y; dst = 5 * y + 100; vec = 1;
-    } else if (j < 44) {                // +xy edge: (0, 0, z) -> (4, 4, z)
-        const int z = j - 40;
-        o = 3; src = 16 * z; dst = 24 + 25 * z;
-    } else if (j < 48) {                // +xz edge: (0, y, 0) -> (4, y, 4)
-        const int y = j - 44;
-        o = 5; src = 4 * y; dst = 104 + 5 * y;
-    } else if (j == 48) {               // +yz row: (x, 0, 0) -> (x, 4, 4)
-        o = 6; src = 0; dst = 120; vec = 1;
-    } else if (j == 49) {               // corner: (0, 0, 0) -> (4, 4, 4)
-        o = 7; src = 0; dst = 124;
-    } else {
-        return 0;
-    }
-    return 1u | ((uint32_t)vec << 1) | ((uint32_t)o << 2) | ((uint32_t)src << 5) | ((uint32_t)dst << 11);
+    const int x = j % 5, y = (j / 5) % 5, z = j / 25;
+    return (x >> 2) | ((y >> 2) << 1) | ((z >> 2) << 2) | (uint32_t)(((x & 3) + 4 * (y & 3) + 16 * (z & 3)) << 3);
 }
 
 // cells of a block per axis inside the volume (0 to 4), 4 bits each
@@ -129,40 +121,54 @@ __device__ __forceinline__ uint32_t cell_limits(const Geom &g, uint32_t bx, uint
     return lx | (ly << 4) | (lz << 8);
 }
 
-// Per-lane constants of phases B and C.
+// Per-lane constants.
 struct LaneConst {
-    uint32_t job0, job1;                // halo jobs lane and lane + 32
-    int cls[4];                         // samples lane + 32r (or -1 past the window)
-    // where each of the lane's two cells starts in the 128-bit mask: cell
-    // lane (z 0..1) starts in word 0 or 1, cell lane + 32 (z 2..3) in word
-    // 1 or 2; `up` says the later of the two, `cshift` the bit in it
-    bool up[2];
-    int cshift[2];
+    uint32_t job[4];                    // copy jobs of samples lane + 32r
+    uint32_t cell[2];                   // place of the lower corners of cells lane and lane + 32
     __device__ __forceinline__ void init(int lane) {
-        job0 = halo_job(lane);
-        job1 = halo_job(lane + 32);
 #pragma unroll
-        for (int r = 0; r < 4; r++) cls[r] = lane + 32 * r < 125 ? lane + 32 * r : -1;
+        for (int r = 0; r < 4; r++) job[r] = halo_job(min(lane + 32 * r, kWindow - 1));
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            const int cell = lane + 32 * h, base = (cell & 3) + 5 * ((cell >> 2) & 3) + 25 * (cell >> 4);
-            up[h] = (base >> 5) != h;
-            cshift[h] = base & 31;
+            const int c = lane + 32 * h;
+            cell[h] = (c & 3) + 5 * ((c >> 2) & 3) + 25 * (c >> 4);
         }
     }
 };
 
-// the 8-bit case of a cell from the 32 mask bits starting at its lower corner
-// (corner c at bit (c&1) + 5((c>>1)&1) + 25(c>>2))
-__device__ __forceinline__ uint32_t case_bits(uint32_t W) {
-    return (W & 3u) | ((W >> 3) & 0xCu) | ((W >> 21) & 0x30u) | ((W >> 24) & 0xC0u);
+// 16-byte global -> shared copy that completes asynchronously; `dst` is a
+// shared-window address
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the newest group
+__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__device__ __forceinline__ uint32_t shared_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// 8 and 4 bytes
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(gmem) : "memory");
+}
+// `off` bytes into shared memory at `base`
+template <class T>
+__device__ __forceinline__ const T &at(const void *base, uint32_t off) {
+    return *reinterpret_cast<const T *>(static_cast<const char *>(base) + off);
 }
 
 // the 128-bit below-iso mask of a staged block: bit i of word r says
 // sample s = 32r + i (s = x + 5y + 25z, s < 125) is below the isovalue
-__device__ __forceinline__ void below_mask(const float *hb, const LaneConst &lc, float iso, uint32_t m[4]) {
+__device__ __forceinline__ void below_mask(const float *hb, float iso, uint32_t m[4]) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int r = 0; r < 4; r++) m[r] = __ballot_sync(0xffffffffu, lc.cls[r] >= 0 && hb[lc.cls[r]] < iso);
+    for (int r = 0; r < 4; r++) {
+        const int i = lane + 32 * r;
+        m[r] = __ballot_sync(0xffffffffu, i < kWindow && hb[i] < iso);
+    }
 }
 
 // Window rows: word r of row k of axis a has bit i set when sample
@@ -216,134 +222,10 @@ __device__ __forceinline__ uint32_t lane_cut_word(const uint32_t m[4], uint32_t 
     return (lo ^ far) & w;
 }
 
-// Phases A-C for the warp tile starting at an occupied candidate, nb_w of
-// kBPW blocks used; `b` is this lane's block (block lane/8 of the tile),
-// loaded by the caller one warp tile ahead.  Leaves the cases in wt.cases and
-// returns the per-cell triangle counts of the lane's two cells, packed one
-// byte per block: n0p for cell lane, n1p for cell lane + 32.  With `cut`
-// (indexed meshes), each block's 12 cut-edge words go to cut[q][0..11];
-// `win` is the window-row table in shared memory.
-__device__ __forceinline__ void stage_and_classify(const DevState &s, const Geom &g, float iso, int nb_w, uint32_t b,
-                                                   WarpTile &wt, const LaneConst &lc, const uint8_t *num_tri,
-                                                   uint32_t &n0p, uint32_t &n1p, uint32_t (*cut)[24],
-                                                   const uint32_t *win) {
-    const int lane = threadIdx.x & 31, bq = lane >> 3, bo = lane & 7;
-    const uint32_t slab = g.nbx * g.nby;
-    // ---- A: +group slots
-    if (bq < nb_w) {
-        uint32_t bx, by, bz;
-        block_coords(g, b, bx, by, bz);
-        const bool ex = bx + 1 < g.nbx, ey = by + 1 < g.nby, ez = bz + 1 < g.nbz;
-        const bool exists = (!(bo & 1) || ex) && (!(bo & 2) || ey) && (!(bo & 4) || ez);
-        const uint32_t nbid = b + ((bo & 1) ? 1u : 0u) + ((bo & 2) ? g.nbx : 0u) + ((bo & 4) ? slab : 0u);
-        wt.nslot[bq][bo] = exists && in_bounds(nbid < g.nb, &s.ctl->status) ? s.islot[nbid] : -1;
-        if (bo == 0) {
-            wt.bid[bq] = b;
-            wt.lim[bq] = cell_limits(g, bx, by, bz);
-        }
-    }
-    __syncwarp();
-    // ---- B: stage samples, two blocks at a time (all their loads first,
-    // then all their stores)
-#pragma unroll
-    for (int half = 0; half < 2; half++) {
-        float4 v[kBPW];
-#pragma unroll
-        for (int qq = 0; qq < kBPW / 2; qq++)
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int q = 2 * half + qq;
-                const uint32_t job = h ? lc.job1 : lc.job0;
-                v[2 * qq + h] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (q < nb_w && (job & 1u)) {
-                    const int32_t sl = wt.nslot[q][(job >> 2) & 7u];
-                    if (sl >= 0 && in_bounds((uint32_t)sl < s.ctl->cap, &s.ctl->status)) {
-                        const float *p = s.slots + (size_t)sl * 64 + ((job >> 5) & 63u);
-                        if (job & 2u) v[2 * qq + h] = __ldg(reinterpret_cast<const float4 *>(p));
-                        else v[2 * qq + h].x = __ldg(p);
-                    }
-                }
-            }
-#pragma unroll
-        for (int qq = 0; qq < kBPW / 2; qq++)
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int q = 2 * half + qq;
-                const uint32_t job = h ? lc.job1 : lc.job0;
-                if (q < nb_w && (job & 1u)) {
-                    float *d = &wt.halo[q][0] + (job >> 11);
-                    d[0] = v[2 * qq + h].x;
-                    if (job & 2u) {
-                        d[1] = v[2 * qq + h].y;
-                        d[2] = v[2 * qq + h].z;
-                        d[3] = v[2 * qq + h].w;
-                    }
-                }
-            }
-    }
-    __syncwarp();
-    // ---- C: classify and count
-    n0p = 0;
-    n1p = 0;
-#pragma unroll
-    for (int q = 0; q < kBPW; q++) {
-        if (q >= nb_w) continue;          // warp-uniform
-        uint32_t cs[2], m[4];
-        below_mask(&wt.halo[q][0], lc, iso, m);
-        const uint32_t lim = wt.lim[q];
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const uint32_t lo = lc.up[h] ? m[h + 1] : m[h];
-            const uint32_t hi = lc.up[h] ? m[h + 2] : m[h + 1];
-            cs[h] = case_bits(__funnelshift_r(lo, hi, lc.cshift[h]));
-        }
-        if (lim != 0x444u) {              // warp-uniform: cells past the volume's last sample are empty
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const uint32_t cell = (uint32_t)lane + 32u * h;
-                const bool valid = (cell & 3u) < (lim & 15u) && ((cell >> 2) & 3u) < ((lim >> 4) & 15u) &&
-                                   (cell >> 4) < (lim >> 8);
-                cs[h] = valid ? cs[h] : 0u;
-            }
-        }
-        if (cut) {                        // compile-time: the block's cut edges
-            const uint32_t w = lane_cut_word(m, lim, win);
-            if (lane < 12) cut[q][lane] = w;
-        }
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            wt.cases[q][lane + 32 * h] = (uint8_t)cs[h];
-            const uint32_t n = num_tri[cs[h]];
-            if (h == 0) n0p |= n << (8 * q);
-            else n1p |= n << (8 * q);
-        }
-    }
-}
-
 // candidates the triangle stage visits: none once the cache update failed
 // (both bits are final before the count kernel starts)
 __device__ __forceinline__ uint32_t mc_candidates(const Ctl *c) {
     return (c->status & (kStatusBudget | kStatusTimeout | kStatusTimeoutLru)) ? 0u : c->n_cand;
-}
-
-// A warp tile located in the launch: volume, first occupied candidate,
-// blocks used, and this lane's block (entry first + lane/8), read ahead.
-struct TileRef {
-    uint32_t v, base, nb_w, b;
-};
-
-template <bool kOne>
-__device__ __forceinline__ TileRef locate_tile(const Launch &L, const uint32_t *pre, uint32_t t, uint32_t total) {
-    TileRef r{0u, 0u, 0u, 0u};
-    if (t >= total) return r;
-    r.v = item_vol<kOne>(pre, L.n, t);
-    const DevState &s = vol_of<kOne>(L, r.v).s;
-    const uint32_t n = s.ctl->n_occ;
-    r.base = (t - item_base<kOne>(pre, r.v)) * kBPW;
-    r.nb_w = min((uint32_t)kBPW, n - r.base);
-    const uint32_t i = r.base + ((uint32_t)(threadIdx.x & 31) >> 3);
-    if (i < n) r.b = s.iocc[i];
-    return r;
 }
 
 }  // namespace
@@ -415,6 +297,12 @@ __device__ __forceinline__ unsigned long long valid_cells(uint32_t lim) {
     const uint32_t lx = lim & 15u, ly = (lim >> 4) & 15u, lz = lim >> 8;
     return ((1ull << lx) - 1ull) * 0x1111111111111111ull & (((1ull << (4 * ly)) - 1ull) * 0x0001000100010001ull) &
            (lz >= 4u ? ~0ull : (1ull << (16 * lz)) - 1ull);
+}
+
+__device__ __forceinline__ unsigned long long crossing_cells(const unsigned long long (&m)[8],
+                                                             unsigned long long valid) {
+    return ((m[0] | m[1] | m[2] | m[3] | m[4] | m[5] | m[6] | m[7]) &
+            ~(m[0] & m[1] & m[2] & m[3] & m[4] & m[5] & m[6] & m[7])) & valid;
 }
 
 __device__ __forceinline__ uint32_t count_triangles(const unsigned long long (&m)[8], unsigned long long valid) {
@@ -494,6 +382,7 @@ struct ScanSmem {
     static constexpr int kR = kCountTile / kThreads;
     TileScan<kR> tri, occ, vtx;
     uint32_t val[kR][kThreads];       // triangles (9 bits), vertices (9), triangles before in the warp (14)
+    unsigned long long cross[kR][kThreads];   // crossing cells
 };
 
 template <bool kOne, bool kIdx>
@@ -531,6 +420,7 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
                 corner_masks(s, g, s.icand[i], m, lim);
                 const unsigned long long valid = valid_cells(lim);
                 nt = count_triangles(m, valid);
+                sm.cross[r][threadIdx.x] = crossing_cells(m, valid);
                 if (kIdx) nv = count_vertices(m, valid, lim);
                 if (s.counts) s.counts[i] = nt | (nv << 16);
             }
@@ -587,6 +477,7 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
             if (nt && in_bounds(at < s.list_cap, &c->status)) {
                 s.iocc[at] = s.icand[i];
                 s.ooff[at] = run;
+                s.ocross[at] = sm.cross[r][threadIdx.x];
                 if (kIdx) s.voff[at] = vrun;
             }
         }
@@ -613,29 +504,277 @@ __global__ void __launch_bounds__(kThreads) debug_cases_kernel(Launch L) {
 }
 
 // ================================================================ emit (Section 4.5)
+//
+// What bounds it: instruction issue (57% of slots) and the shared-memory
+// pipe (69% of its wavefronts), beside the vertices' 48 bytes a triangle.
+// Measured on a 384^3 noise surface (4.3 M triangles, 24 warps an SM): 72 us,
+// 45 M warp instructions.  A triangle per lane with its vertices passed
+// through shared memory, on cases found for every cell, took 85 us and
+// 65 M.  Staging rows of 8 floats by 16-byte copies (x of 5 to 7 unused)
+// left bank conflicts: 82 us.  32 warps an SM (64 registers) 79 us and a
+// larger shared-memory share of the L1 79 us: the L1 serves the windows'
+// shared rows, so the warps' areas are kept small.
+
+// The warp tiles of one launch, as a lane of a warp sees them
+template <bool kOne>
+struct TileWalk {
+    const Launch &L;
+    const uint32_t *pre;
+    uint32_t total;
+
+    // volume, first occupied candidate and blocks of tile t < total
+    __device__ __forceinline__ void locate(uint32_t t, uint32_t &v, uint32_t &base, uint32_t &nb_w) const {
+        v = item_vol<kOne>(pre, L.n, t);
+        base = (t - item_base<kOne>(pre, v)) * kBPW;
+        nb_w = min((uint32_t)kBPW, vol_of<kOne>(L, v).s.ctl->n_occ - base);
+    }
+    // this lane's block of tile t (block lane / 8 of the tile)
+    __device__ __forceinline__ uint32_t block_at(uint32_t t) const {
+        if (t >= total) return kNoBlock;
+        uint32_t v, base, nb_w;
+        locate(t, v, base, nb_w);
+        const uint32_t q = (threadIdx.x & 31) >> 3;
+        return q < nb_w ? vol_of<kOne>(L, v).s.iocc[base + q] : kNoBlock;
+    }
+    // The slot of member lane % 8 of block b's +group (-1: none).  Where the
+    // volume ends the ids run on into the next row: cells that read such a
+    // block are outside the volume and never cross, so any slot will do.
+    __device__ __forceinline__ int32_t slot_at(uint32_t t, uint32_t b) const {
+        if (b == kNoBlock) return -1;
+        const uint32_t v = item_vol<kOne>(pre, L.n, t), o = threadIdx.x & 7;
+        const DevState &s = vol_of<kOne>(L, v).s;
+        const Geom &g = vol_of<kOne>(L, v).g;
+        const unsigned long long id = (unsigned long long)b + ((o & 1) ? 1u : 0u) + ((o & 2) ? g.nbx : 0u) +
+                                      ((o & 4) ? g.nbx * g.nby : 0u);
+        if (id >= g.nb) return -1;
+        const int32_t sl = s.islot[id];
+        return sl >= 0 && in_bounds((uint32_t)sl < s.ctl->cap, &s.ctl->status) ? sl : -1;
+    }
+};
+
+// Phase B: queue the copies of a tile's samples and lists and write down its
+// blocks (this lane's block b and slot from the two functions above)
+template <bool kOne, bool kIdx>
+__device__ __forceinline__ void stage_tile(const TileWalk<kOne> &walk, uint32_t t, uint32_t b, int32_t slot, int buf,
+                                           EmitWarp<kIdx> &wt, const LaneConst &lc) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t v = item_vol<kOne>(walk.pre, walk.L.n, t);
+    const DevState &s = vol_of<kOne>(walk.L, v).s;
+    const uint32_t base = (t - item_base<kOne>(walk.pre, v)) * kBPW;
+    const uint32_t halo = shared_u32(&wt.halo[buf][0][0]);
+    if ((lane & 7) == 0) {
+        const uint32_t q = lane >> 3;
+        wt.bid[buf][q] = b;
+        if (kIdx && b != kNoBlock) {
+            const Geom &g = vol_of<kOne>(walk.L, v).g;
+            uint32_t bx, by, bz;
+            block_coords(g, b, bx, by, bz);
+            wt.lim[kIdx ? buf : 0][q] = cell_limits(g, bx, by, bz);
+        }
+    }
+    if (lane < 2) cp_async16(shared_u32(&wt.cross[buf][2 * lane]), s.ocross + base + 2 * lane);
+    if (lane == 2) cp_async8(shared_u32(&wt.first[buf][0]), s.ooff + base);
+    if (kIdx && lane == 3) cp_async8(shared_u32(&wt.first[buf][1]), s.voff + base);
+    const uint32_t dst = halo + 4 * lane;
+#pragma unroll
+    for (int q = 0; q < kBPW; q++)
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            const int32_t sl = __shfl_sync(0xffffffffu, slot, 8 * q + (lc.job[r] & 7u));
+            if (sl >= 0 && (r < 3 || lane < kWindow - 96))
+                cp_async4(dst + 4 * (q * kWindow + 32 * r), s.slots + (size_t)(uint32_t)sl * 64 + (lc.job[r] >> 3));
+        }
+}
+
+// Phase D: the vertices of the `n` listed triangles, the first of them
+// triangle t0 of the surface.  Lane l of round r writes vertex 32r + l of a
+// chunk of 32 triangles, i.e. corner (32r + l) % 3 of triangle (32r + l) / 3.
+// With kSafe every difference of two samples is in the reciprocal's range (the
+// caller looked at the samples).  Vertices are stored evict-first (a surface
+// is several times the L2, and the hulls, slot map and cached blocks the
+// next extraction reads should stay there).
+template <bool kPacked, bool kSafe, bool kDebug, bool kIdx>
+__device__ __forceinline__ void write_soup(const DevState &s, const Geom &g, float iso, const EmitWarp<kIdx> &wt,
+                                           const EmitTab<kIdx> &tab, int buf, uint32_t n, unsigned long long t0) {
+    const uint32_t lane = threadIdx.x & 31;
+    const Ctl *c = s.ctl;
+    const unsigned long long cap = c->params.tri_cap;
+    // vertices of the list that fit the output
+    const int fit = t0 >= cap ? 0 : 3 * (int)min((unsigned long long)n, cap - t0);
+    float4 *out4 = reinterpret_cast<float4 *>(c->params.out) + 3 * t0 + lane;
+    uint2 *out2 = reinterpret_cast<uint2 *>(c->params.out) + 3 * t0 + lane;
+    const uint32_t last = 4 * (n - 1);
+    uint32_t tri[3];                                       // byte offsets in the list
+#pragma unroll
+    for (int r = 0; r < 3; r++) tri[r] = 4 * ((32 * r + lane) / 3);
+    for (int left = fit - (int)lane; left > -(int)lane; left -= 96) {
+#pragma unroll
+        for (int r = 0; r < 3; r++) {
+            const uint32_t e = at<uint32_t>(wt.tmap, min(tri[r], last));
+            const uint32_t info = at<uint16_t>(tab.corner, (e & 0x1FFFu) | (2 * ((32 * r + lane) % 3)));
+            const uint32_t bid = wt.bid[buf][(e >> 13) & 3u];
+            const uint32_t smp = (e >> 16) + (info & 0xFFu), step = info >> 8;   // byte offsets
+            const float vlo = at<float>(wt.halo[buf], smp), vhi = at<float>(wt.halo[buf], smp + step);
+            const uint2 h = at<uint2>(tab.coord, 2 * smp);
+            const float2 xy = __half22float2(*reinterpret_cast<const __half2 *>(&h.x));
+            float px = xy.x, py = xy.y, pz = __low2float(*reinterpret_cast<const __half2 *>(&h.y));
+            const float tt = edge_fraction<kPacked, kSafe>(iso, vlo, vhi);
+            if (step == 4u) px = __fadd_rn(px, tt);
+            if (step == 20u) py = __fadd_rn(py, tt);
+            if (step == 100u) pz = __fadd_rn(pz, tt);
+            const bool write = left > 32 * r;
+            if (!kPacked) {
+                if (write) __stcs(out4 + 32 * r, make_float4(px, py, pz, __uint_as_float(bid)));
+            } else {
+                // the 10-bit code round(p / 4 * 1023) decides an integer, so every
+                // step is one IEEE float32 operation (the division correctly
+                // rounded), as the oracle computes it
+                const uint32_t qx = (uint32_t)__float2int_rn(__fmul_rn(px, 255.75f));
+                const uint32_t qy = (uint32_t)__float2int_rn(__fmul_rn(py, 255.75f));
+                const uint32_t qz = (uint32_t)__float2int_rn(__fmul_rn(pz, 255.75f));
+                if (write) __stcs(out2 + 32 * r, make_uint2(qx | (qy << 10) | (qz << 20), bid));
+            }
+            if (kDebug) {
+                uint32_t bx, by, bz;
+                block_coords(g, bid, bx, by, bz);
+                const uint32_t i = smp / 4 % kWindow, a = step == 4u ? 0u : (step == 20u ? 1u : 2u);
+                const unsigned long long x = 4ull * bx + i % 5u, y = 4ull * by + (i / 5u) % 5u, z = 4ull * bz + i / 25u;
+                if (write)
+                    s.dbg_edges[3 * t0 + (unsigned)(fit - left) + 32 * r] =
+                        3ull * (x + (unsigned long long)g.nx * (y + (unsigned long long)g.ny * z)) + a;
+            }
+            tri[r] += 128;
+        }
+        out4 += 96;
+        out2 += 96;
+    }
+}
+
+// Phase D of an indexed mesh: the three vertex indices of each listed
+// triangle, `vt` that of the tile's first vertex; lanes as above.  A corner's
+// index is the rank of its edge among the tile's vertices: those before its
+// cut-edge word, then the word's bits below it.
+template <bool kDebug>
+__device__ __forceinline__ void write_indices(const DevState &s, const Geom &g, const EmitWarp<true> &wt,
+                                              const EmitTab<true> &tab, int buf, uint32_t n, unsigned long long t0,
+                                              unsigned long long vt) {
+    const int lane = threadIdx.x & 31;
+    const Ctl *c = s.ctl;
+    const unsigned long long cap = c->params.tri_cap;
+    const uint32_t fit = t0 >= cap ? 0u : (uint32_t)min((unsigned long long)n, cap - t0);
+    uint32_t *out = reinterpret_cast<uint32_t *>(c->params.idx_out) + 3 * t0 + lane;
+    for (uint32_t c0 = 0; c0 < n; c0 += 32) {
+#pragma unroll
+        for (int r = 0; r < 3; r++) {
+            const uint32_t f = 32 * r + lane, tri = min(c0 + f / 3u, n - 1), e = wt.tmap[tri];
+            const uint32_t info = at<uint16_t>(tab.corner, (e & 0x1FFFu) | (2 * (f % 3u)));
+            const uint32_t q = (e >> 13) & 3u, step = info >> 8, a = step == 4u ? 0u : (step == 20u ? 1u : 2u);
+            const uint32_t smp = (e >> 18) - q * kWindow + ((info & 0xFFu) >> 2);
+            const uint32_t *cw = wt.cut[q] + 4 * a + (smp >> 5);
+            const uint32_t rank = cw[12] + __popc(cw[0] & ((1u << (smp & 31)) - 1u));
+            const bool write = 3 * c0 + f < 3 * fit;
+            if (write) out[32 * r] = (uint32_t)(vt + rank);
+            if (kDebug) {
+                uint32_t bx, by, bz;
+                block_coords(g, wt.bid[buf][q], bx, by, bz);
+                const unsigned long long x = 4ull * bx + smp % 5u, y = 4ull * by + (smp / 5u) % 5u, z = 4ull * bz + smp / 25u;
+                if (write)
+                    s.dbg_edges[3 * (t0 + c0) + f] =
+                        3ull * (x + (unsigned long long)g.nx * (y + (unsigned long long)g.ny * z)) + a;
+            }
+        }
+        out += 96;
+    }
+}
+
+// The vertices of an indexed tile, in order (block, axis, sample).  Lanes
+// 0-11 (and 12-23 for a second block) take one word each of a block's cut
+// edges, leave the vertices of the tile before it in cut[q][12..23], and list
+// its edges in the vertex map; then one vertex per lane, the triangle soup's
+// arithmetic, consecutive lanes writing consecutive vertices.  The map holds
+// two blocks (at most 600 vertices); it is written out when full.
+__device__ __forceinline__ void write_vertices(const DevState &s, float iso, EmitWarp<true> &wt, int buf, int nb_w,
+                                               unsigned long long vt) {
+    const int lane = threadIdx.x & 31;
+    const Ctl *c = s.ctl;
+    const bool packed = c->params.format == kVertexPacked;     // warp-uniform
+    const unsigned long long vcap = c->params.vert_cap;
+    float4 *out = reinterpret_cast<float4 *>(c->params.out);
+    uint16_t *vm = reinterpret_cast<uint16_t *>(wt.tmap);      // block (2) | sample (7) | axis (2)
+    uint32_t nvt = 0, first = 0;                               // vertices so far; the map's first one
+    for (int qq = 0; qq < nb_w; qq += 2) {
+        const int q = qq + (lane >= 12 ? 1 : 0), lk = lane % 12, la = lk >> 2, lr = lk & 3;
+        uint32_t w = (lane < 24 && q < nb_w) ? wt.cut[q][lk] : 0u;
+        const uint32_t n = __popc(w);
+        uint32_t incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+        uint32_t rank = nvt + incl - n;                        // the tile's vertices before this word
+        if (lane < 24 && q < nb_w) wt.cut[q][12 + lk] = rank;
+        // listed now, or after what the map holds has been written
+        for (int pass = 0; pass < 2; pass++) {
+            const bool room = nvt - first + tot <= (uint32_t)kVmap;
+            if (room) {
+                while (w) {
+                    const uint32_t i = __ffs(w) - 1;
+                    w &= w - 1;
+                    vm[rank++ - first] = (uint16_t)((q << 9) | ((32 * lr + i) << 2) | la);
+                }
+            }
+            __syncwarp();
+            if (room && qq + 2 < nb_w) break;                  // go on listing
+            const uint32_t to = room ? nvt + tot : nvt;
+            for (uint32_t k = first + lane; k < to; k += 32) {
+                const uint32_t e = vm[k - first], q2 = e >> 9, smp = (e >> 2) & 127u, ax = e & 3u;
+                const uint32_t sx = smp % 5u, sy = (smp / 5u) % 5u, sz = smp / 25u;
+                const float *hp = &wt.halo[buf][q2][smp];
+                const float vlo = hp[0], vhi = hp[ax == 0 ? 1 : (ax == 1 ? 5 : 25)];
+                float px = (float)sx, py = (float)sy, pz = (float)sz;
+                const float tt = packed ? edge_fraction<true>(iso, vlo, vhi) : edge_fraction<false>(iso, vlo, vhi);
+                if (ax == 0) px = __fadd_rn(px, tt);
+                else if (ax == 1) py = __fadd_rn(py, tt);
+                else pz = __fadd_rn(pz, tt);
+                if (vt + k < vcap) {
+                    const uint32_t bid = wt.bid[buf][q2];
+                    if (!packed) {
+                        out[vt + k] = make_float4(px, py, pz, __uint_as_float(bid));
+                    } else {
+                        const uint32_t qx = (uint32_t)__float2int_rn(__fmul_rn(px, 255.75f));
+                        const uint32_t qy = (uint32_t)__float2int_rn(__fmul_rn(py, 255.75f));
+                        const uint32_t qz = (uint32_t)__float2int_rn(__fmul_rn(pz, 255.75f));
+                        reinterpret_cast<uint2 *>(out)[vt + k] = make_uint2(qx | (qy << 10) | (qz << 20), bid);
+                    }
+                }
+            }
+            first = to;
+            __syncwarp();                                      // the map is read
+            if (room) break;
+        }
+        nvt += tot;
+    }
+}
 
 template <int kW, bool kDebug, bool kOne, bool kIdx>
 __device__ __forceinline__ void emit_body(const Launch &L) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     EmitSmem<kW, kIdx> &sm = *reinterpret_cast<EmitSmem<kW, kIdx> *>(smem_raw);
-    __shared__ uint32_t pre[kMaxBatch + 1];
+    uint32_t *pre = reinterpret_cast<uint32_t *>(&sm + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint8_t *tables = vol_of<kOne>(L, 0).s.tables;
-    for (int i = threadIdx.x; i < 256; i += 32 * kW) sm.num_tri[i] = tables[i];
-    for (int i = threadIdx.x; i < 256 * kMaxTriPerCell; i += 32 * kW) {
-        const uint8_t *e = tables + 256 + (i / kMaxTriPerCell) * 16 + 3 * (i % kMaxTriPerCell);
-        sm.tri_row[i] = (uint16_t)(e[0] | (e[1] << 4) | (e[2] << 8));
-    }
+    const EmitTables *tables = vol_of<kOne>(L, 0).s.tables;
+    auto fill = [&](void *dst, const void *src, uint32_t bytes) {
+        for (uint32_t i = threadIdx.x; i < bytes / 16; i += 32 * kW)
+            static_cast<uint4 *>(dst)[i] = __ldg(static_cast<const uint4 *>(src) + i);
+    };
+    static_assert(sizeof(EmitWarp<kIdx>) % 16 == 0 && sizeof(tables->info) % 16 == 0 &&
+                      sizeof(tables->corner) % 16 == 0 && sizeof(tables->coord) % 16 == 0, "16-byte copies");
+    fill(sm.tab.info, tables->info, sizeof(tables->info));
+    fill(sm.tab.corner, tables->corner, sizeof(tables->corner));
+    if (!kIdx) fill(sm.tab.coord, tables->coord, sizeof(tables->coord));
     if (kIdx) load_window_rows(sm.win);
-    if (threadIdx.x < 12) {
-        // edge e: lower corner (dx,dy,dz), axis a; halo offsets of its two samples
-        const int e = threadIdx.x, a = e >> 2, j0 = e & 1, j1 = (e >> 1) & 1;
-        const int dx = a == 0 ? 0 : j0, dy = a == 0 ? j0 : (a == 1 ? 0 : j1), dz = a == 2 ? 0 : j1;
-        const int lo = dx + 5 * dy + 25 * dz, hi = lo + (a == 0 ? 1 : (a == 1 ? 5 : 25));
-        sm.edge_f[e] = make_float4((float)dx, (float)dy, (float)dz,
-                                   __uint_as_float((uint32_t)lo | ((uint32_t)hi << 8) | ((uint32_t)dx << 16) |
-                                                   ((uint32_t)dy << 17) | ((uint32_t)dz << 18) | ((uint32_t)a << 19)));
-    }
     // all failure bits are final before this kernel starts
     const uint32_t total = launch_prefix<kOne>(
         L, [&](uint32_t v) {
@@ -646,238 +785,136 @@ __device__ __forceinline__ void emit_body(const Launch &L) {
     __syncthreads();                                      // the tables
     LaneConst lc;
     lc.init(lane);
-    WarpTile &wt = sm.w[warp];
-    uint16_t *tm = sm.tmap[warp];
-    float4 *stage = sm.stage[warp];
+    EmitWarp<kIdx> &wt = sm.w[warp];
+    const TileWalk<kOne> walk{L, pre, total};
     const uint32_t stride = gridDim.x * kW;
     uint32_t t = blockIdx.x * kW + warp;
-    TileRef nxt = locate_tile<kOne>(L, pre, t, total);
-    for (; t < total; t += stride) {
-        const TileRef cur = nxt;
-        nxt = locate_tile<kOne>(L, pre, t + stride, total);   // next warp tile's blocks, loaded early
-        const DevState &s = vol_of<kOne>(L, cur.v).s;
-        const Geom &g = vol_of<kOne>(L, cur.v).g;
+    if (t >= total) return;
+    // one tile's samples are copied in while the tile before it is written;
+    // its slots were loaded a tile earlier, and its block ids two
+    uint32_t b1, b2;
+    int32_t s1;
+    {
+        const uint32_t b0 = walk.block_at(t);
+        b1 = walk.block_at(t + stride);
+        b2 = walk.block_at(t + 2 * stride);
+        const int32_t s0 = walk.slot_at(t, b0);
+        s1 = walk.slot_at(t + stride, b1);
+        stage_tile<kOne, kIdx>(walk, t, b0, s0, 0, wt, lc);
+        cp_async_commit();
+    }
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int buf = 0; t < total; t += stride, buf ^= 1) {
+        if (t + stride < total) stage_tile<kOne, kIdx>(walk, t + stride, b1, s1, buf ^ 1, wt, lc);
+        cp_async_commit();
+        s1 = walk.slot_at(t + 2 * stride, b2);
+        b1 = b2;
+        b2 = walk.block_at(t + 3 * stride);
+        uint32_t v, base, nb_w;
+        walk.locate(t, v, base, nb_w);
+        const DevState &s = vol_of<kOne>(L, v).s;
+        const Geom &g = vol_of<kOne>(L, v).g;
         const Ctl *c = s.ctl;
         const float iso = c->params.iso;
-        const unsigned long long tri_cap = c->params.tri_cap;
         const bool packed = c->params.format == kVertexPacked;     // warp-uniform
-        float4 *__restrict__ out = reinterpret_cast<float4 *>(c->params.out);
-        const uint32_t base = cur.base;
-        const int nb_w = (int)cur.nb_w;
-        uint32_t n0p, n1p;
-        stage_and_classify(s, g, iso, nb_w, cur.b, wt, lc, sm.num_tri, n0p, n1p, kIdx ? sm.cut[warp] : nullptr,
-                           sm.win);
-        // per-cell offsets inside the warp tile: two packed scans (byte q = block q)
-        uint32_t i0 = n0p, i1 = n1p;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t a0 = __shfl_up_sync(0xffffffffu, i0, o), a1 = __shfl_up_sync(0xffffffffu, i1, o);
-            if (lane >= o) { i0 += a0; i1 += a1; }
-        }
-        const uint32_t s0 = __shfl_sync(0xffffffffu, i0, 31), s1 = __shfl_sync(0xffffffffu, i1, 31);
-        uint32_t wtot = 0;
-#pragma unroll
-        for (int q = 0; q < kBPW; q++)
-            if (q < nb_w) wtot += ((s0 >> (8 * q)) & 0xFFu) + ((s1 >> (8 * q)) & 0xFFu);
-        if (wtot == 0) continue;                       // warp-uniform
-        // consecutive occupied candidates have adjacent outputs: the tile starts
-        // at its first block's
-        const unsigned long long gbase = s.ooff[base];
-        unsigned long long vt = 0;                     // indexed: the tile's first vertex
+        // subtracting -0 instead of 0 leaves a sample of -0 at +0, not below
+        const float iso_sub = iso == 0.0f ? -0.0f : iso;
+        cp_async_wait_prev();
+        __syncwarp();
+        // consecutive occupied candidates have adjacent outputs: the tile
+        // starts at its first block's
+        unsigned long long t0 = wt.first[buf][0], vt = 0;
         if constexpr (kIdx) {
-            // Per block, lanes 0-11 take one word each of its cut edges and the
-            // vertices of the tile before it (an exclusive scan over the lanes,
-            // in vertex order: axis, then sample), and list the word's edges
-            // in the vertex map `tm` at their ranks.
-            vt = s.voff[base];
-            __syncwarp();                              // the words
-            uint32_t nvt = 0;
-            const int lk = lane % 12, la = lk >> 2, lr = lk & 3;
-            for (int qq = 0; qq < nb_w; qq += 2) {     // lanes 0-11: block qq, lanes 12-23: block qq + 1
-                const int q = qq + (lane >= 12 ? 1 : 0);
-                uint32_t w = (lane < 24 && q < nb_w) ? sm.cut[warp][q][lk] : 0u;
-                const uint32_t n = __popc(w);
-                uint32_t incl = n;
+            vt = wt.first[buf][1];
+            for (uint32_t q = 0; q < nb_w; q++) {
+                uint32_t m[4];
+                below_mask(&wt.halo[buf][q][0], iso, m);
+                const uint32_t w = lane_cut_word(m, wt.lim[buf][q], sm.win);
+                if (lane < 12) wt.cut[q][lane] = w;
+            }
+            __syncwarp();
+            write_vertices(s, iso, wt, buf, (int)nb_w, vt);
+            vt += c->params.vtx_base;                  // indices count the vertices of earlier waves
+        }
+        // ---- C: the crossing cells in order
+        uint32_t ncell = 0;
+#pragma unroll
+        for (int q = 0; q < kBPW; q++) {
+            const unsigned long long w2 = q < (int)nb_w ? wt.cross[buf][q] : 0ull;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const uint32_t w = h ? (uint32_t)(w2 >> 32) : (uint32_t)w2;
+                if ((w >> lane) & 1u) wt.cells[ncell + __popc(w & lt)] = (uint16_t)((lc.cell[h] + q * kWindow) | (q << 11));
+                ncell += __popc(w);
+            }
+        }
+        __syncwarp();
+        // 32 cells at a time: their triangles while they fit the list, then D
+        uint32_t n = 0, k0 = 0;
+        bool safe = true;
+        for (;;) {
+            for (; k0 < ncell; k0 += 32) {
+                const uint32_t cell = wt.cells[min(k0 + lane, ncell - 1)];
+                const float *hb = &wt.halo[buf][0][0] + (cell & 0x7FFu);
+                float d[8];
+                float mx = 0.0f, mn = INFINITY;
+                uint32_t cs = 0;
+#pragma unroll
+                for (int k = 7; k >= 0; k--) {
+                    d[k] = __fsub_rn(hb[(k & 1) + 5 * ((k >> 1) & 1) + 25 * (k >> 2)], iso_sub);
+                    cs = __funnelshift_l(__float_as_uint(d[k]), cs, 1);      // below: the difference's sign
+                    mx = fmaxf(mx, fabsf(d[k]));
+                    mn = fminf(mn, fabsf(d[k]));
+                }
+                const uint32_t row = sm.tab.info[cs];
+                const uint32_t k = k0 + lane < ncell ? row >> 13 : 0u;
+                uint32_t incl = k;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
                     if (lane >= o) incl += x;
                 }
-                uint32_t rank = nvt + incl - n;        // the tile's vertices before this word
-                if (lane < 24 && q < nb_w) sm.cut[warp][q][12 + lk] = rank;
-                while (w) {                            // this word's edges: (block, sample, axis)
-                    const uint32_t i = __ffs(w) - 1;
-                    w &= w - 1;
-                    tm[rank++] = (uint16_t)((q << 9) | ((32 * lr + i) << 2) | la);
-                }
-                nvt += __shfl_sync(0xffffffffu, incl, 23);
+                const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+                if (n + tot > (uint32_t)kTmap) break;
+                // the two samples of a cut edge lie on either side of iso, each
+                // between 2^-100 and 2^124 away: their difference is in range
+                safe = safe && __all_sync(0xffffffffu, mn >= 0x1p-100f && mx < 0x1p124f);
+                uint32_t *to = wt.tmap + n + incl - k;
+                const uint32_t e = ((cell & 0x7FFu) << 18) | ((cell >> 11) << 13) | (row & 0x1FFFu);
+                if (k > 0) to[0] = e;
+                if (k > 1) to[1] = e + 8;
+                if (k > 2) to[2] = e + 16;
+                if (k > 3) to[3] = e + 24;
+                if (k > 4) to[4] = e + 32;
+                n += tot;
             }
             __syncwarp();
-            // one vertex per lane, the triangle soup's arithmetic; consecutive
-            // lanes write consecutive vertices
-            const unsigned long long vcap = c->params.vert_cap;
-            for (uint32_t k = lane; k < nvt; k += 32) {
-                const uint32_t e = tm[k];
-                const uint32_t q = e >> 9, smp = (e >> 2) & 127u, ax = e & 3u;
-                const uint32_t sx = smp % 5u, sy = (smp / 5u) % 5u, sz = smp / 25u;
-                const float *hp = &wt.halo[q][0] + smp;
-                const float vlo = hp[0], vhi = hp[ax == 0 ? 1 : (ax == 1 ? 5 : 25)];
-                float px = (float)sx, py = (float)sy, pz = (float)sz;
-                float tt;
-                if (!packed) tt = edge_fraction<false>(iso, vlo, vhi);
-                else tt = edge_fraction<true>(iso, vlo, vhi);
-                if (ax == 0) px = __fadd_rn(px, tt);
-                else if (ax == 1) py = __fadd_rn(py, tt);
-                else pz = __fadd_rn(pz, tt);
-                if (vt + k < vcap) {
-                    if (!packed) {
-                        out[vt + k] = make_float4(px, py, pz, __uint_as_float(wt.bid[q]));
-                    } else {
-                        const uint32_t qx = (uint32_t)__float2int_rn(__fmul_rn(px, 255.75f));
-                        const uint32_t qy = (uint32_t)__float2int_rn(__fmul_rn(py, 255.75f));
-                        const uint32_t qz = (uint32_t)__float2int_rn(__fmul_rn(pz, 255.75f));
-                        reinterpret_cast<uint2 *>(out)[vt + k] = make_uint2(qx | (qy << 10) | (qz << 20), wt.bid[q]);
-                    }
-                }
+            if (n) {                              // warp-uniform
+                if constexpr (kIdx) write_indices<kDebug>(s, g, wt, sm.tab, buf, n, t0, vt);
+                else if (packed) write_soup<true, false, kDebug, kIdx>(s, g, iso, wt, sm.tab, buf, n, t0);
+                else if (safe) write_soup<false, true, kDebug, kIdx>(s, g, iso, wt, sm.tab, buf, n, t0);
+                else write_soup<false, false, kDebug, kIdx>(s, g, iso, wt, sm.tab, buf, n, t0);
             }
-            vt += c->params.vtx_base;                  // indices count the vertices of earlier waves
-            __syncwarp();                              // the vertex map is read: tm takes the triangles
-        }
-        // each lane lists its two cells' triangles at their offsets (unrolled,
-        // predicated stores: the counts differ from lane to lane)
-        uint32_t tacc = 0;
-#pragma unroll 1
-        for (int q = 0; q < nb_w; q++) {
-            const uint32_t n0 = (n0p >> (8 * q)) & 0xFFu, n1 = (n1p >> (8 * q)) & 0xFFu;
-            const uint32_t b0 = (s0 >> (8 * q)) & 0xFFu;
-            const uint32_t o0 = tacc + ((i0 >> (8 * q)) & 0xFFu) - n0;
-            const uint32_t o1 = tacc + b0 + ((i1 >> (8 * q)) & 0xFFu) - n1;
-#pragma unroll
-            for (uint32_t k = 0; k < kMaxTriPerCell; k++) {
-                if (k < n0) tm[o0 + k] = (uint16_t)((q << 9) | (lane << 3) | k);
-                if (k < n1) tm[o1 + k] = (uint16_t)((q << 9) | ((lane + 32) << 3) | k);
-            }
-            tacc += b0 + ((s1 >> (8 * q)) & 0xFFu);
-        }
-        __syncwarp();
-        // one triangle per lane; its three vertices (or, indexed, its three
-        // vertex indices) go through the warp's staging area so that each
-        // store instruction writes contiguous bytes; vertices are stored evict-first
-        // (a surface is several times the L2, and the hulls, slot map and
-        // cached blocks the next extraction reads should stay there)
-        for (uint32_t t0 = 0; t0 < wtot; t0 += 32) {
-            const uint32_t tri = t0 + lane;
-            if (tri < wtot) {
-                const uint32_t e16 = tm[tri];
-                const uint32_t q = e16 >> 9, cell = (e16 >> 3) & 63u, k = e16 & 7u;
-                const uint32_t row = sm.tri_row[wt.cases[q][cell] * kMaxTriPerCell + k];
-                const int cx = (int)(cell & 3u), cy = (int)((cell >> 2) & 3u), cz = (int)(cell >> 4);
-                const float *hb = &wt.halo[q][0] + cx + 5 * cy + 25 * cz;
-                const float wbits = __uint_as_float(wt.bid[q]);
-                const float fx = (float)cx, fy = (float)cy, fz = (float)cz;
-#pragma unroll
-                for (int j = 0; j < 3; j++) {
-                    const float4 ef = sm.edge_f[(row >> (4 * j)) & 0xFu];
-                    const uint32_t info = __float_as_uint(ef.w);
-                    const uint32_t a = (info >> 19) & 3u;
-                    if constexpr (kIdx) {
-                        // the rank of the edge among the tile's vertices: those
-                        // before its word, then its word's bits below it
-                        const int smp = cx + (int)((info >> 16) & 1u) + 5 * (cy + (int)((info >> 17) & 1u)) +
-                                        25 * (cz + (int)((info >> 18) & 1u));
-                        const uint32_t *cw = sm.cut[warp][q] + 4 * a + (smp >> 5);
-                        const uint32_t rank = cw[12] + __popc(cw[0] & ((1u << (smp & 31)) - 1u));
-                        reinterpret_cast<uint32_t *>(stage)[3 * lane + j] = (uint32_t)(vt + rank);
-                    } else {
-                        const float vlo = hb[info & 0xFFu], vhi = hb[(info >> 8) & 0xFFu];
-                        float4 p = make_float4(__fadd_rn(fx, ef.x), __fadd_rn(fy, ef.y), __fadd_rn(fz, ef.z), wbits);
-                        if (!packed) {
-                            // t through the reciprocal: within 2 ulp of the correctly
-                            // rounded quotient (positions within 1e-6)
-                            const float tt = edge_fraction<false>(iso, vlo, vhi);
-                            if (a == 0) p.x = __fadd_rn(p.x, tt);
-                            else if (a == 1) p.y = __fadd_rn(p.y, tt);
-                            else p.z = __fadd_rn(p.z, tt);
-                            stage[3 * lane + j] = p;
-                        } else {
-                            // the 10-bit code round(p / 4 * 1023) decides an integer, so every
-                            // step is one IEEE float32 operation (the division correctly
-                            // rounded), as the oracle computes it
-                            const float tt = edge_fraction<true>(iso, vlo, vhi);
-                            if (a == 0) p.x = __fadd_rn(p.x, tt);
-                            else if (a == 1) p.y = __fadd_rn(p.y, tt);
-                            else p.z = __fadd_rn(p.z, tt);
-                            const uint32_t qx = (uint32_t)__float2int_rn(__fmul_rn(p.x, 255.75f));
-                            const uint32_t qy = (uint32_t)__float2int_rn(__fmul_rn(p.y, 255.75f));
-                            const uint32_t qz = (uint32_t)__float2int_rn(__fmul_rn(p.z, 255.75f));
-                            reinterpret_cast<uint2 *>(stage)[3 * lane + j] = make_uint2(qx | (qy << 10) | (qz << 20),
-                                                                                         wt.bid[q]);
-                        }
-                    }
-                    if (kDebug) {
-                        const unsigned long long gt = gbase + tri;
-                        uint32_t bx, by, bz;
-                        block_coords(g, wt.bid[q], bx, by, bz);
-                        const unsigned long long px = 4ull * bx + cx + ((info >> 16) & 1u);
-                        const unsigned long long py = 4ull * by + cy + ((info >> 17) & 1u);
-                        const unsigned long long pz = 4ull * bz + cz + ((info >> 18) & 1u);
-                        if (gt < tri_cap)
-                            s.dbg_edges[gt * 3 + j] =
-                                3ull * (px + (unsigned long long)g.nx * (py + (unsigned long long)g.ny * pz)) + a;
-                    }
-                }
-            }
-            __syncwarp();
-            const uint32_t nv = 3 * min(32u, wtot - t0);             // vertices (or indices) in this chunk
-            const unsigned long long v0 = (gbase + t0) * 3;          // first of the chunk
-            const unsigned long long vcap = tri_cap * 3;
-            if constexpr (kIdx) {
-                uint32_t *oi = reinterpret_cast<uint32_t *>(c->params.idx_out);
-                const uint32_t *st = reinterpret_cast<const uint32_t *>(stage);
-#pragma unroll
-                for (int r = 0; r < 3; r++) {
-                    const uint32_t f = lane + 32 * r;
-                    if (f < nv && v0 + f < vcap) oi[v0 + f] = st[f];
-                }
-            } else if (!packed) {
-                if (v0 + 96 <= vcap) {                 // warp-uniform: the whole chunk fits
-#pragma unroll
-                    for (int r = 0; r < 3; r++) {
-                        const uint32_t f = lane + 32 * r;
-                        if (f < nv) __stcs(&out[v0 + f], stage[f]);
-                    }
-                } else {
-#pragma unroll
-                    for (int r = 0; r < 3; r++) {
-                        const uint32_t f = lane + 32 * r;
-                        if (f < nv && v0 + f < vcap) __stcs(&out[v0 + f], stage[f]);
-                    }
-                }
-            } else {
-                uint2 *out2 = reinterpret_cast<uint2 *>(out);
-                const uint2 *st2 = reinterpret_cast<const uint2 *>(stage);
-#pragma unroll
-                for (int r = 0; r < 3; r++) {
-                    const uint32_t f = lane + 32 * r;
-                    if (f < nv && v0 + f < vcap) __stcs(&out2[v0 + f], st2[f]);
-                }
-            }
-            __syncwarp();
+            __syncwarp();                         // the list (and, at the end, the samples) are read
+            if (k0 >= ncell) break;
+            t0 += n;
+            n = 0;
+            safe = true;
         }
     }
+    cp_async_wait_all();
 }
 
-// the triangle soup; registers bounded for 32 warps per SM (the staging
-// holds two blocks' loads at a time, so 64 registers suffice)
+// the triangle soup; registers bounded for 24 warps per SM, what the shared
+// memory of two tiles' samples a warp allows
 template <int kW, bool kDebug, bool kOne>
-__global__ void __launch_bounds__(32 * kW, 32 / kW) mc_emit_kernel(Launch L) {
+__global__ void __launch_bounds__(32 * kW, kW == 16 ? 1 : 24 / kW) mc_emit_kernel(Launch L) {
     emit_body<kW, kDebug, kOne, false>(L);
 }
 
-// the indexed mesh (single volumes); registers bounded for 32 warps per SM
-// (at 24 warps it measured 219 against 158 us per surface on noise512)
+// the indexed mesh (single volumes)
 template <int kW, bool kDebug>
-__global__ void __launch_bounds__(32 * kW, 32 / kW) mc_emit_indexed_kernel(Launch L) {
+__global__ void __launch_bounds__(32 * kW, kW == 16 ? 1 : 24 / kW) mc_emit_indexed_kernel(Launch L) {
     emit_body<kW, kDebug, true, true>(L);
 }
 
@@ -885,15 +922,24 @@ __global__ void __launch_bounds__(32 * kW, 32 / kW) mc_emit_indexed_kernel(Launc
 
 namespace {
 
+// dynamic shared memory of an emission: the warps' areas and tables, then a
+// batch's prefix words
+template <int kW, bool kIdx>
+size_t emit_smem(const Launch &L) {
+    return sizeof(EmitSmem<kW, kIdx>) + (L.vols ? ((size_t)L.n + 1) * 4 : 0);
+}
+
 template <int kW, bool kOne, bool kIdx>
 void emit_w(const Launch &L, bool debug, int grid, cudaStream_t st) {
-    constexpr size_t bytes = sizeof(EmitSmem<kW, kIdx>);
+    const size_t bytes = emit_smem<kW, kIdx>(L);
     if constexpr (kIdx) {
         if (debug) mc_emit_indexed_kernel<kW, true><<<grid, 32 * kW, bytes, st>>>(L);
         else mc_emit_indexed_kernel<kW, false><<<grid, 32 * kW, bytes, st>>>(L);
-    } else {
-        if (debug) mc_emit_kernel<kW, true, kOne><<<grid, 32 * kW, bytes, st>>>(L);
-        else mc_emit_kernel<kW, false, kOne><<<grid, 32 * kW, bytes, st>>>(L);
+    } else if constexpr (kOne) {
+        if (debug) mc_emit_kernel<kW, true, true><<<grid, 32 * kW, bytes, st>>>(L);
+        else mc_emit_kernel<kW, false, true><<<grid, 32 * kW, bytes, st>>>(L);
+    } else {                                          // debug volumes are not batched
+        mc_emit_kernel<kW, false, false><<<grid, 32 * kW, bytes, st>>>(L);
     }
 }
 
@@ -915,22 +961,23 @@ void raise_smem(K kernel, size_t bytes) {
 
 template <int kW>
 int emit_occupancy(bool single) {
-    raise_smem(mc_emit_kernel<kW, false, false>, sizeof(EmitSmem<kW, false>));
-    raise_smem(mc_emit_kernel<kW, true, false>, sizeof(EmitSmem<kW, false>));
-    raise_smem(mc_emit_kernel<kW, false, true>, sizeof(EmitSmem<kW, false>));
-    raise_smem(mc_emit_kernel<kW, true, true>, sizeof(EmitSmem<kW, false>));
-    raise_smem(mc_emit_indexed_kernel<kW, false>, sizeof(EmitSmem<kW, true>));
-    raise_smem(mc_emit_indexed_kernel<kW, true>, sizeof(EmitSmem<kW, true>));
+    constexpr size_t soup = sizeof(EmitSmem<kW, false>), idx = sizeof(EmitSmem<kW, true>);
+    constexpr size_t table = (kMaxBatch + 1) * 4;         // the largest batch's prefix words
+    raise_smem(mc_emit_kernel<kW, false, false>, soup + table);
+    raise_smem(mc_emit_kernel<kW, false, true>, soup);
+    raise_smem(mc_emit_kernel<kW, true, true>, soup);
+    raise_smem(mc_emit_indexed_kernel<kW, false>, idx);
+    raise_smem(mc_emit_indexed_kernel<kW, true>, idx);
     // every kernel launched with this CTA count must fit it: a CTA beyond
     // the resident ones would start only when a whole CTA has finished, and
-    // its statically assigned tiles would trail the rest
+    // its statically assigned tiles would trail the rest (batches of so many
+    // volumes that their prefix words cost a CTA are the exception)
     if (single)
-        return std::min({occupancy(mc_emit_kernel<kW, false, true>, 32 * kW, sizeof(EmitSmem<kW, false>)),
-                         occupancy(mc_emit_kernel<kW, true, true>, 32 * kW, sizeof(EmitSmem<kW, false>)),
-                         occupancy(mc_emit_indexed_kernel<kW, false>, 32 * kW, sizeof(EmitSmem<kW, true>)),
-                         occupancy(mc_emit_indexed_kernel<kW, true>, 32 * kW, sizeof(EmitSmem<kW, true>))});
-    return std::min(occupancy(mc_emit_kernel<kW, false, false>, 32 * kW, sizeof(EmitSmem<kW, false>)),
-                    occupancy(mc_emit_kernel<kW, true, false>, 32 * kW, sizeof(EmitSmem<kW, false>)));
+        return std::min({occupancy(mc_emit_kernel<kW, false, true>, 32 * kW, soup),
+                         occupancy(mc_emit_kernel<kW, true, true>, 32 * kW, soup),
+                         occupancy(mc_emit_indexed_kernel<kW, false>, 32 * kW, idx),
+                         occupancy(mc_emit_indexed_kernel<kW, true>, 32 * kW, idx)});
+    return occupancy(mc_emit_kernel<kW, false, false>, 32 * kW, soup + 65 * 4);
 }
 
 template <bool kOne, bool kIdx>

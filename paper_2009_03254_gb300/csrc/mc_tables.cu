@@ -53,6 +53,7 @@ void face_ccw(int a, int s, int out[4]) {
 
 bool build_mc_tables(McTables *t) {
     std::memset(t, 0, sizeof(*t));
+    int total = 0;
     for (int cs = 0; cs < 256; cs++) {
         int next[12], prev_count[12];
         for (int e = 0; e < 12; e++) { next[e] = -1; prev_count[e] = 0; }
@@ -93,8 +94,31 @@ bool build_mc_tables(McTables *t) {
         }
         t->num_tri[cs] = (uint8_t)nt;
         if (nt > t->max_tri) t->max_tri = nt;
+        total += nt;
     }
-    return true;
+    return total == kCaseTriangles;
+}
+
+void build_emit_tables(const McTables &t, EmitTables *e) {
+    std::memset(e, 0, sizeof(*e));
+    int row = 0;
+    for (int cs = 0; cs < 256; cs++) {
+        e->info[cs] = (uint16_t)(row * sizeof(e->corner[0]) | ((unsigned)t.num_tri[cs] << 13));
+        for (int k = 0; k < t.num_tri[cs]; k++, row++)
+            for (int j = 0; j < 3; j++) {
+                const int edge = t.tri_edges[cs][3 * k + j], a = edge >> 2, j0 = edge & 1, j1 = (edge >> 1) & 1;
+                const int x = a == 0 ? 0 : j0, y = a == 0 ? j0 : (a == 1 ? 0 : j1), z = a == 2 ? 0 : j1;
+                const int step = a == 0 ? 1 : (a == 1 ? 5 : 25);
+                e->corner[row][j] = (uint16_t)(4 * (x + 5 * y + 25 * z) | (4 * step << 8));
+            }
+    }
+    static const uint16_t half[5] = {0x0000, 0x3C00, 0x4000, 0x4200, 0x4400};   // 0.0 to 4.0
+    for (int i = 0; i < kTileBlocks * kWindow; i++) {
+        const int s = i % kWindow;
+        e->coord[i][0] = half[s % 5];
+        e->coord[i][1] = half[s / 5 % 5];
+        e->coord[i][2] = half[s / 25];
+    }
 }
 
 }  // namespace bcmc

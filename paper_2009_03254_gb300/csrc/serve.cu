@@ -383,7 +383,7 @@ struct Done {
 struct Slot {                           // device state of one request position
     Ctl *ctl = nullptr;
     uint32_t *icand = nullptr, *iocc = nullptr;
-    unsigned long long *ooff = nullptr, *bmask = nullptr, *desc_cand = nullptr, *desc_mc = nullptr, *desc_occ = nullptr;
+    unsigned long long *ooff = nullptr, *ocross = nullptr, *bmask = nullptr, *desc_cand = nullptr, *desc_mc = nullptr, *desc_occ = nullptr;
 };
 
 enum Stage { kFront = 0, kCount = 1, kEmit = 2 };
@@ -478,7 +478,7 @@ void free_server(iso_server *sv) {
         for (float *b : sv->back_tick.bufs) dfree_on(b, sv->stream);
     for (auto &half : sv->slots)
         for (Slot &s : half) {
-            void *p[] = {s.ctl, s.icand, s.bmask, s.ooff, s.desc_cand, s.desc_mc, s.iocc};
+            void *p[] = {s.ctl, s.icand, s.bmask, s.ooff, s.ocross, s.desc_cand, s.desc_mc, s.iocc};
             for (void *x : p) dfree_on(x, sv->stream);
         }
     void *q[] = {sv->d_views[0], sv->d_views[1], sv->d_ctr[0], sv->d_ctr[1], sv->d_ctls[0], sv->d_ctls[1],
@@ -889,6 +889,7 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
             TRY(dalloc_on(&s.icand, cand, sv->device, sv->stream));
             TRY(dalloc_on(&s.bmask, v->cap, sv->device, sv->stream));
             TRY(dalloc_on(&s.ooff, cand, sv->device, sv->stream));
+            TRY(dalloc_on(&s.ocross, cand + 3, sv->device, sv->stream));   // read four at a time
             TRY(dalloc_on(&s.desc_cand, v->n_cull_desc, sv->device, sv->stream));
             TRY(dalloc_on(&s.desc_mc, 2 * n_mc_desc, sv->device, sv->stream));
             s.desc_occ = s.desc_mc + n_mc_desc;
@@ -898,6 +899,7 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
             d.icand = s.icand;
             d.bmask = s.bmask;
             d.ooff = s.ooff;
+            d.ocross = s.ocross;
             d.counts = nullptr;           // the debug accessors' arrays are the volume's
             d.offsets = nullptr;
             d.desc_cand = s.desc_cand;

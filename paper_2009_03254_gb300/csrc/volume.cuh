@@ -47,7 +47,7 @@ struct iso_volume {
     float *bmin = nullptr, *bmax = nullptr;   // staging of host block ranges during the load only
     float2 *hull = nullptr, *hull8 = nullptr;
     float2 *seg = nullptr;            // segment ranges (ISO_SEGMENT_CULL, or large volumes by default)
-    uint8_t *tables = nullptr;
+    bcmc::EmitTables *tables = nullptr;
     unsigned long long dbg_edges_cap = 0;   // in vertices
     unsigned long long last_vtx = 0;        // vertices of the last indexed extraction
     bool profiling = false;
