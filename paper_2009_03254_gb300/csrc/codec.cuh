@@ -28,14 +28,6 @@ namespace bcmc {
 
 __device__ __forceinline__ uint64_t low_mask(uint32_t n) { return n >= 64 ? ~0ull : ((1ull << n) - 1ull); }
 
-// one word of the stream: through the read-only path unless the same kernel
-// may have written it
-template <bool kReadOnly>
-__device__ __forceinline__ uint64_t load_word(const uint64_t *p) {
-    if constexpr (kReadOnly) return __ldg(p);
-    else return *p;
-}
-
 // ---------------------------------------------------------------- staging
 //
 // A warp decodes up to 32 blocks at a time, one per lane (Section 4.2.1
@@ -54,7 +46,6 @@ __host__ __device__ constexpr uint32_t stage_words(uint32_t rate) { return 32u *
 
 // Copy block `id` of each lane that has one (`have`) into the warp's
 // staging area `stage` (stage_words(rate) words).  Called by all 32 lanes.
-template <bool kReadOnly>
 __device__ __forceinline__ void stage_blocks(const uint64_t *__restrict__ bits, uint32_t rate, uint32_t id, bool have,
                                              uint32_t *stage) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -74,7 +65,7 @@ __device__ __forceinline__ void stage_blocks(const uint64_t *__restrict__ bits, 
             const uint32_t q = (j * magic) >> 16, w = j - q * rate;
             const uint32_t bq = __shfl_sync(0xffffffffu, id, (int)(q & 31u));
             v[k] = 0ull;
-            if (k0 + k < rate && ((have_mask >> q) & 1u)) v[k] = load_word<kReadOnly>(bits + (size_t)bq * rate + w);
+            if (k0 + k < rate && ((have_mask >> q) & 1u)) v[k] = __ldg(bits + (size_t)bq * rate + w);
         }
 #pragma unroll
         for (uint32_t k = 0; k < kInFlight; k++) {
@@ -121,19 +112,8 @@ struct StagedBits {
     }
 };
 
-// inverse of one two-level S-transform step on (ll, hh, h0, h1) -> (a, b, c, d)
-__device__ __forceinline__ void inv_lift4(int32_t &p0, int32_t &p1, int32_t &p2, int32_t &p3) {
-    const int32_t ll = p0, hh = p1, h0 = p2, h1 = p3;
-    const int32_t l1 = (int32_t)((uint32_t)ll - (uint32_t)(hh >> 1));
-    const int32_t l0 = (int32_t)((uint32_t)hh + (uint32_t)l1);
-    const int32_t b = (int32_t)((uint32_t)l0 - (uint32_t)(h0 >> 1));
-    const int32_t a = (int32_t)((uint32_t)h0 + (uint32_t)b);
-    const int32_t d = (int32_t)((uint32_t)l1 - (uint32_t)(h1 >> 1));
-    const int32_t c = (int32_t)((uint32_t)h1 + (uint32_t)d);
-    p0 = a; p1 = b; p2 = c; p3 = d;
-}
-
-// the same on two's-complement words held as uint32 (wrap-around arithmetic)
+// inverse of one two-level S-transform step on (ll, hh, h0, h1) -> (a, b, c, d), two's-complement words
+// held as uint32 (wrap-around arithmetic)
 __device__ __forceinline__ void inv_lift4u(uint32_t &p0, uint32_t &p1, uint32_t &p2, uint32_t &p3) {
     const uint32_t ll = p0, hh = p1, h0 = p2, h1 = p3;
     const uint32_t l1 = ll - (uint32_t)((int32_t)hh >> 1);
@@ -408,33 +388,46 @@ __device__ __forceinline__ DecodeSmem decode_smem_layout(uint64_t *base, uint32_
 }
 
 // ---------------------------------------------------------------- encoder (input generation)
+//
+// The encoder mirrors the decoder: a lane's 64 coefficients become 32 bit
+// planes in its column of shared memory, one loop of uniform steps writes
+// their code into the lane's staged block, and the warp copies its 32 staged
+// blocks out together.  The bits past the budget are simply not kept: the
+// code is a prefix of the unlimited one.  On the way each plane is cut down
+// to what the kept bits say, so the columns end up holding what parse_planes
+// would read back, and finish_planes gives the decoded samples without a
+// parse.
 
-struct BitWriter {
-    uint64_t *w;
-    uint32_t nwords;
-    uint32_t pos, end;
-    uint64_t acc;                          // bits not yet stored, starting at word pos>>6
-    __device__ void put(uint64_t bits, uint32_t count) {   // count <= 64, caller respects the budget
-        while (count) {
-            const uint32_t off = pos & 63;
-            const uint32_t take = min(count, 64u - off);
-            acc |= (bits & low_mask(take)) << off;
-            bits = take < 64 ? bits >> take : 0;
-            count -= take;
-            pos += take;
-            if ((pos & 63) == 0) { w[(pos >> 6) - 1] = acc; acc = 0; }
+// 32-bit words of a staged block being written (bits appended LSB first)
+struct StagedWriter {
+    uint32_t w, left;                      // shared address of the next word; words that may be kept
+    uint64_t acc;                          // bits not yet stored
+    uint32_t cnt;                          // how many (below 32 between calls)
+    __device__ __forceinline__ void word(uint32_t v) {
+        if (left) {
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(w), "r"(v));
+            w += 4;
+            left--;
         }
     }
-    __device__ uint32_t room() const { return end - pos; }
-    __device__ void flush() {
-        if (pos & 63) w[pos >> 6] = acc;
-        for (uint32_t i = (pos + 63) >> 6; i < nwords; i++) w[i] = 0;
+    __device__ __forceinline__ void put(uint32_t bits, uint32_t n) {   // n <= 32; bits beyond n are zero
+        acc |= (uint64_t)bits << cnt;
+        cnt += n;
+        if (cnt >= 32u) {
+            word((uint32_t)acc);
+            acc >>= 32;
+            cnt -= 32u;
+        }
+    }
+    __device__ __forceinline__ void finish() {                         // the rest of the block is zero
+        if (left) word((uint32_t)acc);
+        while (left) word(0u);
     }
 };
 
-// Encode v[64] into `rate` words at w.
-__device__ __forceinline__ void encode_block(const float (&v)[64], uint32_t rate, uint64_t *w) {
-    BitWriter bw{w, rate, 0, rate * 64u, 0};
+// Turn v[64] into bit planes at `planes` + k * stride (plane k, shared-window
+// address) and an exponent; false: the block is zero (no planes written).
+__device__ __forceinline__ bool make_planes(const float (&v)[64], uint32_t planes, uint32_t stride, int &emax) {
     int maxe = 0;
     bool nonzero = false;
 #pragma unroll
@@ -443,13 +436,8 @@ __device__ __forceinline__ void encode_block(const float (&v)[64], uint32_t rate
         nonzero |= (b & 0x7FFFFFFFu) != 0;
         maxe = max(maxe, (int)((b >> 23) & 0xFFu));
     }
-    if (!nonzero) {
-        bw.put(0, 1);
-        bw.flush();
-        return;
-    }
-    const int emax = maxe - 126;           // frexp exponent of the largest sample, >= -126
-    bw.put(1u | ((uint32_t)(emax + 127) << 1), 9);
+    emax = maxe - 126;                     // frexp exponent of the largest sample, >= -126
+    if (!nonzero) return false;
     int32_t q[64];
 #pragma unroll
     for (int i = 0; i < 64; i++) {
@@ -477,41 +465,66 @@ __device__ __forceinline__ void encode_block(const float (&v)[64], uint32_t rate
     }
     transpose32(lo);                       // lo[k] = plane k of coefficients 0-31
     transpose32(hi);
-    uint32_t n = 0;
 #pragma unroll
-    for (int j = 0; j < 32; j++) {
-        const int k = 31 - j;
-        const uint64_t x = (uint64_t)lo[k] | ((uint64_t)hi[k] << 32);
-        if (bw.room() == 0) break;
-        {
-            const uint32_t m = min(n, bw.room());
-            if (m) bw.put(x, m);
-            if (m < n) break;
+    for (int k = 0; k < 32; k++) sts_u64(planes + (uint32_t)k * stride, lo[k], hi[k]);
+    return true;
+}
+
+// Write the code of a block's planes to its staged words and cut the planes
+// down to what the kept bits hold.  One loop for all lanes: a step opens a
+// plane (its verbatim bits), then takes group-test events one by one: a
+// test bit, the zeros and the one of the run up to the next coefficient
+// reached (a one in the last coefficient is not sent), or the 0 test that
+// ends the plane.
+__device__ __forceinline__ void code_planes(StagedWriter &out, uint32_t rate, uint32_t planes, uint32_t stride,
+                                            bool nonzero, int emax) {
+    const uint32_t end = nonzero ? rate * 64u : 0u;
+    uint32_t pos = 9, n = 0;               // n: coefficients reached
+    int k = 31;
+    if (nonzero) out.put(1u | ((uint32_t)(emax + 127) << 1), 9);
+    uint64_t x = 0, kept = 0, rest = 0;    // the plane, what the kept bits say of it, its ones from n on
+    bool opening = true;
+    while (k >= 0 && pos < end) {
+        if (opening) {
+            uint32_t xlo, xhi;
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(xlo), "=r"(xhi) : "r"(planes + (uint32_t)k * stride));
+            x = ((uint64_t)xhi << 32) | xlo;
+            const uint64_t low = low_mask(n);
+            out.put(xlo & (uint32_t)low, min(n, 32u));
+            if (n > 32u) out.put(xhi & (uint32_t)(low >> 32), n - 32u);
+            kept = x & low & low_mask(min(64u, end - pos));
+            rest = x & ~low;
+            pos += n;
         }
-        bool out = false;
-        while (n < 64) {
-            if (bw.room() == 0) { out = true; break; }
-            const uint64_t rest = x >> n;
-            if (!rest) { bw.put(0, 1); break; }
-            bw.put(1, 1);
-            const uint32_t jpos = n + (uint32_t)__ffsll((long long)rest) - 1u;  // first one at or after n
-            if (jpos < 63) {
-                const uint32_t len = jpos - n + 1;          // zeros then the one
-                const uint32_t r = bw.room();
-                if (len > r) { bw.put(0, r); out = true; break; }
-                bw.put(1ull << (len - 1), len);
-                n = jpos + 1;
+        bool done = n >= 64u || pos >= end;
+        if (!done) {
+            if (rest == 0) {               // nothing more in this plane
+                out.put(0u, 1);
+                pos += 1;
+                done = true;
             } else {
-                const uint32_t len = 63 - n;                // zeros up to coefficient 62; 63's one implied
-                const uint32_t r = bw.room();
-                if (len > r) { bw.put(0, r); out = true; break; }
-                if (len) bw.put(0, len);
-                n = 64;
+                const uint32_t p = (uint32_t)__ffsll((long long)rest) - 1u, z = p - n;
+                // the test's 1, z zeros and, unless p is the last coefficient, its 1
+                const uint32_t len = z + (p < 63u ? 2u : 1u);
+                const uint64_t code = 1ull | (p < 63u && z < 63u ? 2ull << z : 0ull);
+                out.put((uint32_t)code, min(len, 32u));
+                if (len > 32u) out.put((uint32_t)(code >> 32), min(len, 64u) - 32u);
+                pos += len;
+                if (pos <= end) kept |= rest & (0ull - rest);
+                rest &= rest - 1;
+                n = p + 1;
+                done = n >= 64u || pos >= end;
             }
         }
-        if (out) break;
+        if (done) {
+            if (pos > end) sts_u64(planes + (uint32_t)k * stride, (uint32_t)kept, (uint32_t)(kept >> 32));
+            else if (pos == end && kept != x) sts_u64(planes + (uint32_t)k * stride, (uint32_t)kept, (uint32_t)(kept >> 32));
+            k--;
+        }
+        opening = done;
     }
-    bw.flush();
+    for (; k >= 0; k--) sts_u64(planes + (uint32_t)k * stride, 0u, 0u);
+    out.finish();
 }
 
 }  // namespace bcmc

@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 768 / kDecodeThreads) decode_n
         const uint32_t b = have ? s.inew[r] : 0u;
         const uint32_t slot = have ? s.newslot[r] : 0u;
         have = have && in_bounds(b < vol_of<kOne>(L, v).g.nb && slot < c->cap, &c->status);
-        stage_blocks<true>(s.bits, rate, b, have, sm.stage);
+        stage_blocks(s.bits, rate, b, have, sm.stage);
         if (!have) continue;
         float val[64];
         decode_staged(sm.stage + (threadIdx.x & 31u) * (2u * rate + 1u), rate, sm.tab, val, sm.planes + threadIdx.x,
