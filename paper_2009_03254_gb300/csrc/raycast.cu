@@ -6,8 +6,10 @@
 // iso_raycast runs the extraction's front for the isovalue (range test,
 // cache update, decode: every block whose 2x2x2 group range holds the
 // isovalue is active, and so is its whole group, so every sample a ray can
-// need is cached), then one thread per pixel (16 x 16 pixel tiles per CTA)
-// casts its ray:
+// need is cached, and its below mask with it), then cross_kernel finds each
+// candidate's crossing cells from the masks (a bit per block, 64 bits per
+// slot), and one thread per pixel (16 x 16 pixel tiles per CTA) casts its
+// ray:
 //   - a slab test against the volume box gives the start; the block, then
 //     the cell, holding the current point starts each level;
 //   - each box's interval comes from its own slab test (not an
@@ -15,9 +17,13 @@
 //     ray), and the next box is one step along the exit axis, so the
 //     visited boxes and their intervals are fixed by the ray;
 //   - a block is searched when its precomputed group range (hull8) holds
-//     the isovalue; a cell when its 8 corners' range does: 5 samples of the
-//     trilinear interpolant on its interval, then 12 bisection steps at the
-//     first change of side;
+//     the isovalue; a cell when its 8 corners' range does, i.e. when it is a
+//     crossing cell (so blocks without any are passed by at once, and only
+//     the samples of crossing cells are read): 5 samples of the trilinear
+//     interpolant on its interval, then 12 bisection steps at the first
+//     change of side;
+//   - a step changes one coordinate, so only that axis' interval is computed
+//     again, by the same operations on the same numbers;
 //   - the hit is shaded from the interpolant's gradient (two-sided Lambert).
 // Every float operation is one IEEE float32 operation (this file is built
 // without multiply-add contraction), so the depths equal the CPU oracle's
@@ -27,6 +33,7 @@
 #include <cstdint>
 
 #include "bcmc.h"
+#include "cell_masks.cuh"
 #include "volume.cuh"
 
 namespace bcmc {
@@ -38,7 +45,8 @@ constexpr int kTile = 16;                               // pixels per tile side 
 struct CastArgs {
     const int32_t *islot;
     const float *slots;
-    const float2 *hull8;
+    const uint32_t *occ;          // a bit per block: some cell crosses
+    const unsigned long long *cross;   // per slot of such a block: its crossing cells
     const Ctl *ctl;
     unsigned long long *hits;
     uint32_t *rgba;
@@ -125,8 +133,41 @@ __device__ bool cell_root(const Ray &r, const float c[8], const int cell[3], flo
     return false;
 }
 
+// The ray's interval on each axis of a box, and the box's own by slab()'s
+// rule: an axis parallel to the ray bounds nothing (the caller has seen that
+// it does not miss the box).
+struct Axes {
+    float mn[3], mx[3];
+    __device__ __forceinline__ void meet(float &tin, float &tout, int &ax) const {
+        float a = -inf_f(), b = inf_f();
+        ax = -1;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            if (mn[k] > a) a = mn[k];
+            if (mx[k] < b) {
+                b = mx[k];
+                ax = k;
+            }
+        }
+        tin = a;
+        tout = b;
+    }
+};
+
+__device__ __forceinline__ void axis_interval(float o, float d, float inv, float lo, float hi, float &mn, float &mx) {
+    const float t0 = (lo - o) * inv, t1 = (hi - o) * inv;
+    mn = d == 0.0f ? -inf_f() : (t0 < t1 ? t0 : t1);
+    mx = d == 0.0f ? inf_f() : (t0 < t1 ? t1 : t0);
+}
+
+// v[ax] without an indexed array
+template <class T>
+__device__ __forceinline__ T pick(const T v[3], int ax) {
+    return ax == 0 ? v[0] : (ax == 1 ? v[1] : v[2]);
+}
+
 // the first hit of the ray; the hit cell's corners in cv
-__device__ bool cast(const CastArgs &a, const Ray &r, int32_t *gs, float &thit, int hc[3], int hb[3], float cv[8]) {
+__device__ bool cast(const CastArgs &a, const Ray &r, float &thit, int hc[3], int hb[3], float cv[8]) {
     const int n[3] = {(int)a.nx, (int)a.ny, (int)a.nz};
     int ncb[3];
 #pragma unroll
@@ -142,60 +183,53 @@ __device__ bool cast(const CastArgs &a, const Ray &r, int32_t *gs, float &thit, 
     if (t0 < 0.0f) t0 = 0.0f;
     if (!(t0 <= t1)) return false;
     int b[3];
+    Axes ba;
 #pragma unroll
-    for (int k = 0; k < 3; k++) b[k] = clampi((int)floorf((r.o[k] + t0 * r.d[k]) * 0.25f), 0, ncb[k] - 1);
+    for (int k = 0; k < 3; k++) {
+        b[k] = clampi((int)floorf((r.o[k] + t0 * r.d[k]) * 0.25f), 0, ncb[k] - 1);
+        const float lo = (float)(4 * b[k]), hi = (float)min(4 * b[k] + 4, n[k] - 1);
+        if (r.d[k] == 0.0f && (r.o[k] < lo || r.o[k] > hi)) return false;   // and so for every block on the way
+        axis_interval(r.o[k], r.d[k], r.inv[k], lo, hi, ba.mn[k], ba.mx[k]);
+    }
     float t = t0;
-    const int stride = blockDim.x;                      // group slots of this thread: gs[k * stride]
     for (;;) {
-        float blo[3], bhi[3];
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            blo[k] = (float)(4 * b[k]);
-            const int h = 4 * b[k] + 4;
-            bhi[k] = (float)(h < n[k] - 1 ? h : n[k] - 1);
-        }
         float bin, bout;
         int bax;
-        if (!slab(r, blo, bhi, bin, bout, bax) || bax < 0) return false;
+        ba.meet(bin, bout, bax);
+        if (bax < 0) return false;
         if (bin < t) bin = t;
         const uint32_t bid = (uint32_t)b[0] + a.nbx * ((uint32_t)b[1] + a.nby * (uint32_t)b[2]);
-        const float2 hull = a.hull8[bid];
-        if (bin <= bout && hull.x < a.iso && a.iso <= hull.y) {
-            // cache slots of the block's group (-1 outside the volume)
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                const int gx = b[0] + (k & 1), gy = b[1] + ((k >> 1) & 1), gz = b[2] + (k >> 2);
-                const bool in = gx < (int)a.nbx && gy < (int)a.nby && gz < (int)a.nbz;
-                gs[k * stride] = in ? a.islot[(uint32_t)gx + a.nbx * ((uint32_t)gy + a.nby * (uint32_t)gz)] : -1;
-            }
+        if (bin <= bout && ((__ldg(a.occ + (bid >> 5)) >> (bid & 31u)) & 1u)) {
+            const unsigned long long cross = __ldg(a.cross + __ldg(a.islot + bid));
             int c[3];
+            Axes ca;
+            bool miss = false;
 #pragma unroll
             for (int k = 0; k < 3; k++) {
-                const int last = 4 * b[k] + 3 < n[k] - 2 ? 4 * b[k] + 3 : n[k] - 2;
-                c[k] = clampi((int)floorf(r.o[k] + bin * r.d[k]), 4 * b[k], last);
+                c[k] = clampi((int)floorf(r.o[k] + bin * r.d[k]), 4 * b[k], min(4 * b[k] + 3, n[k] - 2));
+                const float lo = (float)c[k], hi = (float)(c[k] + 1);
+                miss = miss || (r.d[k] == 0.0f && (r.o[k] < lo || r.o[k] > hi));
+                axis_interval(r.o[k], r.d[k], r.inv[k], lo, hi, ca.mn[k], ca.mx[k]);
             }
-            for (;;) {
-                const float clo[3] = {(float)c[0], (float)c[1], (float)c[2]};
-                const float chi[3] = {(float)(c[0] + 1), (float)(c[1] + 1), (float)(c[2] + 1)};
+            while (!miss) {
                 float cin, cout;
                 int cax;
-                if (!slab(r, clo, chi, cin, cout, cax) || cax < 0) break;
+                ca.meet(cin, cout, cax);
+                if (cax < 0) break;
                 if (cin < bin) cin = bin;
-                if (cin <= cout) {
-                    float mn = inf_f(), mx = -inf_f();
+                const uint32_t cell = (uint32_t)(c[0] & 3) | ((uint32_t)(c[1] & 3) << 2) | ((uint32_t)(c[2] & 3) << 4);
+                if (cin <= cout && ((cross >> cell) & 1ull)) {
 #pragma unroll
                     for (int k = 0; k < 8; k++) {
                         const int x = c[0] + (k & 1), y = c[1] + ((k >> 1) & 1), z = c[2] + (k >> 2);
-                        const int g = ((x >> 2) - b[0]) | (((y >> 2) - b[1]) << 1) | (((z >> 2) - b[2]) << 2);
-                        const int32_t sl = gs[g * stride];
+                        const int32_t sl = __ldg(a.islot + ((uint32_t)(x >> 2) + a.nbx * ((uint32_t)(y >> 2) +
+                                                                                          a.nby * (uint32_t)(z >> 2))));
                         float v = 0.0f;
-                        if (sl >= 0) v = a.slots[(size_t)sl * 64 + (x & 3) + 4 * (y & 3) + 16 * (z & 3)];
+                        if (sl >= 0) v = __ldg(a.slots + (size_t)sl * 64 + (x & 3) + 4 * (y & 3) + 16 * (z & 3));
                         else atomicOr(a.err, 1u);       // never: every group member is cached
                         cv[k] = v;
-                        mn = k == 0 ? v : (v < mn ? v : mn);
-                        mx = k == 0 ? v : (v > mx ? v : mx);
                     }
-                    if (mn < a.iso && a.iso <= mx && cell_root(r, cv, c, a.iso, cin, cout, thit)) {
+                    if (cell_root(r, cv, c, a.iso, cin, cout, thit)) {
 #pragma unroll
                         for (int k = 0; k < 3; k++) {
                             hc[k] = c[k];
@@ -205,31 +239,55 @@ __device__ bool cast(const CastArgs &a, const Ray &r, int32_t *gs, float &thit, 
                     }
                 }
                 // one step along the exit axis (selects, not an indexed array)
-                bool out = false;
+                const float d = pick(r.d, cax);
+                const int cn = pick(c, cax) + (d > 0.0f ? 1 : -1), c0 = 4 * pick(b, cax);
+                if (cn < c0 || cn > min(c0 + 3, pick(n, cax) - 2)) break;
+                float mn, mx;
+                axis_interval(pick(r.o, cax), d, pick(r.inv, cax), (float)cn, (float)(cn + 1), mn, mx);
 #pragma unroll
-                for (int k = 0; k < 3; k++) {
-                    if (k != cax) continue;
-                    c[k] += r.d[k] > 0.0f ? 1 : -1;
-                    const int last = 4 * b[k] + 3 < n[k] - 2 ? 4 * b[k] + 3 : n[k] - 2;
-                    out = c[k] < 4 * b[k] || c[k] > last;
-                }
-                if (out) break;
+                for (int k = 0; k < 3; k++)
+                    if (k == cax) {
+                        c[k] = cn;
+                        ca.mn[k] = mn;
+                        ca.mx[k] = mx;
+                    }
             }
         }
-        bool out = false;
+        const float d = pick(r.d, bax);
+        const int bn = pick(b, bax) + (d > 0.0f ? 1 : -1);
+        if (bn < 0 || bn >= pick(ncb, bax)) return false;
+        float mn, mx;
+        axis_interval(pick(r.o, bax), d, pick(r.inv, bax), (float)(4 * bn), (float)min(4 * bn + 4, pick(n, bax) - 1), mn, mx);
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
-            if (k != bax) continue;
-            b[k] += r.d[k] > 0.0f ? 1 : -1;
-            out = b[k] < 0 || b[k] >= ncb[k];
-        }
-        if (out) return false;
+        for (int k = 0; k < 3; k++)
+            if (k == bax) {
+                b[k] = bn;
+                ba.mn[k] = mn;
+                ba.mx[k] = mx;
+            }
         t = bout;
     }
 }
 
+// The crossing cells of every candidate (blocks without one are not marked),
+// a candidate per thread; `occ` was cleared.
+__global__ void __launch_bounds__(256) cross_kernel(DevState s, Geom g, uint32_t *occ, unsigned long long *cross) {
+    const uint32_t n = mc_candidates(s.ctl);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t b = s.icand[i];
+        unsigned long long m[8];
+        uint32_t lim;
+        corner_masks(s, g, b, m, lim);
+        const unsigned long long x = crossing_cells(m, valid_cells(lim));
+        const int32_t sl = s.islot[b];
+        if (x && sl >= 0) {
+            cross[sl] = x;
+            atomicOr(occ + (b >> 5), 1u << (b & 31u));
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kTile * kTile) raycast_kernel(CastArgs a) {
-    __shared__ int32_t gs[8 * kTile * kTile];
     if (a.ctl->status & (kStatusBudget | kStatusAnyTimeout)) return;   // the cache update failed
     const uint32_t tiles_x = (a.width + kTile - 1) / kTile;
     const int i = (int)((blockIdx.x % tiles_x) * kTile + (threadIdx.x % kTile));
@@ -248,7 +306,7 @@ __global__ void __launch_bounds__(kTile * kTile) raycast_kernel(CastArgs a) {
         const size_t px = (size_t)j * a.width + i;
         float t, cv[8];
         int c[3], b[3];
-        hit = cast(a, r, gs + threadIdx.x, t, c, b, cv);
+        hit = cast(a, r, t, c, b, cv);
         if (!hit) {
             a.hits[px] = ~0ull;
             if (a.rgba) a.rgba[px] = 0u;
@@ -315,16 +373,21 @@ extern "C" int iso_raycast(iso_volume *v, float isovalue, const iso_pinhole *cam
     // the extraction's front for this isovalue: range test, cache update, decode
     *v->host_params = Params{isovalue, kVertexFloat4, 0u, 0u, 0u, 0u, 0ull, 0ull, 0ull, 0ull, 0ull};
     ISO_CK(cudaMemcpyAsync(&v->s.ctl->params, v->host_params, sizeof(Params), cudaMemcpyHostToDevice, st));
-    Launch L{nullptr, 1u, single_counters(v), VolEntry{v->s, v->g, v->n_cull_desc, v->n_lru_desc}};
-    L.one.s.bmask = nullptr;                             // nothing counts here
+    const Launch L{nullptr, 1u, single_counters(v), VolEntry{v->s, v->g, v->n_cull_desc, v->n_lru_desc}};
     launch_front(L, v->plan, st, nullptr);
+    // counters, a bit per block, then the slots' crossing cells
     void *scratch = nullptr;
-    int rc = dalloc_bytes(&scratch, 16, v->device, st);
+    const size_t occ_at = 256, occ_bytes = ((size_t)v->g.nb + 31) / 32 * 4,
+                 cross_at = occ_at + (occ_bytes + 255) / 256 * 256;
+    int rc = dalloc_bytes(&scratch, cross_at + (size_t)v->cap * 8, v->device, st);
     if (rc) return rc;
+    uint32_t *occ = reinterpret_cast<uint32_t *>(static_cast<char *>(scratch) + occ_at);
+    unsigned long long *cross = reinterpret_cast<unsigned long long *>(static_cast<char *>(scratch) + cross_at);
     CastArgs a{};
     a.islot = v->s.islot;
     a.slots = v->s.slots;
-    a.hull8 = v->s.hull8;
+    a.occ = occ;
+    a.cross = cross;
     a.ctl = v->s.ctl;
     a.hits = reinterpret_cast<unsigned long long *>(d_hits);
     a.rgba = d_rgba;
@@ -347,8 +410,9 @@ extern "C" int iso_raycast(iso_volume *v, float isovalue, const iso_pinhole *cam
         a.light[k] = cam->light[k];
     }
     unsigned long long counters[2] = {0, 0};
-    cudaError_t e = cudaMemsetAsync(scratch, 0, 16, st);
+    cudaError_t e = cudaMemsetAsync(scratch, 0, occ_at + occ_bytes, st);
     if (e == cudaSuccess) {
+        cross_kernel<<<v->plan.mc_scan, 256, 0, st>>>(v->s, v->g, occ, cross);
         const uint32_t tiles = ((cam->width + kTile - 1) / kTile) * ((cam->height + kTile - 1) / kTile);
         raycast_kernel<<<tiles, kTile * kTile, 0, st>>>(a);
         e = cudaGetLastError();
