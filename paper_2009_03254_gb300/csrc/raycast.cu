@@ -40,7 +40,8 @@ namespace bcmc {
 
 namespace {
 
-constexpr int kTile = 16;                               // pixels per tile side (one CTA)
+constexpr int kTile = 16;                               // pixels per tile side (four CTAs, 8 x 4 pixels a warp)
+constexpr int kCastThreads = 64;
 
 struct CastArgs {
     const int32_t *islot;
@@ -101,14 +102,14 @@ __device__ __forceinline__ float trilinear(const float c[8], float fx, float fy,
     return c0 + fz * (c1 - c0);
 }
 
-__device__ __forceinline__ float g_at(const Ray &r, const float c[8], const int cell[3], float iso, float t) {
-    const float fx = clamp01(r.o[0] + t * r.d[0] - (float)cell[0]);
-    const float fy = clamp01(r.o[1] + t * r.d[1] - (float)cell[1]);
-    const float fz = clamp01(r.o[2] + t * r.d[2] - (float)cell[2]);
+__device__ __forceinline__ float g_at(const Ray &r, const float c[8], const float cell[3], float iso, float t) {
+    const float fx = clamp01(r.o[0] + t * r.d[0] - cell[0]);
+    const float fy = clamp01(r.o[1] + t * r.d[1] - cell[1]);
+    const float fz = clamp01(r.o[2] + t * r.d[2] - cell[2]);
     return trilinear(c, fx, fy, fz) - iso;
 }
 
-__device__ bool cell_root(const Ray &r, const float c[8], const int cell[3], float iso, float a, float b,
+__device__ __forceinline__ bool cell_root(const Ray &r, const float c[8], const float cell[3], float iso, float a, float b,
                           float &thit) {
     const float h = (b - a) * 0.25f;
     float tk = a;
@@ -166,8 +167,9 @@ __device__ __forceinline__ T pick(const T v[3], int ax) {
     return ax == 0 ? v[0] : (ax == 1 ? v[1] : v[2]);
 }
 
-// the first hit of the ray; the hit cell's corners in cv
-__device__ bool cast(const CastArgs &a, const Ray &r, float &thit, int hc[3], int hb[3], float cv[8]) {
+// The first hit of any ray; the hit cell's corners in cv.  Box by box, every
+// interval from all its planes: for the rays cast() does not take.
+__device__ __noinline__ bool cast_any(const CastArgs &a, const Ray &r, float &thit, float hc[3], uint32_t &hb, float cv[8]) {
     const int n[3] = {(int)a.nx, (int)a.ny, (int)a.nz};
     int ncb[3];
 #pragma unroll
@@ -229,12 +231,11 @@ __device__ bool cast(const CastArgs &a, const Ray &r, float &thit, int hc[3], in
                         else atomicOr(a.err, 1u);       // never: every group member is cached
                         cv[k] = v;
                     }
-                    if (cell_root(r, cv, c, a.iso, cin, cout, thit)) {
+                    const float lo[3] = {(float)c[0], (float)c[1], (float)c[2]};
+                    if (cell_root(r, cv, lo, a.iso, cin, cout, thit)) {
+                        hb = bid;
 #pragma unroll
-                        for (int k = 0; k < 3; k++) {
-                            hc[k] = c[k];
-                            hb[k] = b[k];
-                        }
+                        for (int k = 0; k < 3; k++) hc[k] = lo[k];
                         return true;
                     }
                 }
@@ -269,6 +270,177 @@ __device__ bool cast(const CastArgs &a, const Ray &r, float &thit, int hc[3], in
     }
 }
 
+// A ray's place on one level of the grid (blocks, or the cells of one
+// block): per axis the plane the current box is left through, the ray's
+// parameter there and the boxes left on that side; the box's entry, and its
+// index (block id, or the cell's bit).
+struct Place {
+    float plane[3], exit[3], entry;
+    int left[3], index;
+};
+
+// The first hit of the ray; the hit cell's corners in cv and its low corner
+// in hc.  Called by all lanes of a warp (`live`: this lane has a ray).  For
+// rays whose reciprocals are finite in volumes whose coordinates are exact in
+// float32: no interval is NaN, on every axis a box's entry value is at most
+// its exit value, and the next box's entry value along the exit axis is this
+// box's exit value.  So a box's entry is the larger of the last box's entry
+// and exit, and a step computes one new exit, by axis_interval()'s operations.
+//
+// One loop steps blocks and cells alike, so that the lanes of a warp step
+// together whichever they are at.  A lane at a block to be searched waits
+// until a quarter of the warp's rays do (or none steps), and then all such
+// lanes go into their blocks; a lane at a crossing cell waits for half of
+// them, and then the cells' roots are looked for together.  (Waiting for all
+// of them adds up the longest paths of every stage: 3000 steps for a warp
+// whose longest ray takes 300.)
+// Bound by instruction issue (14 of 32 lanes step at a time) and, at the end,
+// by the latency of the longest rays.  1080p over a 384^3 noise volume: 588
+// us; nested loops that tested every cell's samples took 1080 and had 6 lanes
+// active.  Picking the stepped axis' numbers by selects instead of a branch
+// per axis took 650.
+__device__ __forceinline__ bool cast(const CastArgs &a, const Ray &r, bool live, float &thit, float hc[3], uint32_t &hb,
+                                     float cv[8]) {
+    const int n[3] = {(int)a.nx, (int)a.ny, (int)a.nz};
+    if (n[0] < 2 || n[1] < 2 || n[2] < 2) return false;
+    const float vlo[3] = {0.0f, 0.0f, 0.0f};
+    const float vhi[3] = {(float)(n[0] - 1), (float)(n[1] - 1), (float)(n[2] - 1)};
+    float t0 = 0.0f, t1 = 0.0f;
+    int ax;
+    if (!slab(r, vlo, vhi, t0, t1, ax)) live = false;
+    if (t0 < 0.0f) t0 = 0.0f;
+    if (!(t0 <= t1)) live = false;
+    const int stride[3] = {1, (int)a.nbx, (int)(a.nbx * a.nby)};
+    Place w, blk;                                          // where the ray is; its block while it is in the cells
+    w.entry = -inf_f();
+    w.index = 0;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int last = (n[k] - 2) / 4, b = clampi((int)floorf((r.o[k] + t0 * r.d[k]) * 0.25f), 0, last);
+        const bool up = r.d[k] > 0.0f;
+        const float lo = (float)(4 * b), hi = (float)min(4 * b + 4, n[k] - 1);
+        if (r.d[k] == 0.0f && (r.o[k] < lo || r.o[k] > hi)) live = false;   // and so for every block on the way
+        float mn;
+        axis_interval(r.o[k], r.d[k], r.inv[k], lo, hi, mn, w.exit[k]);
+        if (mn > w.entry) w.entry = mn;
+        w.plane[k] = (float)(up ? 4 * b + 4 : 4 * b);
+        w.left[k] = up ? last - b : b;
+        w.index += b * stride[k];
+    }
+    if (w.entry < t0) w.entry = t0;
+    blk = w;
+    bool found = false, cells = false, searched = false;   // searched: this block is done, step on
+    unsigned long long cross = 0;
+    float tout = 0.0f;
+    auto step = [&]() {
+        const bool p0 = w.exit[0] == tout, p1 = !p0 && w.exit[1] == tout;   // the first axis with the smallest exit
+        const float size = cells ? 1.0f : 4.0f;
+        if (w.entry < tout) w.entry = tout;
+        int out = 0;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const bool go = k == 0 ? p0 : (k == 1 ? p1 : (!p0 && !p1));
+            const bool up = r.d[k] > 0.0f;
+            if (go) {
+                w.plane[k] = __fadd_rn(w.plane[k], up ? size : -size);
+                w.exit[k] = (fminf(w.plane[k], vhi[k]) - r.o[k]) * r.inv[k];
+                w.left[k] -= 1;
+                out = w.left[k];
+                const int by = cells ? 1 << (2 * k) : stride[k];
+                w.index += up ? by : -by;
+            }
+        }
+        if (out < 0 || !(tout < inf_f())) {
+            if (cells) {                                   // out of the block's cells: back to the block
+                w = blk;
+                cells = false;
+                searched = true;
+            } else {
+                live = false;
+            }
+        }
+    };
+    bool root = false, enter = false;                      // what the lane waits for
+    for (;;) {
+        if (live && !root && !enter) {
+            tout = fminf(fminf(w.exit[0], w.exit[1]), w.exit[2]);
+            const bool inside = w.entry <= tout;
+            if (cells) root = inside && ((cross >> w.index) & 1ull);
+            else enter = !searched && inside && ((__ldg(a.occ + ((uint32_t)w.index >> 5)) >> (w.index & 31)) & 1u);
+            if (!(tout < inf_f())) root = enter = false;       // parallel to every axis: step() ends the search
+            if (!root && !enter) {
+                if (!cells) searched = false;
+                step();
+            }
+        }
+        const uint32_t rays = __ballot_sync(0xffffffffu, live), at_cell = __ballot_sync(0xffffffffu, root),
+                       at_block = __ballot_sync(0xffffffffu, enter);
+        if (!rays) return found;
+        const bool stuck = rays == (at_cell | at_block);
+        if (at_block && (stuck || 4 * __popc(at_block) >= __popc(rays))) {
+            if (enter) {
+                enter = false;
+                cross = __ldg(a.cross + __ldg(a.islot + w.index));
+                blk = w;
+                float entry = -inf_f();
+                bool miss = false;
+                int bit = 0;
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    const bool up = r.d[k] > 0.0f;
+                    const int b4 = (int)w.plane[k] - (up ? 4 : 0), last = min(b4 + 3, n[k] - 2);
+                    const int q = clampi((int)floorf(r.o[k] + blk.entry * r.d[k]), b4, last);
+                    const float lo = (float)q, hi = (float)(q + 1);
+                    miss = miss || (r.d[k] == 0.0f && (r.o[k] < lo || r.o[k] > hi));
+                    float mn;
+                    axis_interval(r.o[k], r.d[k], r.inv[k], lo, hi, mn, w.exit[k]);
+                    if (mn > entry) entry = mn;
+                    w.plane[k] = up ? hi : lo;
+                    w.left[k] = up ? last - q : q - b4;
+                    bit += (q - b4) << (2 * k);
+                }
+                w.index = bit;
+                w.entry = entry < blk.entry ? blk.entry : entry;
+                cells = !miss;
+                if (miss) {
+                    w = blk;
+                    searched = true;
+                }
+            }
+            continue;
+        }
+        if (at_cell && (stuck || 2 * __popc(at_cell) >= __popc(rays)) && root) {
+            root = false;
+            float lo[3];
+            int c[3];
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                lo[k] = w.plane[k] - (r.d[k] > 0.0f ? 1.0f : 0.0f);
+                c[k] = (int)lo[k];
+            }
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                const int x = c[0] + (k & 1), y = c[1] + ((k >> 1) & 1), z = c[2] + (k >> 2);
+                const int32_t sl = __ldg(a.islot + ((uint32_t)(x >> 2) + a.nbx * ((uint32_t)(y >> 2) +
+                                                                                  a.nby * (uint32_t)(z >> 2))));
+                float v = 0.0f;
+                if (sl >= 0) v = __ldg(a.slots + (size_t)sl * 64 + (x & 3) + 4 * (y & 3) + 16 * (z & 3));
+                else atomicOr(a.err, 1u);               // never: every group member is cached
+                cv[k] = v;
+            }
+            if (cell_root(r, cv, lo, a.iso, w.entry, tout, thit)) {
+                found = true;
+                live = false;
+                hb = (uint32_t)blk.index;
+#pragma unroll
+                for (int k = 0; k < 3; k++) hc[k] = lo[k];
+            } else {
+                step();
+            }
+        }
+    }
+}
+
 // The crossing cells of every candidate (blocks without one are not marked),
 // a candidate per thread; `occ` was cleared.
 __global__ void __launch_bounds__(256) cross_kernel(DevState s, Geom g, uint32_t *occ, unsigned long long *cross) {
@@ -287,13 +459,18 @@ __global__ void __launch_bounds__(256) cross_kernel(DevState s, Geom g, uint32_t
     }
 }
 
-__global__ void __launch_bounds__(kTile * kTile) raycast_kernel(CastArgs a) {
+__global__ void __launch_bounds__(kCastThreads) raycast_kernel(CastArgs a) {
     if (a.ctl->status & (kStatusBudget | kStatusAnyTimeout)) return;   // the cache update failed
     const uint32_t tiles_x = (a.width + kTile - 1) / kTile;
-    const int i = (int)((blockIdx.x % tiles_x) * kTile + (threadIdx.x % kTile));
-    const int j = (int)((blockIdx.x / tiles_x) * kTile + (threadIdx.x / kTile));
+    // a warp takes 8 x 4 pixels of the tile: nearby rays take similar steps
+    constexpr uint32_t kParts = kTile * kTile / kCastThreads;
+    const uint32_t tile = blockIdx.x / kParts, w = (blockIdx.x % kParts) * (kCastThreads / 32) + (threadIdx.x >> 5),
+                   l = threadIdx.x & 31u;
+    const int i = (int)((tile % tiles_x) * kTile + 8 * (w & 1u) + (l & 7u));
+    const int j = (int)((tile / tiles_x) * kTile + 4 * (w >> 1) + (l >> 3));
+    const bool inside = i < (int)a.width && j < (int)a.height;
     bool hit = false;
-    if (i < (int)a.width && j < (int)a.height) {
+    {
         const float u = ((float)i + 0.5f) / (float)a.width * 2.0f - 1.0f;
         const float v = ((float)j + 0.5f) / (float)a.height * 2.0f - 1.0f;
         Ray r;
@@ -305,22 +482,27 @@ __global__ void __launch_bounds__(kTile * kTile) raycast_kernel(CastArgs a) {
         }
         const size_t px = (size_t)j * a.width + i;
         float t, cv[8];
-        int c[3], b[3];
-        hit = cast(a, r, t, c, b, cv);
-        if (!hit) {
+        float c[3];
+        uint32_t b;
+        bool regular = max(max(a.nx, a.ny), a.nz) < (1u << 24);
+#pragma unroll
+        for (int k = 0; k < 3; k++) regular = regular && fabsf(r.inv[k]) < inf_f() && fabsf(r.d[k]) < inf_f();
+        hit = cast(a, r, inside && regular, t, c, b, cv);
+        if (inside && !regular) hit = cast_any(a, r, t, c, b, cv);
+        if (!inside) {
+        } else if (!hit) {
             a.hits[px] = ~0ull;
             if (a.rgba) a.rgba[px] = 0u;
         } else {
-            const uint32_t id = (uint32_t)b[0] + a.nbx * ((uint32_t)b[1] + a.nby * (uint32_t)b[2]);
-            a.hits[px] = ((unsigned long long)__float_as_uint(t) << 32) | id;
+            a.hits[px] = ((unsigned long long)__float_as_uint(t) << 32) | b;
             if (a.rgba) {
                 const float base[3] = {0.85f, 0.75f, 0.55f};
                 const float l2 = a.light[0] * a.light[0] + a.light[1] * a.light[1] + a.light[2] * a.light[2];
                 const float linv = 1.0f / sqrtf(l2);
                 const float L[3] = {a.light[0] * linv, a.light[1] * linv, a.light[2] * linv};
-                const float fx = clamp01(r.o[0] + t * r.d[0] - (float)c[0]);
-                const float fy = clamp01(r.o[1] + t * r.d[1] - (float)c[1]);
-                const float fz = clamp01(r.o[2] + t * r.d[2] - (float)c[2]);
+                const float fx = clamp01(r.o[0] + t * r.d[0] - c[0]);
+                const float fy = clamp01(r.o[1] + t * r.d[1] - c[1]);
+                const float fz = clamp01(r.o[2] + t * r.d[2] - c[2]);
                 const float gx = (1.0f - fz) * ((1.0f - fy) * (cv[1] - cv[0]) + fy * (cv[3] - cv[2])) +
                                  fz * ((1.0f - fy) * (cv[5] - cv[4]) + fy * (cv[7] - cv[6]));
                 const float gy = (1.0f - fz) * ((1.0f - fx) * (cv[2] - cv[0]) + fx * (cv[3] - cv[1])) +
@@ -414,7 +596,7 @@ extern "C" int iso_raycast(iso_volume *v, float isovalue, const iso_pinhole *cam
     if (e == cudaSuccess) {
         cross_kernel<<<v->plan.mc_scan, 256, 0, st>>>(v->s, v->g, occ, cross);
         const uint32_t tiles = ((cam->width + kTile - 1) / kTile) * ((cam->height + kTile - 1) / kTile);
-        raycast_kernel<<<tiles, kTile * kTile, 0, st>>>(a);
+        raycast_kernel<<<tiles * (kTile * kTile / kCastThreads), kCastThreads, 0, st>>>(a);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(v->host_ctl, v->s.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st);
