@@ -290,6 +290,7 @@ Plan launch_plan(const Plan *want, int device, uint64_t total_blocks, uint64_t t
     }
     int *ctas = &use.prep;
     for (int k = 0; k < 8; k++) ctas[k] = std::max(1, ctas[k]) * sms;
+    use.mc_scan = std::min(use.mc_scan, (int)kMaxCountCtas);
     // no more CTAs than work items (each bound holds for any isovalue)
     auto clamp = [](int &grid, uint64_t items) {
         grid = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)grid, items));
@@ -300,7 +301,7 @@ Plan launch_plan(const Plan *want, int device, uint64_t total_blocks, uint64_t t
     clamp(use.lru_b, tiles_of(total_slots, 32));          // also 4 cached blocks' masks a warp
     clamp(use.decode, tiles_of(total_slots, use.decode_tile));
     clamp(use.mc_emit, tiles_of(total_slots, use.emit_tile));
-    clamp(use.mc_scan, tiles_of(total_slots, kCountTile));
+    clamp(use.mc_scan, tiles_of(total_slots, single ? kThreads : kCountTile));
     return use;
 }
 
@@ -800,7 +801,7 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     // descriptors for the smallest tile of each scan (any plan may run)
     v->n_cull_desc = (g.nb + kMinCullTile - 1) / kMinCullTile;
     v->n_lru_desc = (v->cap + kScanTile - 1) / kScanTile;
-    const uint32_t n_mc_desc = (v->cap + kCountTile - 1) / kCountTile;   // candidates <= cap
+    const uint32_t n_mc_desc = (uint32_t)count_descs(v->cap);   // candidates <= cap
     const bool on_device = (o.flags & ISO_INPUT_ON_DEVICE) != 0;
     TRY(dalloc(v, &v->bits, words));
     if (!on_device) {                 // staging for host ranges (freed once the hulls exist)

@@ -93,7 +93,14 @@ struct Plan {
 constexpr int kThreads = 256;
 constexpr int kScanTile = 4096;          // entries per tile of the cache-update scans
 constexpr int kMinCullTile = 2048;       // smallest cull tile (sizes the cull descriptors)
-constexpr int kCountTile = 1024;         // candidates per tile of the count and offset scan
+constexpr int kCountTile = 1024;         // most candidates per tile of the count and offset scan
+constexpr uint32_t kMaxCountCtas = 2048; // most CTAs of its launch
+// its look-back descriptors for up to n candidates: tiles are smaller only
+// while there is no more than one per CTA
+inline uint64_t count_descs(uint64_t n) {
+    const uint64_t one = (n + kThreads - 1) / kThreads;
+    return (one < kMaxCountCtas ? one : kMaxCountCtas) + (n + kCountTile - 1) / kCountTile;
+}
 constexpr int kDefaultCullTile = 4096, kDefaultDecodeTile = 128, kDefaultCountTile = 32,
               kDefaultScanTile = 2048, kDefaultEmitTile = 32;
 

@@ -305,7 +305,10 @@ __device__ __forceinline__ uint32_t count_vertices(const unsigned long long (&m)
     return n;
 }
 
-// Tiles of kCountTile candidates: counts, the tile's prefixes from up to three
+// Tiles of at most kCountTile candidates, smaller ones while that gives more
+// CTAs a tile (the counting outweighs the look-backs: 11.8 -> 6.7 us for a
+// 64^3 sphere, 24.4 -> 18.9 for 397 x 301 x 259 noise, the same where every
+// CTA had a tile before): counts, the tile's prefixes from up to three
 // look-backs side by side, then the occupied candidates' ids and offsets;
 // the last tile of a volume writes the totals.  Every volume has at least
 // one item; its item 0 records how many look-back descriptors the volume
@@ -317,17 +320,27 @@ struct ScanSmem {
     unsigned long long cross[kR][kThreads];   // crossing cells
 };
 
+// rounds of 256 candidates a tile; batches share the CTAs among volumes and
+// take full tiles
+template <bool kOne>
+__device__ __forceinline__ uint32_t count_rounds(uint32_t n) {
+    constexpr uint32_t kMax = ScanSmem::kR;
+    return kOne ? min(kMax, max(1u, ceil_div(n, gridDim.x * kThreads))) : kMax;
+}
+
 template <bool kOne, bool kIdx>
 __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
-    constexpr int kR = ScanSmem::kR;
-    constexpr uint32_t kScanItems = kCountTile;
+    constexpr uint32_t kR = ScanSmem::kR;
     __shared__ ScanSmem sm;
     __shared__ uint32_t pre[kMaxBatch + 1];
     __shared__ uint32_t s_item;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t total = launch_prefix<kOne>(
-        L, [&](uint32_t v) { return max(1u, ceil_div(mc_candidates(vol_of<kOne>(L, v).s.ctl), kScanItems)); },
+        L, [&](uint32_t v) {
+            const uint32_t n = mc_candidates(vol_of<kOne>(L, v).s.ctl);
+            return max(1u, ceil_div(n, count_rounds<kOne>(n) * kThreads));
+        },
         pre);
     while (true) {
         const uint32_t x = next_item(&L.ctr[kLcScan], &s_item);
@@ -338,12 +351,13 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
         Ctl *c = s.ctl;
         const uint32_t tile = x - item_base<kOne>(pre, v);
         const uint32_t n = mc_candidates(c);
-        const uint32_t ntiles = ceil_div(n, kScanItems);
+        const uint32_t rounds = count_rounds<kOne>(n), tile_size = rounds * kThreads;
+        const uint32_t ntiles = ceil_div(n, tile_size);
         if (tile == 0 && threadIdx.x == 0) c->mc_tiles = ntiles;
         if (ntiles == 0) continue;                        // block-uniform
-        const uint32_t i0 = tile * kScanItems + threadIdx.x;
+        const uint32_t i0 = tile * tile_size + threadIdx.x;
 #pragma unroll 1
-        for (int r = 0; r < kR; r++) {
+        for (uint32_t r = 0; r < rounds; r++) {
             const uint32_t i = i0 + r * kThreads;
             uint32_t nt = 0, nv = 0;
             if (i < n) {
@@ -374,8 +388,8 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
         __syncthreads();
         // warp 0: triangle offsets; warp 1: occupied positions; warp 2: vertex offsets
         if (warp < (kIdx ? 3 : 2)) {
-            TileScan<kR> &ts = warp == 0 ? sm.tri : (warp == 1 ? sm.occ : sm.vtx);
-            const uint32_t tot = scan_tile_counts(ts);
+            TileScan<ScanSmem::kR> &ts = warp == 0 ? sm.tri : (warp == 1 ? sm.occ : sm.vtx);
+            const uint32_t tot = scan_tile_counts(ts, rounds);
             unsigned long long *desc = warp == 0 ? s.desc_mc : (warp == 1 ? s.desc_occ : s.desc_vtx);
             const unsigned long long excl = lookback_exclusive(desc, tile, tot, &c->status, kStatusTimeoutScan);
             if (lane == 0) {
@@ -389,7 +403,7 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
         }
         __syncthreads();
 #pragma unroll 1
-        for (int r = 0; r < kR; r++) {
+        for (uint32_t r = 0; r < rounds; r++) {
             const uint32_t i = i0 + r * kThreads;
             const uint32_t val = sm.val[r][threadIdx.x], nt = val & 511u, nv = (val >> 9) & 511u;
             const unsigned long long run = sm.tri.excl + sm.tri.cnt[r][warp] + (val >> 18);
@@ -696,6 +710,21 @@ __device__ __forceinline__ void emit_body(const Launch &L) {
     EmitSmem<kW, kIdx> &sm = *reinterpret_cast<EmitSmem<kW, kIdx> *>(smem_raw);
     uint32_t *pre = reinterpret_cast<uint32_t *>(&sm + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // all failure bits are final before this kernel starts
+    const uint32_t total = launch_prefix<kOne>(
+        L, [&](uint32_t v) {
+            const Ctl *c = vol_of<kOne>(L, v).s.ctl;
+            return (c->status & (kStatusBudget | kStatusAnyTimeout | kStatusSkip)) ? 0u : ceil_div(c->n_occ, kBPW);
+        },
+        pre);
+    // one tile's samples are copied in while the tile before it is written;
+    // its slots were loaded a tile earlier, and its block ids two (the first
+    // ones before the tables, so that their latencies pass together)
+    const TileWalk<kOne> walk{L, pre, total};
+    const uint32_t stride = gridDim.x * kW;
+    uint32_t t = blockIdx.x * kW + warp;
+    const uint32_t b0 = walk.block_at(t);
+    uint32_t b1 = walk.block_at(t + stride), b2 = walk.block_at(t + 2 * stride);
     const EmitTables *tables = vol_of<kOne>(L, 0).s.tables;
     auto fill = [&](void *dst, const void *src, uint32_t bytes) {
         for (uint32_t i = threadIdx.x; i < bytes / 16; i += 32 * kW)
@@ -707,34 +736,15 @@ __device__ __forceinline__ void emit_body(const Launch &L) {
     fill(sm.tab.corner, tables->corner, sizeof(tables->corner));
     if (!kIdx) fill(sm.tab.coord, tables->coord, sizeof(tables->coord));
     if (kIdx) load_window_rows(sm.win);
-    // all failure bits are final before this kernel starts
-    const uint32_t total = launch_prefix<kOne>(
-        L, [&](uint32_t v) {
-            const Ctl *c = vol_of<kOne>(L, v).s.ctl;
-            return (c->status & (kStatusBudget | kStatusAnyTimeout | kStatusSkip)) ? 0u : ceil_div(c->n_occ, kBPW);
-        },
-        pre);
+    const int32_t s0 = walk.slot_at(t, b0);
+    int32_t s1 = walk.slot_at(t + stride, b1);
     __syncthreads();                                      // the tables
+    if (t >= total) return;
     LaneConst lc;
     lc.init(lane);
     EmitWarp<kIdx> &wt = sm.w[warp];
-    const TileWalk<kOne> walk{L, pre, total};
-    const uint32_t stride = gridDim.x * kW;
-    uint32_t t = blockIdx.x * kW + warp;
-    if (t >= total) return;
-    // one tile's samples are copied in while the tile before it is written;
-    // its slots were loaded a tile earlier, and its block ids two
-    uint32_t b1, b2;
-    int32_t s1;
-    {
-        const uint32_t b0 = walk.block_at(t);
-        b1 = walk.block_at(t + stride);
-        b2 = walk.block_at(t + 2 * stride);
-        const int32_t s0 = walk.slot_at(t, b0);
-        s1 = walk.slot_at(t + stride, b1);
-        stage_tile<kOne, kIdx>(walk, t, b0, s0, 0, wt, lc);
-        cp_async_commit();
-    }
+    stage_tile<kOne, kIdx>(walk, t, b0, s0, 0, wt, lc);
+    cp_async_commit();
     const uint32_t lt = (1u << lane) - 1u;
     for (int buf = 0; t < total; t += stride, buf ^= 1) {
         if (t + stride < total) stage_tile<kOne, kIdx>(walk, t + stride, b1, s1, buf ^ 1, wt, lc);

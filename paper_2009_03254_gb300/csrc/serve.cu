@@ -861,7 +861,7 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
     sv->tri_bytes = o.vertex_format == ISO_VERTEX_PACKED ? 24 : 48;
     const size_t cand = std::min<size_t>(v->cap, v->g.nb);       // candidates of an admitted tick <= cap
     sv->cand_cap = (uint32_t)cand;
-    const size_t n_mc_desc = (cand + kCountTile - 1) / kCountTile;
+    const size_t n_mc_desc = count_descs(cand);
     int rc = ISO_OK;
 #define TRY(x)                                   \
     do {                                         \

@@ -26,16 +26,16 @@ struct TileScan {
 
 // warp 0: turn ts.cnt into exclusive offsets (packed 16-bit fields add
 // without carries: a tile holds at most 4096 entries) and return the
-// tile's packed total in every lane
+// tile's packed total in every lane; rounds from `rounds` on count as empty
 template <int kR>
-__device__ __forceinline__ uint32_t scan_tile_counts(TileScan<kR> &ts) {
+__device__ __forceinline__ uint32_t scan_tile_counts(TileScan<kR> &ts, uint32_t rounds = kR) {
     constexpr int kPer = kR * 8 / 32;
     const int lane = threadIdx.x & 31;
     uint32_t *flat = &ts.cnt[0][0] + kPer * lane;
     uint32_t v[kPer], sum = 0;
 #pragma unroll
     for (int k = 0; k < kPer; k++) {
-        v[k] = flat[k];
+        v[k] = (uint32_t)(kPer * lane + k) < 8u * rounds ? flat[k] : 0u;
         sum += v[k];
     }
     uint32_t incl = sum;
