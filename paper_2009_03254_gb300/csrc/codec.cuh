@@ -91,26 +91,33 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
     return v;
 }
+__device__ __forceinline__ void lds_u64(uint32_t a, uint32_t &lo, uint32_t &hi) {
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(lo), "=r"(hi) : "r"(a));
+}
 __device__ __forceinline__ void sts_u64(uint32_t a, uint32_t lo, uint32_t hi) {
     asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(lo), "r"(hi));
 }
 
-// Bit windows over a staged block at shared address `w` (32-bit words).
-struct StagedBits {
-    uint32_t w;
-    // 32 bits starting at bit pos
-    __device__ __forceinline__ uint32_t win32(uint32_t pos) const {
-        const uint32_t a = w + ((pos >> 5) << 2);
-        return __funnelshift_r(lds_u32(a), lds_u32(a + 4), pos & 31u);
-    }
-    // 64 bits starting at bit pos, as two halves
-    __device__ __forceinline__ void win64(uint32_t pos, uint32_t &lo, uint32_t &hi) const {
-        const uint32_t a = w + ((pos >> 5) << 2), sh = pos & 31u;
-        const uint32_t x = lds_u32(a), y = lds_u32(a + 4), z = lds_u32(a + 8);
-        lo = __funnelshift_r(x, y, sh);
-        hi = __funnelshift_r(y, z, sh);
-    }
-};
+// The mask of the lowest n bits (n > 32: all of them)
+__device__ __forceinline__ uint32_t bit_mask(uint32_t n) {
+    uint32_t r;
+    asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(r) : "r"(n));
+    return r;
+}
+
+// Bit windows over staged blocks.  A position is a bit's place in shared
+// memory (8 x its byte's shared address + its place in the byte), so a
+// window needs no base address; staged blocks start at whole words.
+__device__ __forceinline__ uint32_t win32(uint32_t pos) {     // the 32 bits from pos on
+    const uint32_t a = (pos >> 3) & ~3u;
+    return __funnelshift_r(lds_u32(a), lds_u32(a + 4), pos);
+}
+__device__ __forceinline__ void win64(uint32_t pos, uint32_t &lo, uint32_t &hi) {   // 64 bits, as two halves
+    const uint32_t a = (pos >> 3) & ~3u;
+    const uint32_t x = lds_u32(a), y = lds_u32(a + 4), z = lds_u32(a + 8);
+    lo = __funnelshift_r(x, y, pos);
+    hi = __funnelshift_r(y, z, pos);
+}
 
 // inverse of one two-level S-transform step on (ll, hh, h0, h1) -> (a, b, c, d), two's-complement words
 // held as uint32 (wrap-around arithmetic)
@@ -158,14 +165,16 @@ __device__ __forceinline__ void scale_block(const uint32_t (&q)[64], int e, floa
 // group test, 1: it is a run bit) and a byte of the stream, the entry holds
 // what reading those bits one by one does --
 //   bits 0-7    the run bits met, in order (coefficient n, n + 1, ...)
-//   bits 8-11   how many run bits that is
-//   bits 12-15  bits consumed (8, or fewer when a 0 test ends the plane)
-//   bit 16      a 0 test ended the plane
-//   bit 17      the state after the consumed bits
+//   bit  10     the state after the consumed bits (its place in the entry's
+//               byte offset in the table: state * 1024 + byte * 4)
+//   bit  15     a 0 test ended the plane
+//   bits 16-23  how many run bits that is
+//   bits 24-31  bits consumed (8, or fewer when a 0 test ends the plane)
 // A group test is a 1 followed by the run of later coefficients' bits up to
 // and including the next one, or the 0 that ends the plane, so without the
 // budget and coefficient 63's implied one the table step is exactly eight
 // steps of that rule.  The decoder checks the two exceptions around it.
+constexpr uint32_t kGroupState = 1u << 10, kGroupEnd = 1u << 15;
 __host__ __device__ constexpr uint32_t group_step_entry(uint32_t state, uint32_t byte) {
     uint32_t runbits = 0, count = 0, consumed = 8, ended = 0;
     for (uint32_t i = 0; i < 8; i++) {
@@ -183,7 +192,7 @@ __host__ __device__ constexpr uint32_t group_step_entry(uint32_t state, uint32_t
             if (bit) state = 0;
         }
     }
-    return runbits | (count << 8) | (consumed << 12) | (ended << 16) | (state << 17);
+    return runbits | (state ? kGroupState : 0u) | (ended ? kGroupEnd : 0u) | (count << 16) | (consumed << 24);
 }
 
 constexpr uint32_t kGroupTableEntries = 512;
@@ -193,119 +202,90 @@ __device__ __forceinline__ void load_group_table(uint32_t *tab) {
     for (uint32_t i = threadIdx.x; i < kGroupTableEntries; i += blockDim.x) tab[i] = group_step_entry(i >> 8, i & 255u);
 }
 
-// One group-test event read bit by bit, with every rule: from state 0 a
-// test bit (a 0 ends the plane), then (or from state 1) the rest of a run,
-// at most 63 - n run bits (coefficient 63's one is implied) and no bit past
-// the budget.  Updates pos, n, the plane (xlo, xhi) and `ended`.
-__device__ __forceinline__ void group_event_exact(const StagedBits &st, uint32_t end, uint32_t &pos, uint32_t &n,
-                                                  uint32_t &xlo, uint32_t &xhi, uint32_t state, bool &ended) {
-    if (state == 0) {
-        const uint32_t g = st.win32(pos);
-        pos += 1;
-        if (!(g & 1u)) {
-            ended = true;
-            return;
-        }
-    }
-    const uint32_t lim = 63u - n;                // run bits that may be sent
-    const uint32_t scan = min(lim, end - min(end, pos));   // of which the budget holds
-    uint32_t z = 64u;                            // zeros before the run's one (64: none)
-    for (uint32_t off = 0; off < scan; off += 32) {
-        uint32_t w = st.win32(pos + off);
-        if (scan - off < 32u) w &= (1u << (scan - off)) - 1u;
-        if (w) {
-            z = off + (uint32_t)__ffs(w) - 1u;
-            break;
-        }
-    }
-    if (z < 64u) {                               // z zeros, then coefficient n + z's one
-        pos += z + 1;
-        n += z;
-        if (n < 32u) xlo |= 1u << n;
-        else xhi |= 1u << (n - 32u);
-        n += 1;
-    } else if (scan == lim) {                    // zeros up to coefficient 62: 63's one is implied
-        pos += lim;
-        xhi |= 1u << 31;
-        n = 64;
-    } else {
-        pos = end;                               // the budget ran out inside the run
-    }
-}
-
-// Parse the bit planes of a staged block of `rate` words: plane k (most
-// significant first) goes to shared address planes + k * stride as a 64-bit
-// word whose bit i belongs to the i-th coded coefficient.  A zero block (flag bit 0: the
-// rest is not read) has all planes zero.  Sets emax.
+// Parse the bit planes of a staged block of `rate` words at shared address
+// `words`: plane k (most significant first) goes to shared address
+// planes + k * stride as a 64-bit word whose bit i belongs to the i-th coded
+// coefficient.  A zero block (flag bit 0: the rest is not read) has all
+// planes zero.  Sets emax.
 //
 // The lanes of a warp parse different blocks.  One loop of uniform steps
 // keeps them together: a step takes the plane's verbatim bits when it opens
-// a plane, then up to kSteps table steps of its group tests, all
-// predicated; a lane whose block is done sits the remaining steps out.
+// a plane, then up to kSteps table steps of its group tests out of one
+// 32-bit window, all predicated; a lane whose block is done sits the
+// remaining steps out.  Where a table step would reach coefficient 63, whose
+// one is implied, a step takes one group test and its run instead.  Bits
+// past the budget read as zero: the staged block is followed by a zero word,
+// and a window is used only as far as 9 bits past the budget's last.
 // Once every coefficient is reached (n = 64) a plane is its 64 verbatim
 // bits, which a short loop of its own copies.
 template <int kSteps = 2>
-__device__ __forceinline__ void parse_planes(const StagedBits &st, uint32_t rate, uint32_t tab, uint32_t planes,
+__device__ __forceinline__ void parse_planes(uint32_t words, uint32_t rate, uint32_t tab, uint32_t planes,
                                              uint32_t stride, int &emax) {
-    const uint32_t head = lds_u32(st.w);
+    static_assert(kSteps <= 3, "a window of 30 bits holds three steps of 9");
+    const uint32_t head = lds_u32(words);
     emax = (int)((head >> 1) & 0xFFu) - 127;
-    const uint32_t end = (head & 1u) ? rate * 64u : 0u;
-    uint32_t pos = 9, n = 0;               // n: coefficients reached by the group tests
+    uint32_t pos = words * 8u;
+    const uint32_t end = pos + ((head & 1u) ? rate * 64u : 0u);
+    pos += 9;
+    uint32_t n = 0;                        // coefficients reached by the group tests
     int k = 31;                            // plane, most significant first
-    if (end) {
+    if (head & 1u) {
         // Until a coefficient is reached, a plane has no verbatim bits and a
         // 0 group test ends it: each 0 bit here is a whole empty plane
         // (end - pos >= 55 at every rate, so the window is inside the budget).
-        const uint32_t win = st.win32(pos);
+        const uint32_t win = win32(pos);
         const uint32_t z = win ? (uint32_t)__ffs(win) - 1u : 32u;
         for (uint32_t j = 0; j < z; j++) sts_u64(planes + (31u - j) * stride, 0u, 0u);
         k -= (int)z;
         pos += z;
     }
-    uint32_t xlo = 0u, xhi = 0u, state = 0u;
-    bool opening = true, exact = false;    // exact: the next event is read bit by bit
+    uint32_t xlo = 0u, xhi = 0u, at = tab; // at: the state's half of the table
+    bool opening = true;
     while (k >= 0 && pos < end && n < 64u) {
         if (opening) {                     // the verbatim bits of the n coefficients reached so far
             const uint32_t m = min(n, end - pos);
             uint32_t wlo, whi;
-            st.win64(pos, wlo, whi);
-            xlo = m >= 32u ? wlo : (wlo & ((1u << m) - 1u));
-            xhi = m > 32u ? (whi & ((1u << (m - 32u)) - 1u)) : 0u;   // m < 64 here
+            win64(pos, wlo, whi);
+            xlo = wlo & bit_mask(m);
+            xhi = whi & bit_mask(max(m, 32u) - 32u);
             pos += m;
-            state = 0u;
+            at = tab;
         }
         bool done = pos >= end;
-        if (exact && !done) {              // the run reaches coefficient 63 inside the next byte
-            bool ended = false;
-            group_event_exact(st, end, pos, n, xlo, xhi, state, ended);
-            state = 0u;
-            exact = false;
-            done = ended || pos >= end || n >= 64u;
-        }
+        uint32_t w = win32(pos) << 2;      // (at pos == end: the zero word, and not used)
 #pragma unroll
         for (int t = 0; t < kSteps; t++) {
-            if (done || exact) continue;
-            // bits past the budget read as zero: the staged block is followed
-            // by a zero pad word, and a step reads at most 8 bits on
-            const uint32_t byte = st.win32(pos) & 0xFFu;
-            const uint32_t e = lds_u32(tab + (((state << 8) | byte) << 2));
-            const uint32_t cnt = (e >> 8) & 15u;
-            if (n + cnt > 63u) {           // a run bit for coefficient 63 or later: not a table step
-                exact = true;
-                continue;
+            if (done) continue;
+            const uint32_t e = lds_u32(at + (w & 0x3FCu));
+            const uint32_t cnt = __byte_perm(e, 0u, 0x4442);
+            if (n + cnt <= 62u) {
+                const uint64_t bits = (uint64_t)(e & 0xFFu) << n;
+                xlo |= (uint32_t)bits;
+                xhi |= (uint32_t)(bits >> 32);
+                n += cnt;
+                pos += e >> 24;
+                at = tab + (e & kGroupState);
+                w >>= 8;
+                done = (e & kGroupEnd) != 0u || pos >= end;
+            } else {                       // one event; here n >= 55
+                const bool test = at == tab;
+                const bool ended = test && !(w & 4u);
+                uint32_t used = test ? 1u : 0u;
+                if (!ended) {
+                    const uint32_t lim = 63u - n, run = w >> (2u + used);       // run bits that may be sent
+                    const uint32_t z = (uint32_t)__ffs(run | (1u << lim)) - 1u;  // zeros before the run's one
+                    const bool implied = z == lim;                              // none sent: 63's one is implied
+                    xhi |= 1u << (n + z - 32u);
+                    n += z + 1u;
+                    used += implied ? z : z + 1u;
+                    // the budget ran out inside the run: no one was read
+                    if (pos + used > end) xhi &= 0x7FFFFFFFu;
+                }
+                pos += used;
+                at = tab;
+                w >>= used;
+                done = ended || pos >= end || n >= 64u;
             }
-            const uint64_t bits = (uint64_t)(e & 0xFFu) << n;
-            xlo |= (uint32_t)bits;
-            xhi |= (uint32_t)(bits >> 32);
-            n += cnt;
-            pos += (e >> 12) & 15u;
-            state = (e >> 17) & 1u;
-            if (state && n == 63u && pos <= end) {   // the run reached coefficient 63: its one is implied
-                xhi |= 1u << 31;
-                n = 64;
-                state = 0u;
-            }
-            done = ((e >> 16) & 1u) != 0u || pos >= end || n >= 64u;
         }
         if (done) {
             sts_u64(planes + (uint32_t)k * stride, xlo, xhi);
@@ -313,19 +293,45 @@ __device__ __forceinline__ void parse_planes(const StagedBits &st, uint32_t rate
         }
         opening = done;
     }
-    // every coefficient reached: each remaining plane is the next 64 bits
-    for (; k >= 0 && pos < end; k--) {
-        const uint32_t m = min(64u, end - pos);
-        uint32_t wlo, whi;
-        st.win64(pos, wlo, whi);
-        if (m < 64u) {
-            wlo = m >= 32u ? wlo : (wlo & ((1u << m) - 1u));
-            whi = m > 32u ? (whi & ((1u << (m - 32u)) - 1u)) : 0u;
+    // every coefficient reached: each remaining plane is the next 64 bits,
+    // read two words a plane
+    uint32_t column = planes + (uint32_t)k * stride;        // (k < 0: not used)
+    if (k >= 0 && pos < end) {
+        uint32_t a = (pos >> 3) & ~3u, x = lds_u32(a);
+        for (; k >= 0 && pos + 64u <= end; k--, pos += 64u, a += 8, column -= stride) {
+            const uint32_t y = lds_u32(a + 4), z = lds_u32(a + 8);
+            sts_u64(column, __funnelshift_r(x, y, pos), __funnelshift_r(y, z, pos));
+            x = z;
         }
-        sts_u64(planes + (uint32_t)k * stride, wlo, whi);
-        pos += m;
+        if (k >= 0 && pos < end) {         // the budget ends inside this plane
+            const uint32_t m = end - pos;
+            uint32_t wlo, whi;
+            win64(pos, wlo, whi);
+            sts_u64(column, wlo & bit_mask(m), whi & bit_mask(max(m, 32u) - 32u));
+            k--;
+            column -= stride;
+        }
     }
-    for (; k >= 0; k--) sts_u64(planes + (uint32_t)k * stride, 0u, 0u);
+    for (; k >= 3; k -= 4, column -= 4u * stride) {
+        sts_u64(column, 0u, 0u);
+        sts_u64(column - stride, 0u, 0u);
+        sts_u64(column - 2u * stride, 0u, 0u);
+        sts_u64(column - 3u * stride, 0u, 0u);
+    }
+    for (; k >= 0; k--, column -= stride) sts_u64(column, 0u, 0u);
+}
+
+// 32 words of bit planes to the coefficients' two's complement: a transpose
+// whose odd planes (the negabinary digits of negative weight) are inverted on
+// the way in, then one subtraction each
+__device__ __forceinline__ void coefficients(uint32_t (&a)[32]) {
+    transpose_round<1, true>(a);
+    transpose_round<2>(a);
+    transpose_round<4>(a);
+    transpose_round<8>(a);
+    transpose_round<16>(a);
+#pragma unroll
+    for (int p = 0; p < 32; p++) a[p] -= kNegaMask;
 }
 
 // The second half of decoding a block, after parse_planes has written its
@@ -336,17 +342,18 @@ __device__ __forceinline__ void parse_planes(const StagedBits &st, uint32_t rate
 __device__ __forceinline__ void finish_planes(uint32_t pa, uint32_t ps, int emax, float (&out)[64]) {
     constexpr CodingOrder order = make_coding_order();
     uint32_t q[64];
-    uint32_t a[32];
+    {
+        uint32_t a[32], b[32];             // coded coefficients 0..31 and 32..63
 #pragma unroll
-    for (int j = 0; j < 32; j++) a[j] = lds_u32(pa + (uint32_t)j * ps);
-    transpose32(a);                        // a[p] = negabinary coefficient p (coded order)
+        for (int j = 0; j < 32; j++) lds_u64(pa + (uint32_t)j * ps, a[j], b[j]);
+        coefficients(a);
+        coefficients(b);
 #pragma unroll
-    for (int p = 0; p < 32; p++) q[order.perm[p]] = (a[p] ^ kNegaMask) - kNegaMask;
-#pragma unroll
-    for (int j = 0; j < 32; j++) a[j] = lds_u32(pa + (uint32_t)j * ps + 4u);
-    transpose32(a);                        // a[p] = coefficient 32 + p
-#pragma unroll
-    for (int p = 0; p < 32; p++) q[order.perm[32 + p]] = (a[p] ^ kNegaMask) - kNegaMask;
+        for (int p = 0; p < 32; p++) {
+            q[order.perm[p]] = a[p];
+            q[order.perm[32 + p]] = b[p];
+        }
+    }
 #pragma unroll
     for (int i = 0; i < 16; i++) inv_lift4u(q[i], q[i + 16], q[i + 32], q[i + 48]);             // z
 #pragma unroll
@@ -365,7 +372,7 @@ __device__ __forceinline__ void decode_staged(const uint32_t *staged, uint32_t r
                                               float (&out)[64], uint64_t *planes, uint32_t stride) {
     int emax = 0;
     const uint32_t pa = smem_u32(planes), ps = stride * 8u;
-    parse_planes(StagedBits{smem_u32(staged)}, rate, smem_u32(tab), pa, ps, emax);
+    parse_planes(smem_u32(staged), rate, smem_u32(tab), pa, ps, emax);
     finish_planes(pa, ps, emax, out);
 }
 
@@ -425,6 +432,15 @@ struct StagedWriter {
     }
 };
 
+// the inverse of `coefficients` but for the addition
+__device__ __forceinline__ void digit_planes(uint32_t (&a)[32]) {
+    transpose_round<16>(a);
+    transpose_round<8>(a);
+    transpose_round<4>(a);
+    transpose_round<2>(a);
+    transpose_round<1, false, true>(a);
+}
+
 // Turn v[64] into bit planes at `planes` + k * stride (plane k, shared-window
 // address) and an exponent; false: the block is zero (no planes written).
 __device__ __forceinline__ bool make_planes(const float (&v)[64], uint32_t planes, uint32_t stride, int &emax) {
@@ -460,11 +476,11 @@ __device__ __forceinline__ bool make_planes(const float (&v)[64], uint32_t plane
     uint32_t lo[32], hi[32];
 #pragma unroll
     for (int p = 0; p < 64; p++) {
-        const uint32_t u = ((uint32_t)q[order.perm[p]] + kNegaMask) ^ kNegaMask;
+        const uint32_t u = (uint32_t)q[order.perm[p]] + kNegaMask;   // (its odd digits are inverted as planes)
         if (p < 32) lo[p] = u; else hi[p - 32] = u;
     }
-    transpose32(lo);                       // lo[k] = plane k of coefficients 0-31
-    transpose32(hi);
+    digit_planes(lo);                      // lo[k] = plane k of coefficients 0-31
+    digit_planes(hi);
 #pragma unroll
     for (int k = 0; k < 32; k++) sts_u64(planes + (uint32_t)k * stride, lo[k], hi[k]);
     return true;
@@ -487,7 +503,7 @@ __device__ __forceinline__ void code_planes(StagedWriter &out, uint32_t rate, ui
     while (k >= 0 && pos < end) {
         if (opening) {
             uint32_t xlo, xhi;
-            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(xlo), "=r"(xhi) : "r"(planes + (uint32_t)k * stride));
+            lds_u64(planes + (uint32_t)k * stride, xlo, xhi);
             x = ((uint64_t)xhi << 32) | xlo;
             const uint64_t low = low_mask(n);
             out.put(xlo & (uint32_t)low, min(n, 32u));

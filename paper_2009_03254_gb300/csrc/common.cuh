@@ -256,44 +256,40 @@ __device__ __forceinline__ float edge_fraction(float iso, float vlo, float vhi) 
 
 // ---------------------------------------------------------------- bit tools
 
-// (x & ~m) | (y & m) as one three-input logic instruction
-__device__ __forceinline__ uint32_t select_bits(uint32_t x, uint32_t y, uint32_t m) {
+// one three-input logic instruction (kLut: a = 0xF0, b = 0xCC, c = 0xAA)
+template <int kLut>
+__device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
     uint32_t r;
-    asm("lop3.b32 %0, %1, %2, %3, 0xD8;" : "=r"(r) : "r"(x), "r"(y), "r"(m));   // LUT of (c ? b : a): 0xD8
+    asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(r) : "r"(a), "r"(b), "r"(c), "n"(kLut));
     return r;
 }
+constexpr int kLutSelect = 0xD8;          // c ? b : a
 
-// In-place transpose of a 32x32 bit matrix held in 32 words: afterwards
-// bit j of a[i] is what bit i of a[j] was.  Five rounds of swapping the
-// off-diagonal sub-blocks (16x16, 8x8, ..., 1x1); the 16- and 8-bit rounds
-// move whole bytes, one byte permute per word.
-__device__ __forceinline__ void transpose32(uint32_t (&a)[32]) {
+// Rounds of the in-place transpose of a 32x32 bit matrix held in 32 words
+// (afterwards bit j of a[i] is what bit i of a[j] was): each swaps the
+// off-diagonal kS x kS sub-blocks, and they may run in any order.  The 16-
+// and 8-bit rounds move whole bytes, one byte permute a word; the others
+// take one shift and one three-input select a word: the bits of a[j] under
+// the mask's high half against those of a[j + kS] under its low half.
+// kOddIn / kOddOut (kS == 1): the odd words are inverted first / last, in the
+// selects' tables.
+template <int kS, bool kOddIn = false, bool kOddOut = false>
+__device__ __forceinline__ void transpose_round(uint32_t (&a)[32]) {
+    static_assert(kS == 1 || !(kOddIn || kOddOut), "the odd words are told apart in the round of single bits");
+    constexpr uint32_t m = kS == 4 ? 0x0F0F0F0Fu : (kS == 2 ? 0x33333333u : 0x55555555u), mh = ~m;
 #pragma unroll
-    for (int j = 0; j < 16; j++) {        // (a, b) -> (a.lo16 | b.lo16 << 16, a.hi16 | b.hi16 << 16)
-        const uint32_t x = a[j], y = a[j + 16];
-        a[j] = __byte_perm(x, y, 0x5410);
-        a[j + 16] = __byte_perm(x, y, 0x7632);
-    }
-#pragma unroll
-    for (int j = 0; j < 32; j++) {        // bytes (a0 b0 a2 b2), (a1 b1 a3 b3)
-        if (j & 8) continue;
-        const uint32_t x = a[j], y = a[j + 8];
-        a[j] = __byte_perm(x, y, 0x6240);
-        a[j + 8] = __byte_perm(x, y, 0x7351);
-    }
-    const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-    for (int r = 2; r < 5; r++) {
-        const int s = 16 >> r;
-        const uint32_t m = masks[r], mh = m << s;
-#pragma unroll
-        for (int j = 0; j < 32; j++) {
-            if (j & s) continue;
-            // swap the bits of a[j] under mh with those of a[j + s] under m,
-            // each word as one shift and one three-input select
-            const uint32_t x = a[j], y = a[j + s];
-            a[j] = select_bits(x, y << s, mh);
-            a[j + s] = select_bits(y, x >> s, m);
+    for (int j = 0; j < 32; j++) {
+        if (j & kS) continue;
+        const uint32_t x = a[j], y = a[j + kS];
+        if (kS == 16) {                   // (x.lo16 | y.lo16 << 16, x.hi16 | y.hi16 << 16)
+            a[j] = __byte_perm(x, y, 0x5410);
+            a[j + kS] = __byte_perm(x, y, 0x7632);
+        } else if (kS == 8) {             // bytes (x0 y0 x2 y2), (x1 y1 x3 y3)
+            a[j] = __byte_perm(x, y, 0x6240);
+            a[j + kS] = __byte_perm(x, y, 0x7351);
+        } else {
+            a[j] = lop3<kOddIn ? 0x72 : kLutSelect>(x, y << kS, mh);                     // c ? ~b : a
+            a[j + kS] = lop3<kOddIn ? 0x8D : (kOddOut ? 0x27 : kLutSelect)>(y, x >> kS, m);   // c ? b : ~a; ~(c ? b : a)
         }
     }
 }

@@ -549,12 +549,14 @@ __global__ void __launch_bounds__(kDecodeThreads, 768 / kDecodeThreads) decode_n
 #pragma unroll
         for (int i = 0; i < 16; i++) dst[i] = make_float4(val[4 * i], val[4 * i + 1], val[4 * i + 2], val[4 * i + 3]);
         if (s.bmask) {                                // the block's below mask, while its samples are here
-            const float iso = c->params.iso;
+            // the sign bits of sample - iso (a NaN's is clear; -0 where iso is 0:
+            // -0 - 0 would be -0, which is not below)
+            const float iso = c->params.iso, sub = iso == 0.0f ? -0.0f : iso;
             uint32_t lo = 0, hi = 0;
 #pragma unroll
-            for (int i = 0; i < 32; i++) {
-                if (val[i] < iso) lo |= 1u << i;
-                if (val[32 + i] < iso) hi |= 1u << i;
+            for (int i = 31; i >= 0; i--) {
+                lo = __funnelshift_l(__float_as_uint(__fsub_rn(val[i], sub)), lo, 1);
+                hi = __funnelshift_l(__float_as_uint(__fsub_rn(val[32 + i], sub)), hi, 1);
             }
             s.bmask[slot] = ((unsigned long long)hi << 32) | lo;
         }
