@@ -106,12 +106,9 @@ __global__ void __launch_bounds__(kCodecThreads, 5) decode_list_kernel(const uin
         const uint64_t i = i0 + lane;
         const bool have = i < n;
         stage_blocks(bits, rate, have ? ids[i] : 0u, have, sm.stage);
-        if (!have) continue;
-        float v[64];
+        float v[64];                       // (a lane without a block decodes a zero one)
         decode_staged(sm.stage + lane * (2u * rate + 1u), rate, sm.tab, v, sm.planes + threadIdx.x, blockDim.x);
-        float4 *dst = reinterpret_cast<float4 *>(out + i * 64);
-#pragma unroll
-        for (int q = 0; q < 16; q++) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        store_blocks(out + i0 * 64, lane, __ballot_sync(0xffffffffu, have), v, sm.planes + threadIdx.x, blockDim.x);
     }
 }
 
@@ -130,6 +127,8 @@ __global__ void __launch_bounds__(kCodecThreads, 5) decode_volume_kernel(const u
         const uint32_t b = b0 + lane;
         const bool have = b < g.nb;
         stage_blocks(bits, g.rate, b, have, sm.stage);
+        const uint64_t ahead = (uint64_t)b + gridDim.x * blockDim.x;       // its latency passes during this decode
+        if (ahead < g.nb) prefetch_block(bits, g.rate, (uint32_t)ahead);
         if (!have) continue;
         uint32_t bx, by, bz;
         block_coords(g, b, bx, by, bz);

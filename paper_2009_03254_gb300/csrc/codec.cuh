@@ -82,6 +82,12 @@ __device__ __forceinline__ void stage_blocks(const uint64_t *__restrict__ bits, 
     __syncwarp();
 }
 
+// fetch block id's words into L2 (a later stage_blocks call reads them)
+__device__ __forceinline__ void prefetch_block(const uint64_t *__restrict__ bits, uint32_t rate, uint32_t id) {
+    const uint64_t *p = bits + (size_t)id * rate;
+    for (uint32_t w = 0; w < rate; w += 16) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + w));
+}
+
 // Shared-memory accesses by 32-bit shared-window address (the decoder's
 // loops address the staging area and plane columns this way, so every
 // access is a plain shared-memory load or store).
@@ -374,6 +380,35 @@ __device__ __forceinline__ void decode_staged(const uint32_t *staged, uint32_t r
     const uint32_t pa = smem_u32(planes), ps = stride * 8u;
     parse_planes(smem_u32(staged), rate, smem_u32(tab), pa, ps, emax);
     finish_planes(pa, ps, emax, out);
+}
+
+// Write a warp's decoded blocks, 256 contiguous bytes each: lane i's v[64] to
+// row `to` of 64 floats at `base` if bit i of `have` is set.  A lane's own
+// 16-byte stores would touch 32 lines an instruction and half of each
+// 32-byte sector, so the blocks pass through the warp's plane columns (plane
+// k of its lanes is 256 bytes; the planes are used up), 16-byte pieces
+// swizzled against bank conflicts, and every store writes two whole blocks.
+// Called by all 32 lanes.
+__device__ __forceinline__ void store_blocks(float *base, uint32_t to, uint32_t have, const float (&v)[64],
+                                             uint64_t *planes, uint32_t stride) {
+    const uint32_t lane = threadIdx.x & 31u, rows = smem_u32(planes) - lane * 8u, ps = stride * 8u;
+    __syncwarp();                          // every lane has read its planes
+#pragma unroll
+    for (uint32_t c = 0; c < 16; c++)
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(rows + lane * ps + ((c ^ (lane & 15u)) << 4)),
+                     "f"(v[4 * c]), "f"(v[4 * c + 1]), "f"(v[4 * c + 2]), "f"(v[4 * c + 3]));
+    __syncwarp();
+    const uint32_t half = lane >> 4, piece = lane & 15u;
+#pragma unroll
+    for (uint32_t i = 0; i < 16; i++) {
+        const uint32_t b = 2 * i + half;
+        float4 d;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(d.x), "=f"(d.y), "=f"(d.z), "=f"(d.w)
+                     : "r"(rows + b * ps + ((piece ^ (b & 15u)) << 4)));
+        const uint32_t row = __shfl_sync(0xffffffffu, to, (int)b);
+        if ((have >> b) & 1u) *reinterpret_cast<float4 *>(base + (size_t)row * 64 + 4 * piece) = d;
+    }
 }
 
 // Dynamic shared memory of a decoding kernel of `threads` threads: the

@@ -513,42 +513,54 @@ __global__ void __launch_bounds__(kDecodeThreads, 768 / kDecodeThreads) decode_n
     __shared__ uint32_t pre[kMaxBatch + 1];
     __shared__ TileScan<kRounds> ts;                  // lru_b's work
     __shared__ uint32_t slot_x;
-    const uint32_t warp = threadIdx.x >> 5;
     const DecodeSmem sm = decode_smem_layout(dsm, kDecodeThreads, kOne ? L.one.g.rate : L.max_rate);
     load_group_table(sm.tab);
     __syncthreads();
     const uint32_t total = launch_prefix<kOne>(
         L, [&](uint32_t v) { return max(1u, ceil_div(vol_of<kOne>(L, v).s.ctl->n_assign, kDecodeThreads)); },
         pre);
+    // a chunk's block ids and slots are loaded, and its words fetched into L2,
+    // while the chunk before it is decoded
+    uint32_t b = 0, slot = 0;
+    bool have = false;
+    auto load_ids = [&](uint32_t x) {
+        have = false;
+        if (x >= total) return;
+        const uint32_t v = item_vol<kOne>(pre, L.n, x);
+        const DevState &s = vol_of<kOne>(L, v).s;
+        const uint32_t r = (x - item_base<kOne>(pre, v)) * kDecodeThreads + threadIdx.x;
+        have = r < s.ctl->n_assign;
+        b = have ? s.inew[r] : 0u;
+        slot = have ? s.newslot[r] : 0u;
+    };
+    load_ids(blockIdx.x);
     for (uint32_t x = blockIdx.x; x < total; x += gridDim.x) {
         const uint32_t v = item_vol<kOne>(pre, L.n, x);
         const DevState &s = vol_of<kOne>(L, v).s;
         Ctl *c = s.ctl;
         const uint32_t chunk = x - item_base<kOne>(pre, v);
-        if (c->status & kStatusAnyTimeout) continue;  // block-uniform: no barrier in this loop
-        if (chunk == 0 && threadIdx.x == 0) {         // commit the cache update
+        const bool skip = (c->status & kStatusAnyTimeout) != 0;   // block-uniform: no barrier in this loop
+        if (chunk == 0 && threadIdx.x == 0 && !skip) {            // commit the cache update
             c->S = c->S_next;
             c->u = c->u_next;
             c->lpar = c->lpar_next;
         }
-        const uint32_t n_assign = c->n_assign;
-        const uint32_t r0 = chunk * kDecodeThreads + warp * 32u;
-        if (r0 >= n_assign) continue;                 // warp-uniform
-        const uint32_t r = r0 + (threadIdx.x & 31u);
         const uint32_t rate = vol_of<kOne>(L, v).g.rate;
-        bool have = r < n_assign;
-        const uint32_t b = have ? s.inew[r] : 0u;
-        const uint32_t slot = have ? s.newslot[r] : 0u;
-        have = have && in_bounds(b < vol_of<kOne>(L, v).g.nb && slot < c->cap, &c->status);
-        stage_blocks(s.bits, rate, b, have, sm.stage);
-        if (!have) continue;
-        float val[64];
+        const bool mine = have && !skip && in_bounds(b < vol_of<kOne>(L, v).g.nb && slot < c->cap, &c->status);
+        const uint32_t to = slot, id = b;
+        const uint32_t any = __ballot_sync(0xffffffffu, mine);
+        load_ids(x + gridDim.x);
+        if (any) stage_blocks(s.bits, rate, id, mine, sm.stage);
+        if (have) {                                   // of the next chunk, maybe another volume's
+            const VolEntry &nv = vol_of<kOne>(L, item_vol<kOne>(pre, L.n, x + gridDim.x));
+            if (b < nv.g.nb) prefetch_block(nv.s.bits, nv.g.rate, b);
+        }
+        if (!any) continue;                                       // warp-uniform
+        float val[64];                                // (a lane without a block decodes a zero one)
         decode_staged(sm.stage + (threadIdx.x & 31u) * (2u * rate + 1u), rate, sm.tab, val, sm.planes + threadIdx.x,
                       kDecodeThreads);
-        float4 *dst = reinterpret_cast<float4 *>(s.slots + (size_t)slot * 64);
-#pragma unroll
-        for (int i = 0; i < 16; i++) dst[i] = make_float4(val[4 * i], val[4 * i + 1], val[4 * i + 2], val[4 * i + 3]);
-        if (s.bmask) {                                // the block's below mask, while its samples are here
+        store_blocks(s.slots, to, any, val, sm.planes + threadIdx.x, kDecodeThreads);
+        if (mine && s.bmask) {                        // the block's below mask, while its samples are here
             // the sign bits of sample - iso (a NaN's is clear; -0 where iso is 0:
             // -0 - 0 would be -0, which is not below)
             const float iso = c->params.iso, sub = iso == 0.0f ? -0.0f : iso;
@@ -558,7 +570,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 768 / kDecodeThreads) decode_n
                 lo = __funnelshift_l(__float_as_uint(__fsub_rn(val[i], sub)), lo, 1);
                 hi = __funnelshift_l(__float_as_uint(__fsub_rn(val[32 + i], sub)), hi, 1);
             }
-            s.bmask[slot] = ((unsigned long long)hi << 32) | lo;
+            s.bmask[to] = ((unsigned long long)hi << 32) | lo;
         }
     }
     if constexpr (decode_runs_lru_b<kDecodeThreads>()) {
