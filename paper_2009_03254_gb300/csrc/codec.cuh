@@ -203,9 +203,21 @@ __host__ __device__ constexpr uint32_t group_step_entry(uint32_t state, uint32_t
 
 constexpr uint32_t kGroupTableEntries = 512;
 
-// fill a block's copy of the table (all threads; the caller synchronises)
+struct GroupTable {
+    uint32_t e[kGroupTableEntries];
+};
+__host__ __device__ constexpr GroupTable make_group_table() {
+    GroupTable t{};
+    for (uint32_t i = 0; i < kGroupTableEntries; i++) t.e[i] = group_step_entry(i >> 8, i & 255u);
+    return t;
+}
+__device__ const GroupTable kGroupTable = make_group_table();
+
+// fill a block's copy of the table (all threads; the caller synchronises).
+// Made at compile time: working the entries out took a CTA of 128 some 600
+// instructions a warp, where a chunk of blocks takes 3700.
 __device__ __forceinline__ void load_group_table(uint32_t *tab) {
-    for (uint32_t i = threadIdx.x; i < kGroupTableEntries; i += blockDim.x) tab[i] = group_step_entry(i >> 8, i & 255u);
+    for (uint32_t i = threadIdx.x; i < kGroupTableEntries; i += blockDim.x) tab[i] = __ldg(&kGroupTable.e[i]);
 }
 
 // Parse the bit planes of a staged block of `rate` words at shared address
