@@ -222,55 +222,60 @@ __device__ __forceinline__ uint32_t lane_cut_word(const uint32_t m[4], uint32_t 
 // One candidate per thread.  Its 64 cells are handled together as 64-bit
 // masks: corner c's mask says, per cell, whether that corner is below the
 // isovalue; the eight masks are the block's own below mask and its
-// neighbours' shifted in.  A cell's triangles follow from the case rule
-// without the table: its segments link into C cycles through its E cut
-// edges, a cycle of length l is fanned into l - 2 triangles, so it has
-// E - 2C.  The cycles separate the regions of the cube's surface, one fewer
-// than there are regions: C = B + A - 1 with B the groups of below corners
-// joined by cube edges and A those of above corners joined by edges and
-// face diagonals (a face with two diagonal below corners cuts each off on
-// its own).  A is 2 exactly when two opposite corners are above alone, else
-// 1; B counts the below corners with no below neighbour, plus one if any
-// other exist, plus one more for two opposite parallel edges.  Every term
-// is a mask, and a block's count the sum of their popcounts.
+// neighbours' shifted in.  A crossing cell's triangles follow from its
+// corners without the table.  Its segments link into C cycles through its E
+// cut edges, and a cycle of length l is fanned into l - 2 triangles: E - 2C.
+// The cycles separate the regions of the cube's surface, one fewer than
+// there are regions: C = B + A - 1 with B the groups of below corners joined
+// by cube edges and A those of above corners joined by edges and face
+// diagonals (a face with two diagonal below corners cuts each off on its
+// own).  With k below corners and J edges between them, E = 3k - 2J and
+// B = k - J + (the cycles of those edges), which leaves
+//   k - 2 (cycles of the below edges) - 2 (A - 1):
+// the cycles are the faces with all four corners below (F), and the ring of
+// six around two opposite above corners (H), where A is 2:  k - 2F - 4H.
+// Over 64 cells the terms are carry-save sums of masks and five popcounts.
 //
 // The counting reads 8 bytes a block of each +group (L2 holds most of them)
-// instead of staging 5x5x5 samples.
+// instead of staging 5x5x5 samples.  Three loads in a row and these
+// instructions bound it: with E and C counted edge by edge (44 popcounts, at a
+// quarter of the rate) the 411 k candidates of a 384^3 channel took 8.25
+// million instructions and a tile of 768 7 to 14 us, now 6.35 and 6.
 
-__device__ __forceinline__ uint32_t count_triangles(const unsigned long long (&m)[8], unsigned long long valid) {
-    uint32_t edges = 0, cycles = 0;
-    unsigned long long joined = 0, all = ~0ull;
+__device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) { return lop3<0x96>(a, b, c); }
+__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) { return lop3<0xE8>(a, b, c); }
+
+// triangles of 32 cells with corner masks m; sets the crossing cells
+__device__ __forceinline__ int count_triangles32(const uint32_t (&m)[8], uint32_t valid, uint32_t &cross) {
+    // faces (d, side) with all corners below, and their count as bits s, tw
+    // (at most three in a crossing cell)
+    const uint32_t p01 = m[0] & m[1], p23 = m[2] & m[3], p45 = m[4] & m[5], p67 = m[6] & m[7];
+    const uint32_t f0 = m[0] & m[2] & m[4] & m[6], f1 = m[1] & m[3] & m[5] & m[7];
+    const uint32_t f2 = p01 & p45, f3 = p23 & p67, f4 = p01 & p23, f5 = p45 & p67;
+    const uint32_t sa = xor3(f0, f1, f2), sb = xor3(f3, f4, f5);
+    const uint32_t s = sa ^ sb, tw = (maj3(f0, f1, f2) | maj3(f3, f4, f5)) | (sa & sb);
+    cross = (m[0] | m[1] | m[2] | m[3] | m[4] | m[5] | m[6] | m[7]) & ~(f4 & f5) & valid;
+    // below corners as bits o, t, f
+    const uint32_t oa = xor3(m[0], m[1], m[2]), ob = xor3(m[3], m[4], m[5]), oc = xor3(oa, ob, m[6]);
+    const uint32_t ta = maj3(m[0], m[1], m[2]), tb = maj3(m[3], m[4], m[5]), tc = maj3(oa, ob, m[6]);
+    const uint32_t td = oc & m[7], te = xor3(ta, tb, tc);
+    const uint32_t o = oc ^ m[7], t = te ^ td, f = maj3(ta, tb, tc) ^ (te & td);
+    const uint32_t ring = f & t & ~o & ~(s | tw);
+    return __popc(o & cross) + 2 * (__popc(t & cross) - __popc(s & cross)) +
+           4 * (__popc(f & ~ring & cross) - __popc(tw & cross));
+}
+
+__device__ __forceinline__ uint32_t count_triangles(const unsigned long long (&m)[8], unsigned long long valid,
+                                                    unsigned long long &cross) {
+    uint32_t lo[8], hi[8], clo, chi;
 #pragma unroll
     for (int c = 0; c < 8; c++) {
-        all &= m[c];
-        cycles += __popcll(m[c] & ~(m[c ^ 1] | m[c ^ 2] | m[c ^ 4]) & valid);        // lone below corners
-#pragma unroll
-        for (int d = 1; d < 8; d <<= 1)
-            if (!(c & d)) {
-                edges += __popcll((m[c] ^ m[c | d]) & valid);
-                joined |= m[c] & m[c | d];
-            }
+        lo[c] = (uint32_t)m[c];
+        hi[c] = (uint32_t)(m[c] >> 32);
     }
-    cycles += __popcll(joined & ~all & valid);
-    // two opposite parallel edges below, the rest above (6 ways), or two
-    // opposite corners above, the rest below (4 ways): one cycle more
-    unsigned long long more = 0;
-#pragma unroll
-    for (int d = 1; d < 8; d <<= 1) {                    // edges along d at offsets 0, p, q, p | q
-        const int p = d == 1 ? 2 : 1, q = d == 4 ? 2 : 4;
-        more |= m[0] & m[d] & m[p | q] & m[7] & ~(m[p] | m[p | d] | m[q] | m[q | d]);
-        more |= m[p] & m[p | d] & m[q] & m[q | d] & ~(m[0] | m[d] | m[p | q] | m[7]);
-    }
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        unsigned long long six = ~(m[c] | m[7 - c]);
-#pragma unroll
-        for (int k = 0; k < 8; k++)
-            if (k != c && k != 7 - c) six &= m[k];
-        more |= six;
-    }
-    cycles += __popcll(more & valid);
-    return edges - 2u * cycles;
+    const int n = count_triangles32(lo, (uint32_t)valid, clo) + count_triangles32(hi, (uint32_t)(valid >> 32), chi);
+    cross = ((unsigned long long)chi << 32) | clo;
+    return (uint32_t)n;
 }
 
 // the cut edges of the block's 5x5x5 window: a cell counts its three edges at
@@ -291,16 +296,29 @@ __device__ __forceinline__ uint32_t count_vertices(const unsigned long long (&m)
     }
     uint32_t n = 0;
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const int p = (a + 1) % 3, q = (a + 2) % 3;      // the other two axes
+    for (int half = 0; half < 2; half++) {
+        uint32_t e[4][3];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const int p = (a + 1) % 3, q = (a + 2) % 3;  // the other two axes
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const int c = ((k & 1) << p) | ((k >> 1) << q);
+                unsigned long long w = (m[c] ^ m[c | (1 << a)]) & valid;
+                if (k & 1) w &= last[p];
+                if (k & 2) w &= last[q];
+                e[k][a] = (uint32_t)(w >> (32 * half));
+            }
+        }
+        uint32_t o[4], t[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const int c = ((k & 1) << p) | ((k >> 1) << q);
-            unsigned long long w = (m[c] ^ m[c | (1 << a)]) & valid;
-            if (k & 1) w &= last[p];
-            if (k & 2) w &= last[q];
-            n += __popcll(w);
+            o[k] = xor3(e[k][0], e[k][1], e[k][2]);
+            t[k] = maj3(e[k][0], e[k][1], e[k][2]);
         }
+        n += __popc(xor3(o[0], o[1], o[2])) + __popc(o[3]) +
+             2 * (__popc(maj3(o[0], o[1], o[2])) + __popc(xor3(t[0], t[1], t[2])) + __popc(t[3])) +
+             4 * __popc(maj3(t[0], t[1], t[2]));
     }
     return n;
 }
@@ -365,8 +383,7 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
                 uint32_t lim;
                 corner_masks(s, g, s.icand[i], m, lim);
                 const unsigned long long valid = valid_cells(lim);
-                nt = count_triangles(m, valid);
-                sm.cross[r][threadIdx.x] = crossing_cells(m, valid);
+                nt = count_triangles(m, valid, sm.cross[r][threadIdx.x]);
                 if (kIdx) nv = count_vertices(m, valid, lim);
                 if (s.counts) s.counts[i] = nt | (nv << 16);
             }
