@@ -298,7 +298,7 @@ Plan launch_plan(const Plan *want, int device, uint64_t total_blocks, uint64_t t
     auto tiles_of = [&](uint64_t n, int tile) { return (n + tile - 1) / tile + n_vols; };
     clamp(use.cull, tiles_of(total_blocks, use.cull_tile));
     clamp(use.lru_a, 2 * tiles_of(total_slots, kScanTile) + n_vols);
-    clamp(use.lru_b, tiles_of(total_slots, 32));          // also 4 cached blocks' masks a warp
+    clamp(use.lru_b, tiles_of(total_slots, 64));          // also 8 cached blocks' masks a warp
     clamp(use.decode, tiles_of(total_slots, use.decode_tile));
     clamp(use.mc_emit, tiles_of(total_slots, use.emit_tile));
     clamp(use.mc_scan, tiles_of(total_slots, single ? kThreads : kCountTile));

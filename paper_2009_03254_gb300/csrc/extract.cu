@@ -372,12 +372,14 @@ __global__ void __launch_bounds__(kThreads) lru_a_kernel(Launch L) {
 // The below masks of the active blocks already in the cache (the new ones
 // get theirs from the decode): bit i says sample i is below the isovalue.
 // The count reads these 8 bytes of a block instead of its samples.  A warp
-// takes 4 blocks at a time, all eight 128-byte loads before the ballots.
-// Bound by the reads of 256 bytes a block; it runs in lru_b's launch, whose
+// takes 8 blocks at a time, all sixteen 128-byte loads before the ballots.
+// Bound by the reads of 256 bytes a block, and by how many of them are in
+// flight (4 blocks a warp and 4 CTAs an SM took 45 us where 8 and 6 take 36,
+// 512^3 noise with 400 k cached blocks); it runs in lru_b's launch, whose
 // own work is a few latency-bound tiles, rather than in one of its own.
 // Nothing here reads what the cache update or the decode's commit changes (a
 // hit keeps its slot).  Called by all threads of the block.
-constexpr uint32_t kMaskBlocks = 4;
+constexpr uint32_t kMaskBlocks = 8;
 
 template <bool kOne>
 __device__ __forceinline__ void hit_mask_work(const Launch &L, uint32_t *pre) {
@@ -485,7 +487,7 @@ __device__ __forceinline__ void lru_b_work(const Launch &L, TileScan<kRounds> &t
 }
 
 template <bool kOne>
-__global__ void __launch_bounds__(kThreads) lru_b_kernel(Launch L) {
+__global__ void __launch_bounds__(kThreads, 5) lru_b_kernel(Launch L) {
     __shared__ TileScan<kRounds> ts;
     __shared__ uint32_t pre[kMaxBatch + 1];
     __shared__ uint32_t slot_x;
