@@ -33,6 +33,7 @@ namespace bcmc {
 
 template <bool kOne>
 __global__ void __launch_bounds__(kThreads) prep_kernel(Launch L) {
+    after_previous_stage();
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
     // Bound by the latency of one dependent read a volume (mc_tiles), so every
     // volume gets an equal share of the CTAs: with all CTAs walking the
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(kThreads) cull_kernel(Launch L) {
     __shared__ CullSmem<kR> sm;
     __shared__ uint32_t pre[kMaxBatch + 1];
     __shared__ uint32_t slot_x;
+    after_previous_stage();
     const uint32_t total = launch_prefix<kOne>(
         L, [&](uint32_t v) { return ceil_div(vol_of<kOne>(L, v).g.nb, kR * kThreads); }, pre);
     while (true) {
@@ -292,6 +294,7 @@ __global__ void __launch_bounds__(kThreads) lru_a_kernel(Launch L) {
     __shared__ uint32_t slot_x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
+    after_previous_stage();
     const uint32_t total =
         launch_prefix<kOne>(L, [&](uint32_t v) { return lru_a_items(vol_of<kOne>(L, v).s.ctl); }, pre);
     while (true) {
@@ -491,6 +494,7 @@ __global__ void __launch_bounds__(kThreads, 5) lru_b_kernel(Launch L) {
     __shared__ TileScan<kRounds> ts;
     __shared__ uint32_t pre[kMaxBatch + 1];
     __shared__ uint32_t slot_x;
+    after_previous_stage();
     lru_b_work<kOne>(L, ts, pre, &slot_x);
 }
 
@@ -517,6 +521,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 768 / kDecodeThreads) decode_n
     __shared__ uint32_t slot_x;
     const DecodeSmem sm = decode_smem_layout(dsm, kDecodeThreads, kOne ? L.one.g.rate : L.max_rate);
     load_group_table(sm.tab);
+    after_previous_stage();
     __syncthreads();
     const uint32_t total = launch_prefix<kOne>(
         L, [&](uint32_t v) { return max(1u, ceil_div(vol_of<kOne>(L, v).s.ctl->n_assign, kDecodeThreads)); },
@@ -757,13 +762,13 @@ size_t decode_smem(const Launch &L, int threads) {
 // Algorithm 1 after the cull (both list kernels), then the decode
 template <bool kOne>
 void cache_update(const Launch &L, const Plan &pl, cudaStream_t st, cudaEvent_t *ev, cudaEvent_t bits_ready) {
-    lru_a_kernel<kOne><<<pl.lru_a, kThreads, 0, st>>>(L);
-    if (pl.decode_tile != kThreads) lru_b_kernel<kOne><<<pl.lru_b, kThreads, 0, st>>>(L);   // else the decode's
+    launch_next(L, lru_a_kernel<kOne>, pl.lru_a, kThreads, 0, st);
+    if (pl.decode_tile != kThreads) launch_next(L, lru_b_kernel<kOne>, pl.lru_b, kThreads, 0, st);   // else the decode's
     if (ev) cudaEventRecord(ev[3], st);
     if (bits_ready) cudaStreamWaitEvent(st, bits_ready, 0);   // the bitstream may still be on its way
-    if (pl.decode_tile == 64) decode_new_kernel<64, kOne><<<pl.decode, 64, decode_smem(L, 64), st>>>(L);
-    else if (pl.decode_tile == 256) decode_new_kernel<256, kOne><<<pl.decode, 256, decode_smem(L, 256), st>>>(L);
-    else decode_new_kernel<128, kOne><<<pl.decode, 128, decode_smem(L, 128), st>>>(L);
+    if (pl.decode_tile == 64) launch_next(L, decode_new_kernel<64, kOne>, pl.decode, 64, decode_smem(L, 64), st);
+    else if (pl.decode_tile == 256) launch_next(L, decode_new_kernel<256, kOne>, pl.decode, 256, decode_smem(L, 256), st);
+    else launch_next(L, decode_new_kernel<128, kOne>, pl.decode, 128, decode_smem(L, 128), st);
     if (ev) cudaEventRecord(ev[4], st);
 }
 
@@ -772,14 +777,14 @@ void cull_only(const Launch &L, const Plan &pl, cudaStream_t st) {
     // volumes with segment ranges (the largest) take 8192-block tiles: half
     // the look-back walks of 4096-block tiles, whose depth grows with the
     // tiles in flight
-    if (kOne ? L.one.s.seg != nullptr : L.seg_any != 0) cull_kernel<32, kOne, true><<<pl.cull, kThreads, 0, st>>>(L);
-    else if (pl.cull_tile == 2048) cull_kernel<8, kOne, false><<<pl.cull, kThreads, 0, st>>>(L);
-    else cull_kernel<16, kOne, false><<<pl.cull, kThreads, 0, st>>>(L);
+    if (kOne ? L.one.s.seg != nullptr : L.seg_any != 0) launch_next(L, cull_kernel<32, kOne, true>, pl.cull, kThreads, 0, st);
+    else if (pl.cull_tile == 2048) launch_next(L, cull_kernel<8, kOne, false>, pl.cull, kThreads, 0, st);
+    else launch_next(L, cull_kernel<16, kOne, false>, pl.cull, kThreads, 0, st);
 }
 
 template <bool kOne>
 void front(const Launch &L, const Plan &pl, cudaStream_t st, cudaEvent_t *ev, cudaEvent_t bits_ready) {
-    prep_kernel<kOne><<<pl.prep, kThreads, 0, st>>>(L);
+    launch_next(L, prep_kernel<kOne>, pl.prep, kThreads, 0, st);
     if (ev) cudaEventRecord(ev[1], st);
     cull_only<kOne>(L, pl, st);
     if (ev) cudaEventRecord(ev[2], st);

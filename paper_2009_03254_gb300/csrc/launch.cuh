@@ -19,6 +19,38 @@
 
 namespace bcmc {
 
+// The stages of a small volume's extraction are launched one ahead
+// (launch_next): a stage's CTAs may take their places while the one before it
+// finishes, and wait here for all of it, results included, before they read
+// anything.  Called by every thread of every CTA; launched the ordinary way a
+// kernel waits for nothing.
+__device__ __forceinline__ void after_previous_stage() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Volumes of up to this many blocks are launch-bound: a 64^3 sphere from a
+// warm cache (4096 blocks) takes 57 us with its stages launched ahead, 64
+// without.  In larger ones waiting CTAs hold shared memory that the running
+// stage would have as cache: 96^3 noise from an empty cache (13824 blocks)
+// 146 against 134 us, five surfaces of 512^3 noise 1725 against 1620.
+constexpr uint32_t kAheadBlocks = 8192;
+
+// launch a stage whose kernel calls after_previous_stage
+inline void launch_next(const Launch &L, void (*kernel)(Launch), int grid, int threads, size_t smem, cudaStream_t st) {
+    cudaLaunchAttribute ahead{};
+    ahead.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    ahead.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &ahead;
+    c.numAttrs = !L.vols && L.one.g.nb <= kAheadBlocks ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, L);            // (errors: the caller's cudaGetLastError)
+}
+
 __device__ __forceinline__ uint32_t ceil_div(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
 
 // pre[v] = sum of count(u) for u < v, for v in [0, n]; returns pre[n].

@@ -354,6 +354,7 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
     __shared__ uint32_t s_item;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
+    after_previous_stage();
     const uint32_t total = launch_prefix<kOne>(
         L, [&](uint32_t v) {
             const uint32_t n = mc_candidates(vol_of<kOne>(L, v).s.ctl);
@@ -727,6 +728,7 @@ __device__ __forceinline__ void emit_body(const Launch &L) {
     EmitSmem<kW, kIdx> &sm = *reinterpret_cast<EmitSmem<kW, kIdx> *>(smem_raw);
     uint32_t *pre = reinterpret_cast<uint32_t *>(&sm + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    after_previous_stage();
     // all failure bits are final before this kernel starts
     const uint32_t total = launch_prefix<kOne>(
         L, [&](uint32_t v) {
@@ -892,13 +894,13 @@ template <int kW, bool kOne, bool kIdx>
 void emit_w(const Launch &L, bool debug, int grid, cudaStream_t st) {
     const size_t bytes = emit_smem<kW, kIdx>(L);
     if constexpr (kIdx) {
-        if (debug) mc_emit_indexed_kernel<kW, true><<<grid, 32 * kW, bytes, st>>>(L);
-        else mc_emit_indexed_kernel<kW, false><<<grid, 32 * kW, bytes, st>>>(L);
+        if (debug) launch_next(L, mc_emit_indexed_kernel<kW, true>, grid, 32 * kW, bytes, st);
+        else launch_next(L, mc_emit_indexed_kernel<kW, false>, grid, 32 * kW, bytes, st);
     } else if constexpr (kOne) {
-        if (debug) mc_emit_kernel<kW, true, true><<<grid, 32 * kW, bytes, st>>>(L);
-        else mc_emit_kernel<kW, false, true><<<grid, 32 * kW, bytes, st>>>(L);
+        if (debug) launch_next(L, mc_emit_kernel<kW, true, true>, grid, 32 * kW, bytes, st);
+        else launch_next(L, mc_emit_kernel<kW, false, true>, grid, 32 * kW, bytes, st);
     } else {                                          // debug volumes are not batched
-        mc_emit_kernel<kW, false, false><<<grid, 32 * kW, bytes, st>>>(L);
+        launch_next(L, mc_emit_kernel<kW, false, false>, grid, 32 * kW, bytes, st);
     }
 }
 
@@ -949,9 +951,9 @@ void emit_any(const Launch &L, bool debug, const Plan &pl, cudaStream_t st) {
 }  // namespace
 
 void launch_mc_scan(const Launch &L, bool debug, const Plan &pl, cudaStream_t st, bool indexed) {
-    if (L.vols) mc_scan_kernel<false, false><<<pl.mc_scan, kThreads, 0, st>>>(L);
-    else if (indexed) mc_scan_kernel<true, true><<<pl.mc_scan, kThreads, 0, st>>>(L);
-    else mc_scan_kernel<true, false><<<pl.mc_scan, kThreads, 0, st>>>(L);
+    if (L.vols) launch_next(L, mc_scan_kernel<false, false>, pl.mc_scan, kThreads, 0, st);
+    else if (indexed) launch_next(L, mc_scan_kernel<true, true>, pl.mc_scan, kThreads, 0, st);
+    else launch_next(L, mc_scan_kernel<true, false>, pl.mc_scan, kThreads, 0, st);
     if (debug && !L.vols) debug_cases_kernel<<<pl.mc_scan, kThreads, 0, st>>>(L);
 }
 
