@@ -76,12 +76,12 @@ CPU_ORIGIN = (0, 0, 192)
 REF_WINDOW = (128, 128, 64)       # per-step sample of the reference arm
 L2_FLUSH_BYTES = 512 << 20
 CTL_BYTES = 168                   # control block (struct Ctl): iso_extract reads it back after the scan and after the emission
-KERNELS_PER_SURFACE = 8           # prep, cull, lru_a, lru_b (list append), decode, count, scan, emit
+KERNELS_PER_SURFACE = 7           # prep, cull, lru_a, lru_b (list append), decode, count and scan, emit
 KERNELS_PER_RESET = 2
-KERNELS = ("cull", "cache_update", "decode", "count", "scan", "emit")
+KERNELS = ("cull", "cache_update", "decode", "count", "emit")
 KERNEL_OF = {"cull": ("cull_kernel", "extract.cu"), "cache_update": ("lru_a_kernel+lru_b_kernel", "extract.cu"),
-             "decode": ("decode_new_kernel", "extract.cu"), "count": ("mc_count_kernel", "mc.cu"),
-             "scan": ("mc_scan_kernel", "mc.cu"), "emit": ("mc_emit_kernel", "mc.cu")}
+             "decode": ("decode_new_kernel", "extract.cu"), "count": ("mc_scan_kernel", "mc.cu"),
+             "emit": ("mc_emit_kernel", "mc.cu")}
 
 
 def parse():
@@ -187,7 +187,7 @@ def measured_peaks():
         return None
 
 
-PROFILE_SOURCES = ("extract.cu", "mc.cu", "codec.cuh", "common.cuh", "kernels.cuh", "launch.cuh", "tile_scan.cuh")
+PROFILE_SOURCES = ("extract.cu", "mc.cu", "cell_masks.cuh", "codec.cuh", "common.cuh", "kernels.cuh", "launch.cuh", "tile_scan.cuh")
 
 
 def profile_sources_sha():
@@ -231,11 +231,11 @@ def stage_bytes(stats, rate, nb):
     return {
         "cull": 8 * nb + nb / 8 + 4 * na + 4 * nn + 8 * na + 4 * nc,   # hulls, mask, I_active, I_new, +group hulls, I_cand
         "cache_update": 0.0,
-        "decode": nn * (8 * rate + 256 + 8),                           # compressed in, decoded out, I_new + slot
-        "count": nc * (256 + 4 + 4 + 64),                              # decoded tiles in, id in, count and cases out
-        "scan": nc * (4 + 8) + 4 * no,                                 # counts in, offsets and I_occ out
-        "emit": no * (256 + 4 + 4 + 8 + 64) + 48 * T,                  # per occupied block: decoded tile, I_occ, id,
-                                                                       # offset, cases in; vertices out
+        "decode": nn * (8 * rate + 256 + 8 + 8),                       # compressed in, decoded and mask out, I_new + slot
+        "count": nc * (4 + 4 + 8) + no * (4 + 8 + 8),                  # id, slot, below mask in; per occupied block its
+                                                                       # id, offset and crossing cells out
+        "emit": no * (256 + 4 + 8 + 8) + 48 * T,                       # per occupied block: decoded tile, id, offset,
+                                                                       # crossing cells in; vertices out
     }
 
 
