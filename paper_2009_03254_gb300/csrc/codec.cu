@@ -161,7 +161,8 @@ __global__ void __launch_bounds__(kCodecThreads, 5) decode_volume_kernel(const u
 // Launch a codec kernel over n blocks, a lane each, with no more CTAs than
 // the device holds at once: each fills its group-step table once (a CTA per
 // 128 blocks spent a part of its time on that, and the launch on 20 waves of
-// them: 474 us for the 512^3 decode at 8 bits a value, now 385).  The
+// them: 474 us for the 512^3 decode at 8 bits a value, 385 with resident CTAs,
+// 310 with the present parse).  The
 // resident count is looked up once per kernel, device and rate.
 template <class K, class... A>
 void launch_codec(K kernel, std::atomic<uint32_t> (*known)[33], uint32_t rate, uint64_t n, cudaStream_t st, A... args) {

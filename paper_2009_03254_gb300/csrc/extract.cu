@@ -502,7 +502,9 @@ __global__ void __launch_bounds__(kThreads, 5) lru_b_kernel(Launch L) {
 //
 // Chunks of kDecodeThreads new blocks; each warp of a chunk stages its 32
 // blocks' words in shared memory with coalesced loads and decodes them one
-// per lane (codec.cuh).  Chunk 0 of every volume (each volume has at least
+// per lane (codec.cuh), its next chunk's ids loaded and words fetched into L2
+// meanwhile (two dependent DRAM latencies a chunk before: 68 us for 384^3
+// noise with lanes storing their own blocks, 61 with both).  Chunk 0 of every volume (each volume has at least
 // one) also commits the volume's cache update.  With 256-thread blocks the
 // kernel then does lru_b's work (the list for the next update, which
 // nothing before then reads): its memory latency hides behind the decoding
