@@ -170,7 +170,8 @@ int iso_release_cached_memory(int device);
  *                    with ranges of the decoded values
  *   opt              may be NULL (defaults above)
  * Host inputs are copied; the caller keeps ownership.  With
- * ISO_INPUT_ON_DEVICE they are copied device-to-device.  On success *out
+ * ISO_INPUT_ON_DEVICE they are copied device-to-device (the ranges, read in
+ * place, must be 4-byte aligned: else ISO_ERR_INVALID_ARG).  On success *out
  * owns all device state until iso_release.  Blocks until the upload is done. */
 int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_bytes,
                     uint32_t nx, uint32_t ny, uint32_t nz, uint32_t rate_bits,
@@ -348,7 +349,9 @@ int iso_extract_all_blocks_into(iso_volume *v, float isovalue, float *d_vertices
 /* Decode a whole compressed volume into a dense float32 field (nx*ny*nz,
  * x fastest; samples past the volume edge are dropped), one thread per
  * block (the full-volume decompression the paper times for ZFP).  Device
- * pointers; queued on `stream`, does not block. */
+ * pointers aligned to their elements (8 and 4 bytes; else
+ * ISO_ERR_INVALID_ARG; a 16-byte aligned field is written faster); queued on
+ * `stream`, does not block. */
 int iso_decode_volume(const uint64_t *d_bits, uint32_t nx, uint32_t ny, uint32_t nz, uint32_t rate_bits,
                       float *d_field, void *stream);
 
@@ -445,15 +448,19 @@ int iso_mc_case_table(uint8_t *num_tri, uint8_t *tri_edges);
  * the GPU (for producing test and benchmark inputs; the paper's method
  * itself only decodes).  d_field is nx*ny*nz floats (x fastest);
  * d_bits receives nb*rate words; d_bmin/d_bmax receive each block's range
- * over its decoded in-volume samples.  All pointers are device pointers;
- * the work is queued on `stream` and the call does not block.
+ * over its decoded in-volume samples.  All pointers are device pointers,
+ * each aligned to its elements (4 bytes for floats, 8 for words; else
+ * ISO_ERR_INVALID_ARG; a 16-byte aligned field is read faster); the work is
+ * queued on `stream` and the call does not block.
  * Non-finite samples are not allowed (the output is then unspecified). */
 int iso_encode_field(const float *d_field, uint32_t nx, uint32_t ny, uint32_t nz, uint32_t rate_bits,
                      uint64_t *d_bits, float *d_bmin, float *d_bmax, void *stream);
 
 /* Decode blocks ids[0..n) of a device-resident compressed volume into
- * out (n*64 floats, block-local order), device pointers, queued on
- * `stream` (Section 4.2.1 applied to an explicit list). */
+ * out (n*64 floats, block-local order), device pointers aligned to their
+ * elements (8 bytes for d_bits, 4 for the others; else ISO_ERR_INVALID_ARG;
+ * 16-byte aligned output is written faster), queued on `stream` (Section
+ * 4.2.1 applied to an explicit list). */
 int iso_decode_blocks(const uint64_t *d_bits, uint32_t rate_bits, const uint32_t *d_ids, uint64_t n,
                       float *d_out, void *stream);
 

@@ -774,6 +774,9 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     if (compressed_bytes != (size_t)g.nb * g.rate * 8) return ISO_ERR_INVALID_ARG;
     iso_options o{};
     if (opt) o = *opt;
+    // ranges on the device are read in place, as floats
+    if ((o.flags & ISO_INPUT_ON_DEVICE) && (misaligned(block_min, 4) || misaligned(block_max, 4)))
+        return ISO_ERR_INVALID_ARG;
     double frac = o.initial_cache_fraction > 0 ? o.initial_cache_fraction : 0.1;
 
     iso_volume *v = new (std::nothrow) iso_volume();
@@ -988,7 +991,7 @@ int iso_extract_indexed_into(iso_volume *v, float isovalue, int vertex_format, v
 
 int iso_decode_volume(const uint64_t *d_bits, uint32_t nx, uint32_t ny, uint32_t nz, uint32_t rate_bits,
                       float *d_field, void *stream) {
-    if (!d_bits || !d_field) return ISO_ERR_INVALID_ARG;
+    if (!d_bits || !d_field || misaligned(d_bits, 8) || misaligned(d_field, 4)) return ISO_ERR_INVALID_ARG;
     Geom g;
     int rc = geometry(nx, ny, nz, rate_bits, &g);
     if (rc) return rc;
@@ -1123,7 +1126,9 @@ int iso_cache_reset(iso_volume *v) {
 
 int iso_encode_field(const float *d_field, uint32_t nx, uint32_t ny, uint32_t nz, uint32_t rate_bits,
                      uint64_t *d_bits, float *d_bmin, float *d_bmax, void *stream) {
-    if (!d_field || !d_bits || !d_bmin || !d_bmax) return ISO_ERR_INVALID_ARG;
+    if (!d_field || !d_bits || !d_bmin || !d_bmax || misaligned(d_field, 4) || misaligned(d_bits, 8) ||
+        misaligned(d_bmin, 4) || misaligned(d_bmax, 4))
+        return ISO_ERR_INVALID_ARG;
     Geom g;
     int rc = geometry(nx, ny, nz, rate_bits, &g);
     if (rc) return rc;
@@ -1136,7 +1141,8 @@ int iso_decode_blocks(const uint64_t *d_bits, uint32_t rate_bits, const uint32_t
                       void *stream) {
     if (rate_bits < 1 || rate_bits > 32) return ISO_ERR_INVALID_ARG;
     if (n == 0) return ISO_OK;
-    if (!d_bits || !d_ids || !d_out) return ISO_ERR_INVALID_ARG;
+    if (!d_bits || !d_ids || !d_out || misaligned(d_bits, 8) || misaligned(d_ids, 4) || misaligned(d_out, 4))
+        return ISO_ERR_INVALID_ARG;
     launch_decode_list(d_bits, rate_bits, d_ids, n, d_out, (cudaStream_t)stream);
     CK(cudaGetLastError());
     return ISO_OK;

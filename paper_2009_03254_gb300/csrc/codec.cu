@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kCodecThreads, 5) decode_list_kernel(const uin
     extern __shared__ uint64_t dsm[];
     const DecodeSmem sm = codec_smem(dsm, rate);
     const uint32_t lane = threadIdx.x & 31u;
+    const bool aligned = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
     for (uint64_t i0 = blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); i0 < n;
          i0 += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t i = i0 + lane;
@@ -108,7 +109,8 @@ __global__ void __launch_bounds__(kCodecThreads, 5) decode_list_kernel(const uin
         stage_blocks(bits, rate, have ? ids[i] : 0u, have, sm.stage);
         float v[64];                       // (a lane without a block decodes a zero one)
         decode_staged(sm.stage + lane * (2u * rate + 1u), rate, sm.tab, v, sm.planes + threadIdx.x, blockDim.x);
-        store_blocks(out + i0 * 64, lane, __ballot_sync(0xffffffffu, have), v, sm.planes + threadIdx.x, blockDim.x);
+        store_blocks(out + i0 * 64, lane, __ballot_sync(0xffffffffu, have), v, sm.planes + threadIdx.x, blockDim.x,
+                     aligned);
     }
 }
 
@@ -118,10 +120,10 @@ __global__ void __launch_bounds__(kCodecThreads, 5) decode_list_kernel(const uin
 // contiguous span of the field, and the staging loads read one contiguous
 // span of the bitstream.
 __global__ void __launch_bounds__(kCodecThreads, 5) decode_volume_kernel(const uint64_t *__restrict__ bits, Geom g,
-                                                                      float *field) {
+                                                                      float *field, uint32_t skew) {
     extern __shared__ uint64_t dsm[];
     const DecodeSmem sm = codec_smem(dsm, g.rate);
-    const bool rows16 = (g.nx & 3u) == 0;       // every row starts 16-byte aligned
+    const bool rows16 = (skew & 3u) == 0;       // every row starts 16-byte aligned
     const uint32_t lane = threadIdx.x & 31u;
     for (uint32_t b0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); b0 < g.nb; b0 += gridDim.x * blockDim.x) {
         const uint32_t b = b0 + lane;
@@ -188,7 +190,10 @@ void launch_codec(K kernel, std::atomic<uint32_t> (*known)[33], uint32_t rate, u
 std::atomic<uint32_t> g_known[3][64][33];               // decode_volume, encode, decode_list
 
 void launch_decode_volume(const uint64_t *bits, const Geom &g, float *field, cudaStream_t st) {
-    launch_codec(decode_volume_kernel, g_known[0], g.rate, g.nb, st, bits, g, field);
+    // rows are aligned when they hold a multiple of four floats and the field,
+    // which may start at any float, is
+    const uint32_t skew = g.nx | (uint32_t)((reinterpret_cast<uintptr_t>(field) & 15u) / 4u);
+    launch_codec(decode_volume_kernel, g_known[0], g.rate, g.nb, st, bits, g, field, skew);
 }
 
 void launch_encode(const float *field, const Geom &g, uint64_t *bits, float *bmin, float *bmax, cudaStream_t st) {

@@ -408,9 +408,10 @@ __device__ __forceinline__ void decode_staged(const uint32_t *staged, uint32_t r
 // 32-byte sector, so the blocks pass through the warp's plane columns (plane
 // k of its lanes is 256 bytes; the planes are used up), 16-byte pieces
 // swizzled against bank conflicts, and every store writes two whole blocks.
-// Called by all 32 lanes.
+// A caller's buffer that is not 16-byte aligned (`aligned` false, the same in
+// every lane) takes 4-byte stores.  Called by all 32 lanes.
 __device__ __forceinline__ void store_blocks(float *base, uint32_t to, uint32_t have, const float (&v)[64],
-                                             uint64_t *planes, uint32_t stride) {
+                                             uint64_t *planes, uint32_t stride, bool aligned = true) {
     const uint32_t lane = threadIdx.x & 31u, rows = smem_u32(planes) - lane * 8u, ps = stride * 8u;
     __syncwarp();                          // every lane has read its planes
 #pragma unroll
@@ -427,7 +428,16 @@ __device__ __forceinline__ void store_blocks(float *base, uint32_t to, uint32_t 
                      : "=f"(d.x), "=f"(d.y), "=f"(d.z), "=f"(d.w)
                      : "r"(rows + b * ps + ((piece ^ (b & 15u)) << 4)));
         const uint32_t row = __shfl_sync(0xffffffffu, to, (int)b);
-        if ((have >> b) & 1u) *reinterpret_cast<float4 *>(base + (size_t)row * 64 + 4 * piece) = d;
+        float *dst = base + (size_t)row * 64 + 4 * piece;
+        if (!((have >> b) & 1u)) continue;
+        if (aligned) {
+            *reinterpret_cast<float4 *>(dst) = d;
+        } else {
+            dst[0] = d.x;
+            dst[1] = d.y;
+            dst[2] = d.z;
+            dst[3] = d.w;
+        }
     }
 }
 
