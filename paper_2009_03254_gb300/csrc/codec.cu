@@ -33,7 +33,7 @@ __device__ __forceinline__ DecodeSmem codec_smem(uint64_t *base, uint32_t rate) 
 // words to memory one by one and parsed them again for the range took 1160.
 __global__ void __launch_bounds__(kCodecThreads, 4) encode_kernel(const float *__restrict__ field, Geom g, uint64_t *bits,
                                                                float *bmin, float *bmax) {
-    extern __shared__ uint64_t dsm[];
+    extern __shared__ __align__(16) uint64_t dsm[];
     const DecodeSmem sm = decode_smem_layout(dsm, kCodecThreads, g.rate);
     const uint32_t planes = smem_u32(sm.planes + threadIdx.x), ps = 8u * kCodecThreads;
     const uint32_t lane = threadIdx.x & 31u, stride = 2u * g.rate + 1u;   // words a staged block takes
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kCodecThreads, 4) encode_kernel(const float *_
 __global__ void __launch_bounds__(kCodecThreads, 5) decode_list_kernel(const uint64_t *__restrict__ bits, uint32_t rate,
                                                                     const uint32_t *__restrict__ ids, uint64_t n,
                                                                     float *out) {
-    extern __shared__ uint64_t dsm[];
+    extern __shared__ __align__(16) uint64_t dsm[];
     const DecodeSmem sm = codec_smem(dsm, rate);
     const uint32_t lane = threadIdx.x & 31u;
     const bool aligned = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kCodecThreads, 5) decode_list_kernel(const uin
 // span of the bitstream.
 __global__ void __launch_bounds__(kCodecThreads, 5) decode_volume_kernel(const uint64_t *__restrict__ bits, Geom g,
                                                                       float *field, uint32_t skew) {
-    extern __shared__ uint64_t dsm[];
+    extern __shared__ __align__(16) uint64_t dsm[];
     const DecodeSmem sm = codec_smem(dsm, g.rate);
     const bool rows16 = (skew & 3u) == 0;       // every row starts 16-byte aligned
     const uint32_t lane = threadIdx.x & 31u;

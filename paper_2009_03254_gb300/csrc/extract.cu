@@ -517,7 +517,7 @@ template <int kDecodeThreads, bool kOne>
 __global__ void __launch_bounds__(kDecodeThreads, 768 / kDecodeThreads) decode_new_kernel(Launch L) {   // 24 warps/SM
     // dynamic: the plane columns (32 words per thread), then one staging
     // area per warp for the launch's largest rate
-    extern __shared__ uint64_t dsm[];
+    extern __shared__ __align__(16) uint64_t dsm[];
     __shared__ uint32_t pre[kMaxBatch + 1];
     __shared__ TileScan<kRounds> ts;                  // lru_b's work
     __shared__ uint32_t slot_x;
