@@ -626,9 +626,11 @@ typedef struct iso_server_options {
 } iso_server_options;
 
 /* v must not be loaded with ISO_DEBUG.  The server keeps 2 * max_batch
- * request positions (a running tick's and the next tick's), each with
- * candidate, occupied-list, offset and below-mask arrays of min(cache slots,
- * nb) entries (24 bytes each), and creates two streams: the backs run at the
+ * request positions (a running tick's and the next tick's; a control block
+ * and look-back descriptors each) and, for each of the max_batch requests of
+ * a tick, candidate, below-mask, occupied-list, offset and crossing-cell
+ * arrays of min(cache slots, nb) entries (32 bytes a slot together, shared by
+ * the two positions), and creates two streams: the backs run at the
  * device's highest stream priority, the fronts at its lowest, so a front
  * overlapping a back takes only the SMs the back leaves idle.  Meshes are
  * complete when a request finishes (the server waits for its emission). */

@@ -37,8 +37,9 @@
 // tick's union takes more than half the cache (room_to_pin).  An overlapping
 // front also counts the running tick's isovalues as active (pins), so the
 // cache update it makes never evicts a block the running tick reads.  The
-// two ticks use alternate halves of the request positions, so the new front
-// never writes lists the running back reads.  Decoded blocks and all
+// two ticks use alternate halves of the request positions (control blocks and
+// look-back descriptors); the lists need one set, since the new front writes
+// only what the running tick's count has read (Lists).  Decoded blocks and all
 // metadata stay resident between ticks.  If a union does not fit in the
 // cache budget, its requests go back to the queue (an unpinned tick then
 // takes half as many requests, down to one; a pinned one is simply retried
@@ -380,10 +381,27 @@ struct Done {
     iso_mesh mesh;
 };
 
-struct Slot {                           // device state of one request position
+// Device state of one request position (a request of the running tick or of
+// the next one): what the next tick's front clears while the running tick's
+// back still reads its own.
+struct Slot {
     Ctl *ctl = nullptr;
-    uint32_t *icand = nullptr, *iocc = nullptr;
-    unsigned long long *ooff = nullptr, *ocross = nullptr, *bmask = nullptr, *desc_cand = nullptr, *desc_mc = nullptr, *desc_occ = nullptr;
+    unsigned long long *desc_cand = nullptr, *desc_mc = nullptr, *desc_occ = nullptr;
+};
+
+// The arrays of a tick's j-th request, one set for both halves.  Candidates
+// and below masks are written by a front and last read by its tick's count,
+// and no front is launched before the count of the tick ahead of it is done
+// (advance() admits while the back is empty or emitting).  The occupied lists
+// are written by a count and read by the emission rounds, and a count is
+// queued only when the back is empty.  So neither ever holds two ticks' data:
+// 32 bytes a cache slot and request, where a set for each half took 64 (a
+// volume of 250 M slots and 8 requests: 64 GB instead of 128).
+struct Lists {
+    uint32_t *icand = nullptr;
+    unsigned long long *bmask = nullptr;
+    uint32_t *iocc = nullptr;
+    unsigned long long *ooff = nullptr, *ocross = nullptr;
 };
 
 enum Stage { kFront = 0, kCount = 1, kEmit = 2 };
@@ -416,6 +434,7 @@ struct iso_server {
     uint32_t cand_cap = 0;              // room of each request's candidate list
     uint64_t held_bytes = 0;            // finished meshes not yet taken
     Slot slots[2][kMaxServe];           // two halves: a tick's back and the next tick's front
+    Lists lists[kMaxServe];             // shared by the halves
     VolEntry views[2][kMaxServe];       // per-request views of the volume
     VolEntry *d_views[2] = {};          // the same in device memory (the back's launch tables)
     uint32_t *d_ctr[2] = {};            // work counters of each half's back launches
@@ -449,11 +468,11 @@ ServeArgs serve_args(const iso_server *sv, const Tick &t, const std::vector<Requ
     for (uint32_t j = 0; j < a.k; j++) {
         a.iso[j] = t.reqs[j].iso;
         a.ctl[j] = sv->slots[p][j].ctl;
-        a.icand[j] = sv->slots[p][j].icand;
+        a.icand[j] = sv->lists[j].icand;
         a.desc_cand[j] = sv->slots[p][j].desc_cand;
         a.desc_mc[j] = sv->slots[p][j].desc_mc;
         a.desc_occ[j] = sv->slots[p][j].desc_occ;
-        a.bmask[j] = sv->slots[p][j].bmask;
+        a.bmask[j] = sv->lists[j].bmask;
     }
     a.k_pin = pins ? (uint32_t)pins->size() : 0u;
     for (uint32_t j = 0; j < a.k_pin; j++) a.iso[a.k + j] = (*pins)[j].iso;
@@ -478,9 +497,13 @@ void free_server(iso_server *sv) {
         for (float *b : sv->back_tick.bufs) dfree_on(b, sv->stream);
     for (auto &half : sv->slots)
         for (Slot &s : half) {
-            void *p[] = {s.ctl, s.icand, s.bmask, s.ooff, s.ocross, s.desc_cand, s.desc_mc, s.iocc};
+            void *p[] = {s.ctl, s.desc_cand, s.desc_mc};
             for (void *x : p) dfree_on(x, sv->stream);
         }
+    for (Lists &l : sv->lists) {
+        void *p[] = {l.icand, l.bmask, l.iocc, l.ooff, l.ocross};
+        for (void *x : p) dfree_on(x, sv->stream);
+    }
     void *q[] = {sv->d_views[0], sv->d_views[1], sv->d_ctr[0], sv->d_ctr[1], sv->d_ctls[0], sv->d_ctls[1],
                  sv->d_params};
     for (void *x : q) dfree_on(x, sv->stream);
@@ -878,6 +901,14 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
     TRY(cuda_ok(cudaStreamCreateWithPriority(&sv->front, cudaStreamNonBlocking, prio_low)));
     TRY(cuda_ok(cudaEventCreateWithFlags(&sv->count_done, cudaEventDisableTiming)));
     for (cudaEvent_t &e : sv->emit_done) TRY(cuda_ok(cudaEventCreateWithFlags(&e, cudaEventDisableTiming)));
+    for (uint32_t j = 0; j < sv->max_batch; j++) {
+        Lists &l = sv->lists[j];
+        TRY(dalloc_on(&l.icand, cand, sv->device, sv->stream));
+        TRY(dalloc_on(&l.bmask, v->cap, sv->device, sv->stream));
+        TRY(dalloc_on(&l.iocc, cand, sv->device, sv->stream));
+        TRY(dalloc_on(&l.ooff, cand, sv->device, sv->stream));
+        TRY(dalloc_on(&l.ocross, cand + 3, sv->device, sv->stream));   // read four at a time
+    }
     for (int p = 0; p < 2; p++) {
         TRY(cuda_ok(cudaEventCreateWithFlags(&sv->front_done[p], cudaEventDisableTiming)));
         TRY(dalloc_on(&sv->d_views[p], kMaxServe, sv->device, sv->stream));
@@ -886,26 +917,22 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
         for (uint32_t j = 0; j < sv->max_batch; j++) {
             Slot &s = sv->slots[p][j];
             TRY(dalloc_on(&s.ctl, 1, sv->device, sv->stream));
-            TRY(dalloc_on(&s.icand, cand, sv->device, sv->stream));
-            TRY(dalloc_on(&s.bmask, v->cap, sv->device, sv->stream));
-            TRY(dalloc_on(&s.ooff, cand, sv->device, sv->stream));
-            TRY(dalloc_on(&s.ocross, cand + 3, sv->device, sv->stream));   // read four at a time
             TRY(dalloc_on(&s.desc_cand, v->n_cull_desc, sv->device, sv->stream));
             TRY(dalloc_on(&s.desc_mc, 2 * n_mc_desc, sv->device, sv->stream));
             s.desc_occ = s.desc_mc + n_mc_desc;
-            TRY(dalloc_on(&s.iocc, cand, sv->device, sv->stream));
+            const Lists &l = sv->lists[j];
             DevState d = v->s;            // the volume's cache and geometry, the request's own lists
             d.ctl = s.ctl;
-            d.icand = s.icand;
-            d.bmask = s.bmask;
-            d.ooff = s.ooff;
-            d.ocross = s.ocross;
+            d.icand = l.icand;
+            d.bmask = l.bmask;
+            d.ooff = l.ooff;
+            d.ocross = l.ocross;
             d.counts = nullptr;           // the debug accessors' arrays are the volume's
             d.offsets = nullptr;
             d.desc_cand = s.desc_cand;
             d.desc_mc = s.desc_mc;
             d.desc_occ = s.desc_occ;
-            d.iocc = s.iocc;
+            d.iocc = l.iocc;
             d.voff = nullptr;
             d.desc_vtx = nullptr;
             d.dbg_edges = nullptr;
@@ -927,7 +954,7 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
                              st) == cudaSuccess;
         for (uint32_t j = 0; ok && j < sv->max_batch; j++) {
             ok = cudaMemsetAsync(sv->slots[p][j].ctl, 0, sizeof(Ctl), st) == cudaSuccess &&   // no field undefined
-                 cudaMemsetAsync(sv->slots[p][j].icand, 0, cand * 4, st) == cudaSuccess &&
+                 (p != 0 || cudaMemsetAsync(sv->lists[j].icand, 0, cand * 4, st) == cudaSuccess) &&
                  cudaMemsetAsync(sv->slots[p][j].desc_mc, 0, n_mc_desc * 16, st) == cudaSuccess;
         }
     }
