@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <unordered_map>
@@ -319,6 +320,17 @@ int status_to_error(iso_volume *v, uint32_t st) {
     return ISO_OK;
 }
 
+void keep_pass(iso_volume *v, const Ctl &c, bool indexed) {
+    const bool failed = (c.status & (kStatusBudget | kStatusAnyTimeout)) != 0;
+    v->last_n_active = c.n_active;
+    v->last_n_new = c.n_new;
+    v->last_n_cand = c.n_cand;
+    v->last_slots = c.S;
+    v->last_n_occ = failed ? 0u : std::min(c.n_occ, v->s.list_cap);
+    v->last_pass_tris = c.n_tri;
+    v->last_pass_vtx = indexed ? c.n_vtx : 0ull;
+}
+
 void fill_stats(const Ctl &c, iso_stats *st, uint32_t reruns) {
     st->num_triangles = c.n_tri;
     st->n_active = c.n_active;
@@ -364,7 +376,7 @@ int free_volume(iso_volume *v) {
     DevState &s = v->s;
     void *ptrs[] = {v->bits, v->bmin, v->bmax, v->hull, v->hull8, v->seg, v->tables, s.mactive, s.iactive, s.inew, s.icand,
                     s.islot, s.slast, s.sblock, s.lbuf[0], s.lbuf[1], s.newslot, s.slots, s.desc_cull, s.desc_cand,
-                    s.desc_lru_a, s.desc_lru_b, s.desc_mc, s.ctl, s.ihit, s.bmask, s.counts, s.offsets, s.iocc, s.ooff, s.ocross,
+                    s.desc_lru_a, s.desc_lru_b, s.desc_mc, s.ctl, s.ihit, s.bmask, s.iocc, s.ooff, s.ocross,
                     s.cases, s.dbg_edges, s.voff};
     for (void *p : ptrs) dfree_on(p, v->stream);
     cudaStreamSynchronize(v->stream);
@@ -531,12 +543,7 @@ int run(iso_volume *v, float iso, void *out, unsigned long long cap_tris, Phase 
         v->split_emit = phase == Phase::kEmit;
         collect_stage_times(v);
     }
-    if (phase != Phase::kEmit) {
-        v->last_n_active = v->host_ctl->n_active;
-        v->last_n_new = v->host_ctl->n_new;
-        v->last_n_cand = v->host_ctl->n_cand;
-        v->last_slots = v->host_ctl->S;
-    }
+    if (phase != Phase::kEmit) keep_pass(v, *v->host_ctl, indexed);
     v->last_tris = v->host_ctl->n_tri;
     v->last_vtx = indexed ? v->host_ctl->n_vtx : 0ull;
     return status_to_error(v, v->host_ctl->status);
@@ -636,6 +643,35 @@ int extract_to(iso_volume *v, float iso, void *out, unsigned long long cap_tris,
         stats->num_vertices = ix ? v->host_ctl->n_vtx : 0ull;
     }
     return rc;
+}
+
+// Triangles (and vertices, from bit 16 on) or offsets of the last count's n
+// candidates, host arrays, either of them: the count keeps offsets only for
+// the occupied candidates, and both lists are in ascending block order, so
+// the others are those in between.
+int candidate_counts(iso_volume *v, uint32_t *tris, uint64_t *offsets, uint64_t n) {
+    const uint32_t n_occ = v->last_n_occ;
+    const bool indexed = v->last_pass_vtx != 0;
+    std::unique_ptr<uint32_t[]> cand(new (std::nothrow) uint32_t[n]), occ(new (std::nothrow) uint32_t[n_occ + 1u]);
+    std::unique_ptr<uint64_t[]> first(new (std::nothrow) uint64_t[n_occ + 1u]),
+        vtx(indexed ? new (std::nothrow) uint64_t[n_occ + 1u] : nullptr);
+    if (!cand || !occ || !first || (indexed && !vtx)) return ISO_ERR_OOM;
+    CK(cudaMemcpy(cand.get(), v->s.icand, n * 4, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(occ.get(), v->s.iocc, (size_t)n_occ * 4, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(first.get(), v->s.ooff, (size_t)n_occ * 8, cudaMemcpyDeviceToHost));
+    if (indexed) CK(cudaMemcpy(vtx.get(), v->s.voff, (size_t)n_occ * 8, cudaMemcpyDeviceToHost));
+    first[n_occ] = v->last_pass_tris;
+    if (indexed) vtx[n_occ] = v->last_pass_vtx;
+    uint32_t k = 0;                                  // the first occupied candidate not before i
+    for (uint64_t i = 0; i < n; i++) {
+        if (offsets) offsets[i] = first[k];
+        const bool is = k < n_occ && occ[k] == cand[i];
+        if (tris) tris[i] = is ? (uint32_t)(first[k + 1] - first[k]) |
+                                     (indexed ? (uint32_t)(vtx[k + 1] - vtx[k]) << 16 : 0u)
+                               : 0u;
+        if (is) k++;
+    }
+    return ISO_OK;
 }
 
 // built once per process (a function-local static: thread-safe initialisation,
@@ -838,8 +874,6 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     s.desc_occ = s.desc_mc + n_mc_desc;
     s.desc_vtx = s.desc_occ + n_mc_desc;
     TRY(dalloc(v, &s.ctl, 1));
-    TRY(dalloc(v, &s.counts, v->cap));
-    TRY(dalloc(v, &s.offsets, v->cap));
     TRY(dalloc(v, &s.iocc, s.list_cap));
     TRY(dalloc(v, &s.ooff, s.list_cap));
     TRY(dalloc(v, &s.ocross, (size_t)s.list_cap + 3));   // read four at a time
@@ -1167,8 +1201,8 @@ int iso_debug_get(iso_volume *v, int which, void *host_dst, size_t bytes, uint64
         case ISO_DBG_CELL_CASES:
             if (!dbg || !v->s.cases) return ISO_ERR_INVALID_ARG;
             src = v->s.cases; n = 64ull * std::min<uint64_t>(v->last_n_cand, v->s.list_cap); elem = 1; break;
-        case ISO_DBG_BLOCK_TRIS: src = v->s.counts; n = v->last_n_cand; elem = 4; break;
-        case ISO_DBG_BLOCK_OFFSETS: src = v->s.offsets; n = v->last_n_cand; elem = 8; break;
+        case ISO_DBG_BLOCK_TRIS: n = std::min<uint64_t>(v->last_n_cand, v->s.list_cap); elem = 4; break;
+        case ISO_DBG_BLOCK_OFFSETS: n = std::min<uint64_t>(v->last_n_cand, v->s.list_cap); elem = 8; break;
         case ISO_DBG_CANDIDATES: src = v->s.icand; n = std::min<uint64_t>(v->last_n_cand, v->s.list_cap); elem = 4; break;
         case ISO_DBG_EDGE_IDS:
             if (!dbg) return ISO_ERR_INVALID_ARG;
@@ -1182,6 +1216,9 @@ int iso_debug_get(iso_volume *v, int which, void *host_dst, size_t bytes, uint64
     if (n == 0) return ISO_OK;
     if (!host_dst || bytes < n * elem) return ISO_ERR_CAPACITY;
     CK(cudaStreamSynchronize(v->stream));
+    if (which == ISO_DBG_BLOCK_TRIS || which == ISO_DBG_BLOCK_OFFSETS)
+        return candidate_counts(v, which == ISO_DBG_BLOCK_TRIS ? static_cast<uint32_t *>(host_dst) : nullptr,
+                                which == ISO_DBG_BLOCK_OFFSETS ? static_cast<uint64_t *>(host_dst) : nullptr, n);
     CK(cudaMemcpy(host_dst, src, n * elem, cudaMemcpyDeviceToHost));
     return ISO_OK;
 }

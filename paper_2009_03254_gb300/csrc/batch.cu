@@ -159,10 +159,7 @@ int finish_batch(iso_batch *b, iso_stats *stats, int *status) {
     for (uint32_t i = 0; i < b->n; i++) {
         iso_volume *v = b->vols[i];
         *v->host_ctl = b->h_ctls[i];
-        v->last_n_active = v->host_ctl->n_active;
-        v->last_n_new = v->host_ctl->n_new;
-        v->last_n_cand = v->host_ctl->n_cand;
-        v->last_slots = v->host_ctl->S;
+        keep_pass(v, *v->host_ctl, false);
         v->last_tris = v->host_ctl->n_tri;
         const int rc = status_to_error(v, v->host_ctl->status);
         if (stats) fill_stats(*v->host_ctl, &stats[i], 0);

@@ -37,8 +37,6 @@ struct DevState {
     unsigned long long *bmask; // per slot: bit i says sample i of its block is below this extraction's
                                // isovalue (active blocks only; null where nothing counts: a serving
                                // tick of several requests takes each request's masks on its own)
-    uint32_t *counts;          // debug access: triangles of each candidate (null in a request's view)
-    unsigned long long *offsets; // debug access: exclusive prefix of counts (null in a request's view)
     uint32_t *iocc;            // I_occ: ids of the occupied candidates (ascending)
     unsigned long long *ooff;  // first triangle of each occupied candidate
     unsigned long long *ocross;  // its crossing cells, bit x + 4y + 16z

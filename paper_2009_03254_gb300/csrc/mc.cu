@@ -386,7 +386,6 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
                 const unsigned long long valid = valid_cells(lim);
                 nt = count_triangles(m, valid, sm.cross[r][threadIdx.x]);
                 if (kIdx) nv = count_vertices(m, valid, lim);
-                if (s.counts) s.counts[i] = nt | (nv << 16);
             }
             uint32_t incl = nt;
 #pragma unroll
@@ -436,7 +435,6 @@ __global__ void __launch_bounds__(kThreads, 4) mc_scan_kernel(Launch L) {
                 }
                 vrun = sm.vtx.excl + sm.vtx.cnt[r][warp] + (vincl - nv);
             }
-            if (i < n && s.offsets) s.offsets[i] = run;
             const uint32_t at = (uint32_t)sm.occ.excl + sm.occ.cnt[r][warp] + __popc(ob & lt);
             if (nt && in_bounds(at < s.list_cap, &c->status)) {
                 s.iocc[at] = s.icand[i];

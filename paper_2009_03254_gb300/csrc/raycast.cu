@@ -607,10 +607,7 @@ extern "C" int iso_raycast(iso_volume *v, float isovalue, const iso_pinhole *cam
         (void)cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? ISO_ERR_OOM : ISO_ERR_CUDA;
     }
-    v->last_n_active = v->host_ctl->n_active;
-    v->last_n_new = v->host_ctl->n_new;
-    v->last_n_cand = v->host_ctl->n_cand;
-    v->last_slots = v->host_ctl->S;
+    keep_pass(v, *v->host_ctl, false);               // (no triangles are counted)
     v->last_tris = 0;
     rc = status_to_error(v, v->host_ctl->status);
     if (rc) return rc;

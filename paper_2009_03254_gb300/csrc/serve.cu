@@ -927,8 +927,6 @@ int iso_server_create(iso_server **out, iso_volume *v, const iso_server_options 
             d.bmask = l.bmask;
             d.ooff = l.ooff;
             d.ocross = l.ocross;
-            d.counts = nullptr;           // the debug accessors' arrays are the volume's
-            d.offsets = nullptr;
             d.desc_cand = s.desc_cand;
             d.desc_mc = s.desc_mc;
             d.desc_occ = s.desc_occ;

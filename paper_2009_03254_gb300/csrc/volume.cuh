@@ -56,6 +56,9 @@ struct iso_volume {
     float stage_ms[ISO_NUM_STAGES] = {};
     unsigned long long last_tris = 0;
     uint32_t last_n_active = 0, last_n_new = 0, last_n_cand = 0, last_slots = 0;
+    // what the last count left in the occupied lists (a wave's, not its surface's)
+    uint32_t last_n_occ = 0;
+    unsigned long long last_pass_tris = 0, last_pass_vtx = 0;
 };
 
 namespace bcmc_host {
@@ -110,6 +113,9 @@ struct DeviceGuard {              // make a device current for the call
         if (prev >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != prev) cudaSetDevice(prev);
     }
 };
+
+// Keep what a pass's control block says of the pass, for later calls.
+void keep_pass(iso_volume *v, const bcmc::Ctl &c, bool indexed);
 
 // Error of an extraction from its status bits.  After a timeout the
 // volume's cache bookkeeping may be inconsistent: it is emptied on the

@@ -90,3 +90,54 @@ def test_ticks_that_share_lists_keep_apart(max_batch, budget):
         srv.release()
         vol.release()
         alone.release()
+
+
+def test_volume_bytes_a_block(held):
+    import torch
+    dims, rate = (160, 160, 240), 2
+    nb = int(np.prod(oracle.block_dims(dims)))
+    bits = torch.zeros((nb, rate), dtype=torch.int64, device="cuda")
+    rng = torch.zeros(nb, dtype=torch.float32, device="cuda")
+    before = held()
+    vol = pkg().Volume(bits, dims, rate, rng, rng)
+    try:
+        # bitstream, two hulls, slot map, samples, then nine lists of 4 bytes
+        # a slot and three of 8; a byte for what is kept by the tile
+        assert held() - before <= (8 * rate + 16 + 4 + 256 + 9 * 4 + 3 * 8 + 1) * nb
+    finally:
+        vol.release()
+
+
+def by_candidate(vol, ref, vertices=None):
+    cand = vol.debug("candidates")
+    at = np.searchsorted(ref["ids"], cand)
+    assert np.array_equal(ref["ids"][at], cand)
+    tris = vol.debug("block_tris")
+    assert np.array_equal(tris & 0xFFFF, ref["block_tri"][at])
+    assert (tris >> 16).sum() == (vertices or 0) and not (tris >> 16)[ref["block_tri"][at] == 0].any()
+    assert np.array_equal(vol.debug("block_offsets"), ref["block_off"][at])
+
+
+# the triangles and offsets of every candidate, which no extraction writes:
+# after soups, indexed meshes and a cache reset, and none after a ray cast
+def test_candidates_counts_on_request():
+    p = pkg()
+    dims, rate = (41, 34, 27), 8
+    bits, bmin, bmax = noise(dims, rate)
+    vol = p.Volume(bits, dims, rate, bmin, bmax)
+    try:
+        for iso in (0.1, -0.4):
+            ref = oracle.extract(bits, dims, rate, bmin, bmax, iso)
+            vol.extract(iso).release()
+            by_candidate(vol, ref)
+            vol.cache_reset()
+            by_candidate(vol, ref)
+            verts, idx, st = vol.extract_indexed(iso)
+            by_candidate(vol, ref, st["num_vertices"])
+        vol.extract(float(bmax.max()) + 1.0).release()
+        assert len(vol.debug("block_tris")) == 0
+        vol.raycast(0.1, (-9, 15, 12), (1, 0, 0), (0, 1, 0), (0, 0, 1), (0, 0, 1), 16, 16)
+        assert len(vol.debug("block_tris")) == len(vol.debug("candidates")) > 0
+        assert not vol.debug("block_tris").any()
+    finally:
+        vol.release()
