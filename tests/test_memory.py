@@ -1,7 +1,7 @@
 """Device memory the calls hold: bytes a cache slot of a server's request
 lists, and that the lists which two ticks share never mix their requests.
 PyTorch's caching allocator serves the library here, so its own count of
-allocated bytes is the measure (rounded up to 512 bytes an allocation)."""
+requested bytes is the measure."""
 import numpy as np
 import pytest
 
@@ -20,14 +20,15 @@ def built():
 
 @pytest.fixture
 def held():
-    """held(): bytes the library holds, through PyTorch's allocator"""
+    """held(): bytes asked of PyTorch's allocator and not given back (with the
+    library's among them); held(peak=True): the most since the last reset"""
     import torch
     torch.cuda.synchronize()
     pkg().use_torch_allocator()
 
-    def count():
+    def count(peak=False):
         torch.cuda.synchronize()
-        return torch.cuda.memory_allocated()
+        return torch.cuda.memory_stats()["requested_bytes.all." + ("peak" if peak else "current")]
     try:
         yield count
     finally:
