@@ -39,7 +39,7 @@ struct DevState {
                                // tick of several requests takes each request's masks on its own)
     uint32_t *iocc;            // I_occ: ids of the occupied candidates (ascending)
     unsigned long long *ooff;  // first triangle of each occupied candidate
-    unsigned long long *ocross;  // its crossing cells, bit x + 4y + 16z
+    unsigned long long *ocross;  // its crossing cells, bit x + 4y + 16z (a ray cast: by slot)
     unsigned long long *desc_occ;  // look-back descriptors of the occupied count (next to desc_mc)
     unsigned long long *desc_vtx;  // look-back descriptors of the vertex count (next to desc_occ; null
                                    // where indexed meshes are never made)

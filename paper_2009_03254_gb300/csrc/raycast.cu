@@ -557,14 +557,15 @@ extern "C" int iso_raycast(iso_volume *v, float isovalue, const iso_pinhole *cam
     ISO_CK(cudaMemcpyAsync(&v->s.ctl->params, v->host_params, sizeof(Params), cudaMemcpyHostToDevice, st));
     const Launch L{nullptr, 1u, single_counters(v), VolEntry{v->s, v->g, v->n_cull_desc, v->n_lru_desc}};
     launch_front(L, v->plan, st, nullptr);
-    // counters, a bit per block, then the slots' crossing cells
+    // counters, then a bit per block.  The slots' crossing cells go where an
+    // extraction keeps its occupied candidates' (no emission follows, and there
+    // are as many entries as slots), so a cast holds next to nothing of its own
     void *scratch = nullptr;
-    const size_t occ_at = 256, occ_bytes = ((size_t)v->g.nb + 31) / 32 * 4,
-                 cross_at = occ_at + (occ_bytes + 255) / 256 * 256;
-    int rc = dalloc_bytes(&scratch, cross_at + (size_t)v->cap * 8, v->device, st);
+    const size_t occ_at = 256, occ_bytes = ((size_t)v->g.nb + 31) / 32 * 4;
+    int rc = dalloc_bytes(&scratch, occ_at + occ_bytes, v->device, st);
     if (rc) return rc;
     uint32_t *occ = reinterpret_cast<uint32_t *>(static_cast<char *>(scratch) + occ_at);
-    unsigned long long *cross = reinterpret_cast<unsigned long long *>(static_cast<char *>(scratch) + cross_at);
+    unsigned long long *cross = v->s.ocross;
     CastArgs a{};
     a.islot = v->s.islot;
     a.slots = v->s.slots;

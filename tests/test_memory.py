@@ -142,3 +142,30 @@ def test_candidates_counts_on_request():
         assert not vol.debug("block_tris").any()
     finally:
         vol.release()
+
+
+# a cast's own memory is a bit a block, and what it leaves in the volume's
+# lists does not reach the extractions after it
+def test_raycast_bytes_a_block(held):
+    import torch
+    p = pkg()
+    dims, rate = (120, 96, 100), 8
+    nb = int(np.prod(oracle.block_dims(dims)))
+    bits, bmin, bmax = noise(dims, rate)
+    vol = p.Volume(bits, dims, rate, bmin, bmax)
+    cam = ((-40, 48, 50), (1, 0, 0), (0, 0.8, 0), (0, 0, 0.8), (0, 0, 1), 64, 48)
+    hits, rgba = (torch.empty((48, 64), dtype=d, device="cuda") for d in (torch.int64, torch.int32))
+    try:
+        m = vol.extract(0.2)
+        want = m.vertices.cpu().numpy().view(np.uint32).copy()
+        m.release()
+        before = held()
+        torch.cuda.reset_peak_memory_stats()
+        vol.raycast(-0.3, *cam, hits=hits, rgba=rgba)
+        assert held(peak=True) - before <= nb // 8 + 2048
+        assert int((hits != -1).sum()) > 0
+        m = vol.extract(0.2)
+        assert np.array_equal(m.vertices.cpu().numpy().view(np.uint32), want)
+        m.release()
+    finally:
+        vol.release()
