@@ -567,7 +567,8 @@ int iso_batch_get_shape(const iso_batch *b, iso_launch_shape *shape);
  * The chosen shape is applied if the whole batch runs faster with it than
  * with the defaults, and returned in *best; best_ms[0] and best_ms[1] (may
  * be NULL) receive the cold-cache batch time of the default shape and of
- * the applied one.  The caches are left empty. */
+ * the applied one.  The fields without effect (count_ctas, count_tile,
+ * scan_tile) come back as their defaults.  The caches are left empty. */
 int iso_batch_tune(iso_batch *b, const float *isovalues, float *d_vertices, uint64_t capacity_triangles,
                    int trials, iso_launch_shape *best, float *best_ms);
 

@@ -33,7 +33,7 @@ std::mutex g_pool_mutex;
 cudaMemPool_t g_pool[kMaxPoolDevices] = {};
 struct OccEntry {
     int device;
-    int key[8];                   // tile sizes, single/batch, largest rate, segment ranges
+    int key[6];                   // tile sizes, single/batch, largest rate, segment ranges
     Plan limits;
 };
 std::vector<OccEntry> g_occ;      // occupancy limits per (device, tile variants)
@@ -200,8 +200,8 @@ void dfree_on(void *p, cudaStream_t st) {
     else cudaFreeAsync(p, st);
 }
 
-int shape_to_want(const iso_launch_shape *shape, Plan *out) {
-    Plan w{};
+int shape_to_want(const iso_launch_shape *shape, WantedPlan *out) {
+    WantedPlan w{};
     // CTAs per SM beyond any occupancy limit mean "the limit"; tile sizes
     // are checked exactly (values that do not fit an int are invalid)
     auto c = [](uint32_t x) { return (int)std::min<uint32_t>(x, 1024u); };
@@ -211,26 +211,28 @@ int shape_to_want(const iso_launch_shape *shape, Plan *out) {
     w.lru_a = w.lru_b = c(shape->cache_update_ctas);
     w.decode = c(shape->decode_ctas);
     w.decode_tile = t(shape->decode_tile);
-    w.mc_count = c(shape->count_ctas);
     w.count_tile = t(shape->count_tile);
     w.mc_scan = c(shape->scan_ctas);
     w.scan_tile = t(shape->scan_tile);
     w.mc_emit = c(shape->emit_ctas);
     w.emit_tile = t(shape->emit_tile);
-    if (!valid_tiles(default_tiles(&w))) return ISO_ERR_INVALID_ARG;
+    const bool unused_ok = (w.count_tile == 0 || w.count_tile == 16 || w.count_tile == 32 || w.count_tile == 64) &&
+                           (w.scan_tile == 0 || w.scan_tile == 1024 || w.scan_tile == 2048 || w.scan_tile == 4096);
+    if (!unused_ok || !valid_tiles(default_tiles(&w))) return ISO_ERR_INVALID_ARG;
     *out = w;
     return ISO_OK;
 }
 
-iso_launch_shape shape_of(const Plan &want, int device, bool single, uint32_t max_rate, bool seg) {
+iso_launch_shape shape_of(const WantedPlan &want, int device, bool single, uint32_t max_rate, bool seg) {
     // CTAs per SM that run: the requested number clamped to the occupancy limit
     const Plan tiles = default_tiles(&want);
     const Plan lim = occupancy_limits_of(device, tiles, single, max_rate, seg);
     auto run = [](int w, int mx) { return (uint32_t)(w > 0 ? std::min(w, mx) : mx); };
     return iso_launch_shape{run(want.cull, lim.cull), (uint32_t)tiles.cull_tile, run(want.lru_a, lim.lru_a),
                             run(want.decode, lim.decode), (uint32_t)tiles.decode_tile,
-                            run(want.mc_count, lim.mc_count), (uint32_t)tiles.count_tile,
-                            run(want.mc_scan, lim.mc_scan), (uint32_t)tiles.scan_tile,
+                            1u, (uint32_t)(want.count_tile ? want.count_tile : kDefaultCountTile),
+                            run(want.mc_scan, lim.mc_scan),
+                            (uint32_t)(want.scan_tile ? want.scan_tile : kDefaultScanTile),
                             run(want.mc_emit, lim.mc_emit), (uint32_t)tiles.emit_tile};
 }
 
@@ -256,19 +258,17 @@ Plan default_tiles(const Plan *want) {
     Plan t{};
     t.cull_tile = want && want->cull_tile ? want->cull_tile : kDefaultCullTile;
     t.decode_tile = want && want->decode_tile ? want->decode_tile : kDefaultDecodeTile;
-    t.count_tile = want && want->count_tile ? want->count_tile : kDefaultCountTile;
-    t.scan_tile = want && want->scan_tile ? want->scan_tile : kDefaultScanTile;
     t.emit_tile = want && want->emit_tile ? want->emit_tile : kDefaultEmitTile;
     return t;
 }
 
 Plan occupancy_limits_of(int device, const Plan &tiles, bool single, uint32_t max_rate, bool seg) {
-    const int key[8] = {tiles.cull_tile, tiles.decode_tile, tiles.count_tile, tiles.scan_tile, tiles.emit_tile,
-                        single ? 1 : 0, (int)max_rate, seg ? 1 : 0};
+    const int key[6] = {tiles.cull_tile, tiles.decode_tile, tiles.emit_tile, single ? 1 : 0, (int)max_rate,
+                        seg ? 1 : 0};
     std::lock_guard<std::mutex> lock(g_pool_mutex);
     for (const OccEntry &e : g_occ)
-        if (e.device == device && std::equal(key, key + 8, e.key)) return e.limits;
-    OccEntry e{device, {key[0], key[1], key[2], key[3], key[4], key[5], key[6], key[7]},
+        if (e.device == device && std::equal(key, key + 6, e.key)) return e.limits;
+    OccEntry e{device, {key[0], key[1], key[2], key[3], key[4], key[5]},
                occupancy_limits(tiles, single, max_rate, seg)};
     g_occ.push_back(e);
     return e.limits;
@@ -282,7 +282,7 @@ Plan launch_plan(const Plan *want, int device, uint64_t total_blocks, uint64_t t
     if (want) {
         int *dst = &use.prep;
         const int *src = &want->prep, *mx = &lim.prep;
-        for (int k = 0; k < 8; k++) dst[k] = src[k] > 0 ? std::min(src[k], mx[k]) : mx[k];
+        for (int k = 0; k < kPlanKernels; k++) dst[k] = src[k] > 0 ? std::min(src[k], mx[k]) : mx[k];
     }
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0) {
@@ -290,7 +290,7 @@ Plan launch_plan(const Plan *want, int device, uint64_t total_blocks, uint64_t t
         sms = 1;
     }
     int *ctas = &use.prep;
-    for (int k = 0; k < 8; k++) ctas[k] = std::max(1, ctas[k]) * sms;
+    for (int k = 0; k < kPlanKernels; k++) ctas[k] = std::max(1, ctas[k]) * sms;
     use.mc_scan = std::min(use.mc_scan, (int)kMaxCountCtas);
     // no more CTAs than work items (each bound holds for any isovalue)
     auto clamp = [](int &grid, uint64_t items) {
@@ -709,7 +709,7 @@ extern "C" {
 
 int iso_set_shape(iso_volume *v, const iso_launch_shape *shape) {
     if (!v || !shape) return ISO_ERR_INVALID_ARG;
-    Plan w{};
+    WantedPlan w{};
     const int rc = shape_to_want(shape, &w);
     if (rc) return rc;
     DeviceGuard dg(v->device);
@@ -971,8 +971,8 @@ int iso_load_volume(iso_volume **out, const void *compressed, size_t compressed_
     }
     // single-volume defaults (128-block decode CTAs, with the list append in
     // its own kernel, beat 256-block CTAs that append after decoding)
-    v->want = Plan{};
-    v->want.scan_tile = 4096;         // reported; the count and scan has one tile size
+    v->want = WantedPlan{};
+    v->want.scan_tile = 4096;         // reported only
     v->plan = launch_plan(&v->want, v->device, g.nb, v->cap, 1, true, g.rate, v->seg != nullptr);
     TRYC(cudaGetLastError());
     *out = v;

@@ -22,8 +22,8 @@ using namespace bcmc;
 using namespace bcmc_host;
 
 namespace {
-constexpr int kBatchEvents = 8;   // before, after prep, cull, cache update, decode, count, scan, emit
-constexpr int kKernels = 6;       // tuned kernels: cull, cache update, decode, count, scan, emit
+constexpr int kBatchEvents = 7;   // before, after prep, cull, cache update, decode, count and scan, emit
+constexpr int kKernels = 5;       // tuned kernels: cull, cache update, decode, count and scan, emit
 constexpr int kVariants = 3;      // tile-size variants per kernel (at most)
 }  // namespace
 
@@ -42,7 +42,7 @@ struct iso_batch {
     BatchOut *h_bo = nullptr;
     Ctl *h_ctls = nullptr;
     unsigned long long *h_tri_base = nullptr;
-    Plan want{};                          // launch shape: CTAs per SM and tiles, 0 = default
+    WantedPlan want{};                    // launch shape: CTAs per SM and tiles, 0 = default
     Plan plan{};                          // what runs
     uint64_t total_blocks = 0, total_slots = 0;
     uint32_t max_rate = 1;                // the largest rate among the volumes
@@ -61,20 +61,21 @@ Launch launch_of(const iso_batch *b) {
 }
 
 // per tuned kernel: its CTA field and tile field in a Plan (tile: null
-// for the cache update, which has one tile size), and the tile variants
+// for the cache update and the count, which have no choice), and the tile
+// variants
 int *ctas_field(Plan &p, int k) {
-    int *f[kKernels] = {&p.cull, &p.lru_a, &p.decode, &p.mc_count, &p.mc_scan, &p.mc_emit};
+    int *f[kKernels] = {&p.cull, &p.lru_a, &p.decode, &p.mc_scan, &p.mc_emit};
     return f[k];
 }
 
 int *tile_field(Plan &p, int k) {
-    int *f[kKernels] = {&p.cull_tile, nullptr, &p.decode_tile, &p.count_tile, &p.scan_tile, &p.emit_tile};
+    int *f[kKernels] = {&p.cull_tile, nullptr, &p.decode_tile, nullptr, &p.emit_tile};
     return f[k];
 }
 
 constexpr int kTileVariants[kKernels][kVariants] = {
-    {2048, 4096, 4096}, {0, 0, 0}, {64, 128, 256}, {16, 32, 64}, {1024, 2048, 4096}, {16, 32, 64}};
-constexpr int kNumVariants[kKernels] = {2, 1, 3, 3, 3, 3};
+    {2048, 4096, 4096}, {0, 0, 0}, {64, 128, 256}, {0, 0, 0}, {16, 32, 64}};
+constexpr int kNumVariants[kKernels] = {2, 1, 3, 1, 3};
 
 void set_ctas(Plan &p, int k, int ctas) {
     *ctas_field(p, k) = ctas;
@@ -88,7 +89,7 @@ void drop_graph(iso_batch *b) {
     b->graph = nullptr;
 }
 
-void apply_shape(iso_batch *b, const Plan &want) {
+void apply_shape(iso_batch *b, const WantedPlan &want) {
     b->want = want;
     b->plan = launch_plan(&b->want, b->device, b->total_blocks, b->total_slots, b->n, false, b->max_rate,
                           b->seg_any != 0);
@@ -103,12 +104,11 @@ int enqueue_batch(iso_batch *b, cudaStream_t st, bool prof) {
     if (prof) cudaEventRecord(b->ev[0], st);
     launch_batch_params(L, b->d_iso, st);
     launch_front(L, b->plan, st, prof ? b->ev : nullptr);
-    if (prof) cudaEventRecord(b->ev[5], st);             // no kernel of the count's own: the scan counts
     launch_mc_scan(L, false, b->plan, st);
-    if (prof) cudaEventRecord(b->ev[6], st);
+    if (prof) cudaEventRecord(b->ev[5], st);
     launch_batch_offsets(L, b->d_bo, b->d_tri_base, st);
     launch_mc_emit(L, false, b->plan, st);
-    if (prof) cudaEventRecord(b->ev[7], st);
+    if (prof) cudaEventRecord(b->ev[6], st);
     launch_batch_gather(L, b->d_ctls, st);
     ISO_CK(cudaMemcpyAsync(b->h_ctls, b->d_ctls, b->n * sizeof(Ctl), cudaMemcpyDeviceToHost, st));
     ISO_CK(cudaMemcpyAsync(b->h_tri_base, b->d_tri_base, (b->n + 1) * sizeof(unsigned long long),
@@ -277,7 +277,7 @@ int iso_batch_create(iso_batch **out, iso_volume *const *volumes, uint32_t n, vo
         return ISO_ERR_CUDA;
     }
 #undef TRY
-    apply_shape(b, Plan{});
+    apply_shape(b, WantedPlan{});
     *out = b;
     return ISO_OK;
 }
@@ -300,7 +300,7 @@ int iso_batch_extract(iso_batch *b, const float *isovalues, float *d_vertices, u
 int iso_batch_set_shape(iso_batch *b, const iso_launch_shape *shape) {
     if (!b || !shape) return ISO_ERR_INVALID_ARG;
     DeviceGuard dg(b->device);
-    Plan w{};
+    WantedPlan w{};
     const int rc = shape_to_want(shape, &w);
     if (rc) return rc;
     apply_shape(b, w);
@@ -319,7 +319,7 @@ int iso_batch_tune(iso_batch *b, const float *isovalues, float *d_vertices, uint
     DeviceGuard dg(b->device);
     int rc = set_inputs(b, isovalues, d_vertices, capacity_triangles);
     if (rc) return rc;
-    const Plan keep = b->want;
+    const WantedPlan keep = b->want;
     // one cold run with `want`: per-kernel times (ms) and the total
     auto timed = [&](const Plan &want, float *kernel_ms, float *total_ms) -> int {
         b->plan = launch_plan(&want, b->device, b->total_blocks, b->total_slots, b->n, false, b->max_rate,
@@ -335,7 +335,7 @@ int iso_batch_tune(iso_batch *b, const float *isovalues, float *d_vertices, uint
             ISO_CK(cudaEventElapsedTime(&ms, b->ev[k + 1], b->ev[k + 2]));
             kernel_ms[k] = ms;
         }
-        ISO_CK(cudaEventElapsedTime(total_ms, b->ev[0], b->ev[7]));
+        ISO_CK(cudaEventElapsedTime(total_ms, b->ev[0], b->ev[6]));
         return ISO_OK;
     };
     float best_t[kKernels];
@@ -373,7 +373,7 @@ int iso_batch_tune(iso_batch *b, const float *isovalues, float *d_vertices, uint
             }
         }
     }
-    Plan chosen{};
+    WantedPlan chosen{};
     for (int k = 0; k < kKernels; k++) {
         set_ctas(chosen, k, best_ctas[k]);
         if (tile_field(chosen, k)) *tile_field(chosen, k) = best_tile[k];
@@ -388,7 +388,7 @@ int iso_batch_tune(iso_batch *b, const float *isovalues, float *d_vertices, uint
         if (rc) { apply_shape(b, keep); return rc; }
         chosen_ms = std::min(chosen_ms, tot);
     }
-    apply_shape(b, chosen_ms <= default_ms ? chosen : Plan{});
+    apply_shape(b, chosen_ms <= default_ms ? chosen : WantedPlan{});
     rc = reset_caches(b);
     if (rc) return rc;
     if (best) rc = iso_batch_get_shape(b, best);

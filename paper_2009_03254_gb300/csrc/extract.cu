@@ -888,8 +888,6 @@ Plan occupancy_limits(const Plan &tiles, bool single, uint32_t rate, bool seg) {
 bool valid_tiles(const Plan &pl) {
     return (pl.cull_tile == 2048 || pl.cull_tile == 4096) &&
            (pl.decode_tile == 64 || pl.decode_tile == 128 || pl.decode_tile == 256) &&
-           (pl.count_tile == 16 || pl.count_tile == 32 || pl.count_tile == 64) &&
-           (pl.scan_tile == 1024 || pl.scan_tile == 2048 || pl.scan_tile == 4096) &&
            (pl.emit_tile == 16 || pl.emit_tile == 32 || pl.emit_tile == 64);
 }
 

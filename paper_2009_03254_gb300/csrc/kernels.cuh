@@ -79,13 +79,18 @@ struct Launch {
 // tile size of each kernel that has a choice.  Any choice computes the
 // same results; the batch autotuner picks the fastest.
 struct Plan {
-    int prep, cull, lru_a, lru_b, decode, mc_count, mc_scan, mc_emit;   // CTAs per launch
+    int prep, cull, lru_a, lru_b, decode, mc_scan, mc_emit;   // CTAs per launch
     int cull_tile;       // block ranges per cull tile: 2048 or 4096
     int decode_tile;     // new blocks per decode CTA (one per thread): 64, 128 or 256
-    int count_tile;      // 16, 32 or 64, and
-    int scan_tile;       // 1024, 2048 or 4096: checked and reported; one kernel counts and scans, in
-                         // tiles of kCountTile
     int emit_tile;       // candidates per emit CTA round (4 per warp): 16, 32 or 64
+};
+constexpr int kPlanKernels = 7;          // its CTA fields
+
+// A launch shape as a caller asked for it (0: default): the plan, and the
+// tile sizes of a count and a scan of their own, which are checked and
+// reported but choose nothing (one kernel counts and scans).
+struct WantedPlan : Plan {
+    int count_tile, scan_tile;
 };
 
 constexpr int kThreads = 256;
@@ -99,8 +104,8 @@ inline uint64_t count_descs(uint64_t n) {
     const uint64_t one = (n + kThreads - 1) / kThreads;
     return (one < kMaxCountCtas ? one : kMaxCountCtas) + (n + kCountTile - 1) / kCountTile;
 }
-constexpr int kDefaultCullTile = 4096, kDefaultDecodeTile = 128, kDefaultCountTile = 32,
-              kDefaultScanTile = 2048, kDefaultEmitTile = 32;
+constexpr int kDefaultCullTile = 4096, kDefaultDecodeTile = 128, kDefaultEmitTile = 32;
+constexpr int kDefaultCountTile = 32, kDefaultScanTile = 2048;   // reported only
 
 // The isovalue, output buffer and its capacity are read from Ctl::params.
 // Front of the pipeline: prep, cull, cache update (two kernels), decode.

@@ -966,7 +966,6 @@ void mc_occupancy(Plan *pl, bool single) {
     // every variant's shared-memory limit is raised, whichever is asked for
     const int e4 = emit_occupancy<4>(single), e8 = emit_occupancy<8>(single), e16 = emit_occupancy<16>(single);
     pl->mc_emit = std::max(1, pl->emit_tile == 16 ? e4 : (pl->emit_tile == 64 ? e16 : e8));
-    pl->mc_count = 1;
     // the soup's and the indexed mesh's counts share the CTA count
     pl->mc_scan = single ? std::min(occupancy(mc_scan_kernel<true, false>, kThreads, 0),
                                     occupancy(mc_scan_kernel<true, true>, kThreads, 0))
