@@ -242,8 +242,11 @@ __device__ __forceinline__ unsigned long long lookback_exclusive(unsigned long l
 
 // t = (iso - v_lo) / (v_hi - v_lo) on a cut edge (iso lies between the two
 // samples, so |iso - v_lo| <= |v_hi - v_lo|), each difference rounded once.
-// The quotient goes through the reciprocal (kExact false: within 2 ulp for
-// divisors in [2^-126, 2^126]) or is correctly rounded (kExact true).  A
+// The quotient a / b is formed as a * (1 / b) (kExact false) or correctly
+// rounded (kExact true).  The PTX ISA gives rcp.approx an error of at most one
+// unit in the last place, 2^-23 of the value, for a normal divisor with a
+// normal reciprocal; the product rounds once more (2^-24), and so did both
+// differences: t is within 5 * 2^-24 of the real quotient.  A
 // difference outside [2^-100, 2^125) -- samples near +-FLT_MAX, whose
 // difference can even overflow, or samples so close that it is tiny -- is
 // formed from the samples scaled by 2^-4 or 2^64: the scaling is exact up to
@@ -261,7 +264,7 @@ __device__ __forceinline__ float edge_fraction(float iso, float vlo, float vhi) 
         b = __fsub_rn(__fmul_rn(vhi, sc), slo);
     }
     if (kExact) return __fdiv_rn(a, b);
-    float r;                             // b is normal and its reciprocal too, so this is __fdividef's quotient
+    float r;                             // b is normal and its reciprocal too
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
     return __fmul_rn(a, r);
 }
