@@ -187,7 +187,8 @@ def measured_peaks():
         return None
 
 
-PROFILE_SOURCES = ("extract.cu", "mc.cu", "cell_masks.cuh", "codec.cuh", "common.cuh", "kernels.cuh", "launch.cuh", "tile_scan.cuh")
+PROFILE_SOURCES = ("extract.cu", "mc.cu", "mc_tables.cu", "cell_masks.cuh", "codec.cuh", "common.cuh", "kernels.cuh",
+                   "launch.cuh", "mc_tables.cuh", "tile_scan.cuh")
 
 
 def profile_sources_sha():
