@@ -136,7 +136,8 @@ typedef struct iso_mesh {
  * memory pool of its own per device, which keeps freed memory for reuse.
  * iso_set_allocator routes every later device allocation of the library
  * (volume state, meshes, scratch of batches, servers and renders) through
- * the caller: alloc(bytes, device, stream, ctx) returns memory usable in
+ * the caller: alloc(bytes, device, stream, ctx) returns memory, aligned as
+ * cudaMalloc's is (256 bytes), usable in
  * the order of `stream` (NULL for failure: ISO_ERR_OOM), free(ptr, device,
  * stream, ctx) takes it back in that stream's order (a PyTorch caching
  * allocator fits both).  Each allocation is returned to the allocator that

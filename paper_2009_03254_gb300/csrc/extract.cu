@@ -396,7 +396,7 @@ __device__ __forceinline__ void hit_mask_work(const Launch &L, uint32_t *pre) {
         pre);
     const int lane = threadIdx.x & 31;
     const uint32_t stride = (gridDim.x * blockDim.x) >> 5;
-    auto slot_of = [&](uint32_t t, uint32_t &v) {       // the slot of block lane % 4 of warp tile t
+    auto slot_of = [&](uint32_t t, uint32_t &v) {       // the slot of block lane % kMaskBlocks of warp tile t
         v = 0u;
         if (t >= total) return -1;
         v = item_vol<kOne>(pre, L.n, t);
@@ -503,8 +503,12 @@ __global__ void __launch_bounds__(kThreads, 5) lru_b_kernel(Launch L) {
 // Chunks of kDecodeThreads new blocks; each warp of a chunk stages its 32
 // blocks' words in shared memory with coalesced loads and decodes them one
 // per lane (codec.cuh), its next chunk's ids loaded and words fetched into L2
-// meanwhile (two dependent DRAM latencies a chunk before: 68 us for 384^3
-// noise with lanes storing their own blocks, 61 with both).  Chunk 0 of every volume (each volume has at least
+// meanwhile (two dependent DRAM latencies a chunk before: 68 us for the 333 k
+// new blocks of a 384^3 noise volume with lanes storing their own blocks, 61
+// with both).  Registers are bounded for 24 warps an SM, which the shared
+// memory of rates 1 and 2 allows (20 at 3 bits a value and more); at these 80
+// registers the compiler spills 24 bytes of stores and 16 of loads a thread
+// (72 and 60 over batches).  Chunk 0 of every volume (each volume has at least
 // one) also commits the volume's cache update.  With 256-thread blocks the
 // kernel then does lru_b's work (the list for the next update, which
 // nothing before then reads): its memory latency hides behind the decoding

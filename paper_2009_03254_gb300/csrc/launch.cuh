@@ -30,10 +30,13 @@ __device__ __forceinline__ void after_previous_stage() {
 }
 
 // Volumes of up to this many blocks are launch-bound: a 64^3 sphere from a
-// warm cache (4096 blocks) takes 57 us with its stages launched ahead, 64
+// warm cache (4096 blocks) takes 46 us with its stages launched ahead, 52
 // without.  In larger ones waiting CTAs hold shared memory that the running
-// stage would have as cache: 96^3 noise from an empty cache (13824 blocks)
-// 146 against 134 us, five surfaces of 512^3 noise 1725 against 1620.
+// stage would have as cache.  Whole calls as graphs, warm and cold, spheres at
+// 16 and noise at 8 bits a value: from 512 to 8000 blocks launching ahead took
+// between 7 us less and 1 more; at 9261 blocks 6 less (sphere, warm) to 7 more
+// (noise, cold), at 13824 up to 8 more, at 21952 up to 4 more; five surfaces of
+// 512^3 noise 1725 against 1620.
 constexpr uint32_t kAheadBlocks = 8192;
 
 // launch a stage whose kernel calls after_previous_stage

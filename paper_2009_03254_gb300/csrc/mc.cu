@@ -240,7 +240,8 @@ __device__ __forceinline__ uint32_t lane_cut_word(const uint32_t m[4], uint32_t 
 // instead of staging 5x5x5 samples.  Three loads in a row and these
 // instructions bound it: with E and C counted edge by edge (44 popcounts, at a
 // quarter of the rate) the 411 k candidates of a 384^3 channel took 8.25
-// million instructions and a tile of 768 7 to 14 us, now 6.35 and 6.
+// million instructions and a tile of three rounds (768 candidates) 7 to 14 us,
+// now 6.35 and 6.
 
 __device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) { return lop3<0x96>(a, b, c); }
 __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) { return lop3<0xE8>(a, b, c); }
@@ -467,10 +468,12 @@ __global__ void __launch_bounds__(kThreads) debug_cases_kernel(Launch L) {
 
 // ================================================================ emit (Section 4.5)
 //
-// What bounds it: instruction issue (57% of slots) and the shared-memory
-// pipe (69% of its wavefronts), beside the vertices' 48 bytes a triangle.
-// Measured on a 384^3 noise surface (4.3 M triangles, 24 warps an SM): 72 us,
-// 45 M warp instructions.  A triangle per lane with its vertices passed
+// What bounds it: instruction issue (58% of slots) and the latency of the
+// shared-memory gathers (51% of its wavefronts, the first of the stalls),
+// beside the vertices' 48 bytes a triangle (39% of the DRAM peak), counted on a
+// 384^3 noise surface of 2.95 M triangles: 66 us, 40.7 M warp instructions.
+// The variants below were timed on a surface of 4.3 M triangles (24 warps an
+// SM): 72 us, 45 M warp instructions.  A triangle per lane with its vertices passed
 // through shared memory, on cases found for every cell, took 85 us and
 // 65 M.  Staging rows of 8 floats by 16-byte copies (x of 5 to 7 unused)
 // left bank conflicts: 82 us.  32 warps an SM (64 registers) 79 us and a

@@ -295,8 +295,9 @@ struct Place {
 // of them adds up the longest paths of every stage: 3000 steps for a warp
 // whose longest ray takes 300.)
 // Bound by instruction issue (14 of 32 lanes step at a time) and, at the end,
-// by the latency of the longest rays.  1080p over a 384^3 noise volume: 588
-// us; nested loops that tested every cell's samples took 1080 and had 6 lanes
+// by the latency of the longest rays (68% of issue slots; the benchmark's view
+// of 384^3 noise, 534 M warp instructions, takes 810 us).  1080p over another
+// 384^3 noise volume, where the variants were timed: 588 us; nested loops that tested every cell's samples took 1080 and had 6 lanes
 // active.  Picking the stepped axis' numbers by selects instead of a branch
 // per axis took 650.
 __device__ __forceinline__ bool cast(const CastArgs &a, const Ray &r, bool live, float &thit, float hc[3], uint32_t &hb,
