@@ -428,11 +428,10 @@ __device__ __forceinline__ void store_blocks(float *base, uint32_t to, uint32_t 
                      : "=f"(d.x), "=f"(d.y), "=f"(d.z), "=f"(d.w)
                      : "r"(rows + b * ps + ((piece ^ (b & 15u)) << 4)));
         const uint32_t row = __shfl_sync(0xffffffffu, to, (int)b);
-        float *dst = base + (size_t)row * 64 + 4 * piece;
-        if (!((have >> b) & 1u)) continue;
         if (aligned) {
-            *reinterpret_cast<float4 *>(dst) = d;
-        } else {
+            if ((have >> b) & 1u) *reinterpret_cast<float4 *>(base + (size_t)row * 64 + 4 * piece) = d;
+        } else if ((have >> b) & 1u) {
+            float *dst = base + (size_t)row * 64 + 4 * piece;
             dst[0] = d.x;
             dst[1] = d.y;
             dst[2] = d.z;
