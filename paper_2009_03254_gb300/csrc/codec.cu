@@ -27,9 +27,10 @@ __device__ __forceinline__ DecodeSmem codec_smem(uint64_t *base, uint32_t rate) 
 // contiguous, so 16 bytes a lane where rows are aligned), make and code the
 // planes, copy the 32 staged blocks out as one contiguous span of the
 // bitstream, and take each block's range over its in-volume samples as the
-// kept bits decode.  Bound by instruction issue: the coding loop is a few
-// dozen steps of some 40 instructions, beside the two transforms.  499 x 333
-// x 218 samples at 6 bits a value: 273 us.  A thread per block that wrote its
+// kept bits decode.  Bound by instruction issue and latency at 16 warps an SM
+// (56% of issue slots, 62% of the ALU pipe): the coding loop is a few dozen
+// steps of some 40 instructions, beside the two transforms.  499 x 333 x 218
+// samples at 6 bits a value: 273 us.  A thread per block that wrote its
 // words to memory one by one and parsed them again for the range took 1160.
 __global__ void __launch_bounds__(kCodecThreads, 4) encode_kernel(const float *__restrict__ field, Geom g, uint64_t *bits,
                                                                float *bmin, float *bmax) {
